@@ -4,8 +4,11 @@
 // that all give bitwise the same dt, time and totals.
 #pragma once
 
+#include <type_traits>
+
 #include "aux_kernels.h"
 #include "hydro_device.cuh"
+#include "learned_arith.cuh"
 
 namespace gh {
 namespace fin {
@@ -24,7 +27,9 @@ __device__ __forceinline__ T cell_speed(const ReduceArgs<T>& A, size_t c, bool& 
     if constexpr (COH) u[v] = __ldcg(A.U + v * A.ncell + c);
     else u[v] = A.U[v * A.ncell + c];
   }
-  recover<NDIM>(u, w);
+  // the corrected 2D FP32 scheme takes its dt from here: its own roundings
+  if constexpr (NDIM == 2 && std::is_same<T, float>::value) lf::recover(u, w);
+  else recover<NDIM>(u, w);
   const T p = gm1 * w[NV - 1];
   bad |= !(w[0] > T(0)) || !(p > T(0));
   const T cs = sqrt(gamma * p / w[0]);

@@ -84,6 +84,16 @@ __device__ __forceinline__ double minmod3(double a, double b, double c) {
   return klo > 0 ? lo : (khi < -1 ? hi : 0.0);  // strictly positive / strictly negative
 }
 
+// Double word: one comparison orders b and c, and a normalised pair has the
+// sign of its high part.
+__device__ __forceinline__ dw minmod3(dw a, dw b, dw c) {
+  const bool l = b < c;
+  dw lo = l ? b : c, hi = l ? c : b;
+  if (a < lo) lo = a;
+  if (hi < a) hi = a;
+  return lo.hi > 0.0f ? lo : (hi.hi < 0.0f ? hi : dw(0.0f, 0.0f));
+}
+
 // max(0, a, b), x == 0 and x >= 0 for the wave speeds and the HLLC branch:
 // plain for float and double word, on the integer pipe for double.
 template <class T>
@@ -95,139 +105,206 @@ __device__ __forceinline__ double max0(double a, double b) {
 }
 template <class T>
 __device__ __forceinline__ bool is_zero(T x) { return x == T(0); }
+__device__ __forceinline__ bool is_zero(dw x) { return x.hi == 0.0f; }
 __device__ __forceinline__ bool is_zero(double x) { return ((unsigned long long)__double_as_longlong(x) << 1) == 0; }
 template <class T>
 __device__ __forceinline__ bool nonneg(T x) { return x >= T(0); }
+__device__ __forceinline__ bool nonneg(dw x) { return x.hi >= 0.0f; }
 __device__ __forceinline__ bool nonneg(double x) { return okey(x) >= -1; }
+
+// Correctly rounded operations that the compiler may neither fuse nor split.
+// Every kernel family (tiles, batch, one-launch, learned, multilevel) inlines
+// the functions below, and writing the roundings out keeps the same cell and
+// face bitwise the same in all of them, whatever surrounds the call.
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ dw add_rn(dw a, dw b) { return a + b; }
+__device__ __forceinline__ dw sub_rn(dw a, dw b) { return a - b; }
+__device__ __forceinline__ dw mul_rn(dw a, dw b) { return a * b; }
+__device__ __forceinline__ dw fma_rn(dw a, dw b, dw c) { return fma(a, b, c); }
+// a / 2 (exact) and c - a / 2
+__device__ __forceinline__ float half_of(float a) { return __fmul_rn(0.5f, a); }
+__device__ __forceinline__ double half_of(double a) { return __dmul_rn(0.5, a); }
+__device__ __forceinline__ dw half_of(dw a) { return dw(__fmul_rn(0.5f, a.hi), __fmul_rn(0.5f, a.lo)); }
+__device__ __forceinline__ float sub_half(float c, float a) { return __fmaf_rn(-0.5f, a, c); }
+__device__ __forceinline__ double sub_half(double c, double a) { return __fma_rn(-0.5, a, c); }
+__device__ __forceinline__ dw sub_half(dw c, dw a) { return c - half_of(a); }
+
+// Values a distance h s below and above wc (the two faces of a cell).
+template <class T>
+__device__ __forceinline__ void face_pair(T s, T h, T wc, T& lo, T& hi) {
+  lo = fma_rn(-s, h, wc);
+  hi = fma_rn(s, h, wc);
+}
+__device__ __forceinline__ void face_pair(dw s, dw h, dw wc, dw& lo, dw& hi) {
+  const dw d = s * h;
+  lo = wc - d;
+  hi = wc + d;
+}
 
 // Limited slope of cell c from its neighbours (Eq. MinMod; theta is in g).
 template <class T>
 __device__ __forceinline__ T limited_slope(T wm, T wc, T wp, const Geo<T>& g) {
-  return minmod3((wc - wm) * g.ticm, (wp - wm) * g.ipm, (wp - wc) * g.tipc);
+  return minmod3(mul_rn(sub_rn(wc, wm), g.ticm), mul_rn(sub_rn(wp, wm), g.ipm), mul_rn(sub_rn(wp, wc), g.tipc));
 }
 
 // Division, reciprocal and square root used by the flux arithmetic.  FP64
-// takes Newton reciprocals from an FP32 seed (a few ulp, far inside its 1e-10
-// parity bar); FP32 uses the hardware approximations (a few ulp, far inside
-// its 1e-5 bar).
-// FP64 reciprocal by Newton's method for 1/x: the FP32 hardware approximation
-// as the seed (relative error ~2^-22), then two steps r <- r + r (1 - x r),
-// each of which squares the relative error (~2^-44, then the FP64 rounding
-// level): four FP64 FMAs in place of an IEEE division on GB300's slow FP64
-// pipe, within a few ulp.  Arguments whose exponent lies outside the normal
-// FP32 range (and 0, infinities, NaN) take the IEEE division; the test is on
-// the exponent bits, on the integer pipe.
-__device__ __forceinline__ double frcp(double x) {
+// takes Newton-type reciprocals from an FP32 seed (a few ulp, far inside its
+// 1e-10 parity bar); FP32 uses the hardware approximations (a few ulp, far
+// inside its 1e-5 bar).
+//
+// FP64 seeds: conversions between the formats of values in the normal FP32
+// range, on the integer pipe (rebias the exponent, move the mantissa; the
+// truncation to FP32 costs a relative 2^-23 at most, which the correction
+// steps below remove), because GB300 runs an FP64 conversion at the rate of
+// its slow FP64 pipe.
+__device__ __forceinline__ float seed_float(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b;
+  const unsigned mag = __funnelshift_l(lo, (hi & 0x7fffffffu) - (896u << 20), 3);
+  return __uint_as_float((hi & 0x80000000u) | mag);
+}
+__device__ __forceinline__ double seed_double(float f) {
+  const unsigned u = __float_as_uint(f);
+  const unsigned hi = (u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20));
+  return __longlong_as_double((long long)(((unsigned long long)hi << 32) | (unsigned long long)(u << 29)));
+}
+// Biased exponent in [900, 1146] (|x| ~ 1e-37 .. 1e37): the range in which the
+// seeds and their reciprocals are normal FP32 numbers.
+__device__ __forceinline__ bool seed_range(double x) {
   const unsigned ex = (unsigned)((unsigned long long)__double_as_longlong(x) >> 52) & 0x7ffu;
-  if (ex - 900u > 246u) return 1.0 / x;  // biased exponent outside [900, 1146] (|x| ~ 1e-37 .. 1e37)
-  double r = (double)__fdividef(1.0f, (float)x);
-  r = fma(r, fma(-x, r, 1.0), r);
-  r = fma(r, fma(-x, r, 1.0), r);
+  return ex - 900u <= 246u;
+}
+// Hardware FP32 reciprocal and reciprocal square root (relative error about
+// 2^-23); arguments above 2^126 give 0.
+__device__ __forceinline__ float frcp(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
+}
+__device__ __forceinline__ float frsqrt(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+// FP64 reciprocal: seed r with relative error ~2^-22, then 1/x = r (1 + e +
+// e^2 + ...) with the exact residual e = 1 - x r: the cubic step r + r (e +
+// e^2) leaves e^3 ~ 2^-66, below the FP64 rounding level, in three FP64 FMAs
+// in place of an IEEE division on GB300's slow FP64 pipe.  Arguments outside
+// the normal FP32 range (and 0, infinities, NaN) take the IEEE division.
+__device__ __forceinline__ double frcp(double x) {
+  if (!seed_range(x)) return 1.0 / x;
+  const double r = seed_double(frcp(seed_float(x)));
+  const double e = fma_rn(-x, r, 1.0);
+  return fma_rn(r, fma_rn(e, e, e), r);
 }
 // a / b from the reciprocal and one residual correction q + r (a - b q).
 __device__ __forceinline__ double fdiv(double a, double b) {
   const double r = frcp(b);
-  const double q = a * r;
-  return fma(r, fma(-b, q, a), q);
+  const double q = mul_rn(a, r);
+  return fma_rn(r, fma_rn(-b, q, a), q);
 }
-__device__ __forceinline__ float fdiv(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ float frcp(float x) { return __fdividef(1.0f, x); }
-// Correctly rounded sum that the compiler may not fuse with a product feeding
-// it: keeps the stage combine bitwise the same in every kernel that inlines it,
-// whatever the surrounding code lets the compiler contract.
-__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
-__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
-// sqrt of a positive argument
-__device__ __forceinline__ double fsqrt(double x) { return sqrt(x); }
-__device__ __forceinline__ float fsqrt(float x) { return x * rsqrtf(x); }
+__device__ __forceinline__ float fdiv(float a, float b) { return mul_rn(a, frcp(b)); }
 // double-word: the operations of dword.cuh
 __device__ __forceinline__ dw fdiv(dw a, dw b) { return a / b; }
 __device__ __forceinline__ dw frcp(dw x) { return dw(1.0f, 0.0f) / x; }
-__device__ __forceinline__ dw fsqrt(dw x) { return sqrt(x); }
-__device__ __forceinline__ dw add_rn(dw a, dw b) { return a + b; }
 
-// Sound speed c = sqrt(gamma p / n) (Sec. 3.5).  FP64: gamma p rsqrt(gamma p n),
-// one reciprocal square root (CUDA's rsqrt, 1 ulp) in place of an IEEE division
-// and an IEEE square root on the slow FP64 pipe; 0 where gamma p is not
-// positive.  FP32: the same form with the hardware approximation (one
-// multi-function-unit operation instead of two).  Double word: the quotient
-// and square root of dword.cuh.
-template <class T>
-__device__ __forceinline__ T sound_speed(T gamma, T p, T n) { return fsqrt(gamma * fdiv(p, n)); }
+// Sound speed c = sqrt(gamma p / n) (Sec. 3.5) as gp rsqrt(gp n), gp = gamma p.
+// FP64: seed r = rsqrt(x) with relative error ~2^-22, residual e = 1 - x r^2,
+// then x^(-1/2) = r (1 - e)^(-1/2) = r (1 + e/2 + 3 e^2/8 + ...), which leaves
+// 5 e^3/16 ~ 2^-65: seven FP64 operations; CUDA's rsqrt outside the seed range,
+// and 0 where gamma p is not positive.  FP32: the hardware approximation.
+// Double word: the quotient and square root of dword.cuh.
+__device__ __forceinline__ dw sound_speed(dw gamma, dw p, dw n) { return sqrt(gamma * (p / n)); }
 __device__ __forceinline__ float sound_speed(float gamma, float p, float n) {
-  const float gp = gamma * p;
-  return gp * rsqrtf(gp * n);
+  const float gp = mul_rn(gamma, p);
+  return mul_rn(gp, frsqrt(mul_rn(gp, n)));
 }
 __device__ __forceinline__ double sound_speed(double gamma, double p, double n) {
-  const double gp = gamma * p;
-  return okey(gp) > 0 ? gp * rsqrt(gp * n) : 0.0;
+  const double gp = mul_rn(gamma, p), x = mul_rn(gp, n);
+  if (!(okey(gp) > 0)) return 0.0;
+  if (!seed_range(x)) return mul_rn(gp, rsqrt(x));
+  const double r = seed_double(frsqrt(seed_float(x)));
+  const double e = fma_rn(-mul_rn(x, r), r, 1.0);
+  const double c = mul_rn(gp, r);
+  return fma_rn(mul_rn(c, e), fma_rn(0.375, e, 0.5), c);
 }
 
 // ---------------------------------------------------------------------------
-// Conserved -> primitive recovery.
+// Conserved -> primitive recovery: v = S / D, e = G - S.v / 2.
 //
-// FP64 path: plain double arithmetic.
-// Mixed path (FP32 storage): e = G - |S|^2 / (2 D) cancels when the kinetic
-// energy density is a large part of G.  Where the kinetic part is at most
-// half of G the FP32 difference loses at most one bit and is used as is;
-// elsewhere the difference is formed in FP64 as e D = G D - |S|^2 / 2, where
-// every product of two FP32 values is exact, so the cancellation loses
-// nothing, and the well-conditioned division by D runs in FP32.
+// FP64 and double word: as written.
+// Mixed path (FP32 storage): the difference cancels when the kinetic energy is
+// a large part of G.  Where it is at most half of G the FP32 difference loses
+// at most one bit and is used as is.  Elsewhere v is extended by its residual,
+// v = v_r + v_l with v_l = (S - v_r D) / D, every product S v_r is split into
+// its rounded value and rounding error, and the sums carry their rounding
+// errors (Knuth's TwoSum), so that S.v / 2 is known to about 2^-46; the leading
+// difference G - s/2 is exact there (the two lie within a factor 2), and its
+// correction is added last.  The result is as exact as the FP32 state allows
+// (a rounding of G alone moves e by 2^-25 G), without the FP64 pipe, which an
+// earlier FP64 branch here kept 44% busy in the FP32 batch kernel (Riemann
+// problems carry much kinetic energy): 256 problems, 20 steps with their
+// copies in and out, 20.97 -> 17.85 ms.
 // ---------------------------------------------------------------------------
-template <int NDIM>
-__device__ __forceinline__ void recover(const double (&u)[NDIM + 2], double (&w)[NDIM + 2]) {
+template <int NDIM, class T>
+__device__ __forceinline__ void recover(const T (&u)[NDIM + 2], T (&w)[NDIM + 2]) {
   constexpr int NV = NDIM + 2;
-  const double rn = frcp(u[0]);
-  double v2 = 0.0;
+  const T rn = frcp(u[0]);
   w[0] = u[0];
 #pragma unroll
-  for (int q = 0; q < NDIM; ++q) {
-    w[1 + q] = u[1 + q] * rn;
-    v2 += w[1 + q] * w[1 + q];
-  }
-  w[NV - 1] = u[NV - 1] - 0.5 * u[0] * v2;
+  for (int q = 0; q < NDIM; ++q) w[1 + q] = mul_rn(u[1 + q], rn);
+  T sv = mul_rn(u[1], w[1]);
+#pragma unroll
+  for (int q = 1; q < NDIM; ++q) sv = fma_rn(u[1 + q], w[1 + q], sv);
+  w[NV - 1] = sub_half(u[NV - 1], sv);
 }
 
-// e D = G D - |S|^2 / 2 in FP64 (products of FP32 values are exact in FP64).
-// Kept out of line so that only lanes that need it execute FP64 instructions.
-static __device__ __noinline__ float energy_density_times_n_fp64(float n, float s1, float s2, float s3, float G) {
-  const double s2d = fma((double)s1, (double)s1, fma((double)s2, (double)s2, (double)s3 * (double)s3));
-  return (float)fma(-0.5, s2d, (double)G * (double)n);
-}
-
-// Double-word path: the FP64 formulas in double-word arithmetic.
+// e of a cell whose kinetic energy exceeds half of G: the compensated form
+// (v_r: the rounded velocities, rn: the reciprocal of D).
 template <int NDIM>
-__device__ __forceinline__ void recover(const dw (&u)[NDIM + 2], dw (&w)[NDIM + 2]) {
-  constexpr int NV = NDIM + 2;
-  const dw rn = frcp(u[0]);
-  dw v2 = dw(0.0f, 0.0f);
-  w[0] = u[0];
+__device__ __forceinline__ float energy_compensated(const float (&u)[NDIM + 2], const float (&vr)[NDIM], float rn) {
+  float s = 0.0f, t = 0.0f;  // S.v = s + t
 #pragma unroll
   for (int q = 0; q < NDIM; ++q) {
-    w[1 + q] = u[1 + q] * rn;
-    v2 = fma(w[1 + q], w[1 + q], v2);
+    const float S = u[1 + q];
+    const float vl = mul_rn(fma_rn(-vr[q], u[0], S), rn);
+    const float p = mul_rn(S, vr[q]);
+    const float pe = fma_rn(S, vl, fma_rn(S, vr[q], -p));
+    if (q == 0) {
+      s = p;
+      t = pe;
+    } else {
+      float z, ze;
+      two_sum(s, p, z, ze);
+      s = z;
+      t = add_rn(t, add_rn(ze, pe));
+    }
   }
-  w[NV - 1] = u[NV - 1] - dw(0.5f, 0.0f) * u[0] * v2;
+  return sub_half(sub_half(u[NDIM + 1], s), t);
 }
 
 template <int NDIM>
 __device__ __forceinline__ void recover(const float (&u)[NDIM + 2], float (&w)[NDIM + 2]) {
   constexpr int NV = NDIM + 2;
   const float rn = frcp(u[0]);
-  float s2 = 0.0f;
+  float vr[NDIM];
 #pragma unroll
-  for (int q = 0; q < NDIM; ++q) s2 = fmaf(u[1 + q], u[1 + q], s2);
-  const float ke = 0.5f * s2 * rn;
-  float e = u[NV - 1] - ke;
-  if (__builtin_expect(!(ke <= 0.5f * u[NV - 1]), 0)) {
-    const float eD = energy_density_times_n_fp64(u[0], u[1], NDIM > 1 ? u[2] : 0.0f, NDIM > 2 ? u[3] : 0.0f,
-                                                 u[NV - 1]);
-    e = eD * rn;
-  }
+  for (int q = 0; q < NDIM; ++q) vr[q] = mul_rn(u[1 + q], rn);
+  float sv = mul_rn(u[1], vr[0]);
+#pragma unroll
+  for (int q = 1; q < NDIM; ++q) sv = fma_rn(u[1 + q], vr[q], sv);
+  float e = sub_half(u[NV - 1], sv);
+  if (__builtin_expect(!(e >= half_of(u[NV - 1])), 0)) e = energy_compensated<NDIM>(u, vr, rn);
   w[0] = u[0];
 #pragma unroll
-  for (int q = 0; q < NDIM; ++q) w[1 + q] = u[1 + q] * rn;
+  for (int q = 0; q < NDIM; ++q) w[1 + q] = vr[q];
   w[NV - 1] = e;
 }
 
@@ -240,18 +317,24 @@ __device__ __forceinline__ void recover(const float (&u)[NDIM + 2], float (&w)[N
 //   HLLC         Eq. MiddleWaveSpeed for alpha_m, then one middle state on the
 //                side selected by the sign of alpha_m (Eq. FluxHLLC), written
 //                with the signed outer wave speed S_K (S_L = -alpha_-,
-//                S_R = alpha_+):
-//                  D*  = D_K (S_K - v_K) / (S_K - alpha_m)
-//                  p*  = p_K + D_K (S_K - v_K)(alpha_m - v_K)
-//                  G*  = [(S_K - v_K) G_K - p_K v_K + p* alpha_m] / (S_K - alpha_m)
-//                  S*  = D* (alpha_m e_Q + transverse v_K)
-//                  F*  = F_K + S_K (U* - U_K)
+//                S_R = alpha_+), d_K = S_K - v_K and a_K = D_K d_K:
+//                  D* = a_K / (S_K - alpha_m)
+//                  p* = p_K + a_K (alpha_m - v_K)
+//                  G* = (d_K G_K - p_K v_K + p* alpha_m) / (S_K - alpha_m)
 //                which are the outer jump conditions of Sec. 3.2 solved for the
-//                middle state (this form satisfies p*_L = p*_R).
-//                alpha_- = 0 gives F_L, alpha_+ = 0 gives F_R (upwind): those
-//                cases select that side, where S_K = 0, so F* = F_K exactly
-//                once the factor 1 / (S_K - alpha_m) of the (unused) middle
-//                state is replaced by 0 to keep it finite.
+//                middle state (this form satisfies p*_L = p*_R).  The middle
+//                state moves with alpha_m, so its flux is
+//                  F* = alpha_m U* + p* (0, e_Q, alpha_m):
+//                D* alpha_m, that times (alpha_m, transverse v_K) plus p* in
+//                the normal momentum, and (G* + p*) alpha_m; neither F_K nor U_K
+//                beyond G_K is formed, about 20 operations a face fewer than
+//                F_K + S_K (U* - U_K).  Measured with the shorter reciprocal
+//                and sound speed above, ms per RK2 step, HLLC: FP64 128^3
+//                4.90 -> 4.22 (bound by the FP64 pipe), double word 128^3
+//                1.36 -> 1.14, FP32 256^3 1.436 -> 1.383 (bound by issue).
+//                alpha_- = 0 gives F_L, alpha_+ = 0 gives F_R (upwind): there
+//                S_K = 0, and alpha_m is replaced by v_K, for which U* = U_K
+//                and the formulas above are F_K.
 // ---------------------------------------------------------------------------
 // Conserved state U(W) and physical flux F^Q(U) of one side of a face
 // (Sec. 3.5): p is its pressure, w[1 + Q] its normal velocity.
@@ -259,17 +342,16 @@ template <class T, int NDIM, int Q>
 __device__ __forceinline__ void side_state(const T (&w)[NDIM + 2], T p, T (&u)[NDIM + 2], T (&f)[NDIM + 2]) {
   constexpr int NV = NDIM + 2;
   const T n = w[0], vq = w[1 + Q];
-  T v2 = T(0);
+  T v2 = mul_rn(w[1], w[1]);
 #pragma unroll
-  for (int q = 0; q < NDIM; ++q) v2 += w[1 + q] * w[1 + q];
+  for (int q = 1; q < NDIM; ++q) v2 = fma_rn(w[1 + q], w[1 + q], v2);
   u[0] = n;
 #pragma unroll
-  for (int q = 0; q < NDIM; ++q) u[1 + q] = n * w[1 + q];
-  u[NV - 1] = w[NV - 1] + T(0.5) * n * v2;
+  for (int q = 0; q < NDIM; ++q) u[1 + q] = mul_rn(n, w[1 + q]);
+  u[NV - 1] = fma_rn(half_of(n), v2, w[NV - 1]);
 #pragma unroll
-  for (int v = 0; v < NV - 1; ++v) f[v] = u[v] * vq;
-  f[1 + Q] += p;
-  f[NV - 1] = (u[NV - 1] + p) * vq;
+  for (int v = 0; v < NV - 1; ++v) f[v] = v == 1 + Q ? fma_rn(u[v], vq, p) : mul_rn(u[v], vq);
+  f[NV - 1] = mul_rn(add_rn(u[NV - 1], p), vq);
 }
 
 template <class T, int NDIM, int Q, int SOLVER>
@@ -277,48 +359,49 @@ __device__ __forceinline__ void face_flux(const T (&wl)[NDIM + 2], const T (&wr)
                                           T gamma, T gm1, T (&F)[NDIM + 2]) {
   constexpr int NV = NDIM + 2;
   const T nl = wl[0], nr = wr[0];
-  const T pl = gm1 * wl[NV - 1], pr = gm1 * wr[NV - 1];
+  const T pl = mul_rn(gm1, wl[NV - 1]), pr = mul_rn(gm1, wr[NV - 1]);
   const T vl = wl[1 + Q], vr = wr[1 + Q];
   const T cl = sound_speed(gamma, pl, nl);
   const T cr = sound_speed(gamma, pr, nr);
-  const T ap = max0(vl + cl, vr + cr);
-  const T am = max0(cl - vl, cr - vr);
+  const T ap = max0(add_rn(vl, cl), add_rn(vr, cr));
+  const T am = max0(sub_rn(cl, vl), sub_rn(cr, vr));
 
   if constexpr (SOLVER == SOLVER_HLL) {
     T ul[NV], ur[NV], fl[NV], fr[NV];
     side_state<T, NDIM, Q>(wl, pl, ul, fl);
     side_state<T, NDIM, Q>(wr, pr, ur, fr);
-    const T inv = frcp(ap + am);
-    const T apam = ap * am;
+    const T inv = frcp(add_rn(ap, am));
+    const T apam = mul_rn(ap, am);
 #pragma unroll
-    for (int v = 0; v < NV; ++v) F[v] = (ap * fl[v] + am * fr[v] - apam * (ur[v] - ul[v])) * inv;
+    for (int v = 0; v < NV; ++v)
+      F[v] = mul_rn(fma_rn(-apam, sub_rn(ur[v], ul[v]), fma_rn(am, fr[v], mul_rn(ap, fl[v]))), inv);
   } else {
-    // HLLC.  Only the selected side K enters F* = F_K + S_K (U* - U_K), so
-    // its primitives are selected first and U_K, F_K formed once.
-    const T sl = am + vl;  // = -(S_L - v_L) > 0
-    const T sr = ap - vr;  // =   S_R - v_R  > 0
-    const T ml = nl * vl, mr = nr * vr;  // normal momenta
-    const T alpha_m = fdiv(mr * sr + ml * sl - (pr - pl), nr * sr + nl * sl);
-    const bool left = is_zero(am) || (!is_zero(ap) && nonneg(alpha_m));
+    const T sl = add_rn(am, vl);  // = -(S_L - v_L) > 0
+    const T sr = sub_rn(ap, vr);  // =   S_R - v_R  > 0
+    const T al = mul_rn(nl, sl), ar = mul_rn(nr, sr);
+    const T alpha = fdiv(fma_rn(ar, vr, fma_rn(al, vl, sub_rn(pl, pr))), add_rn(ar, al));
+    const bool left = is_zero(am) || (!is_zero(ap) && nonneg(alpha));
     const T SK = left ? -am : ap;
+    const T dK = left ? -sl : sr;
+    const T aK = left ? -al : ar;
     const T pK = left ? pl : pr;
     T wK[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) wK[v] = left ? wl[v] : wr[v];
-    const T nK = wK[0], vK = wK[1 + Q];
-    T uK[NV], fK[NV];
-    side_state<T, NDIM, Q>(wK, pK, uK, fK);
-    const T dK = SK - vK;  // S_K - v_K
-    const T rden = is_zero(SK) ? T(0) : frcp(SK - alpha_m);
-    const T Ds = nK * dK * rden;
-    const T ps = pK + nK * dK * (alpha_m - vK);
-    T us[NV];
-    us[0] = Ds;
+    const T vK = wK[1 + Q];
+    const T a = is_zero(SK) ? vK : alpha;
+    T v2 = mul_rn(wK[1], wK[1]);
 #pragma unroll
-    for (int q = 0; q < NDIM; ++q) us[1 + q] = Ds * (q == Q ? alpha_m : wK[1 + q]);
-    us[NV - 1] = (dK * uK[NV - 1] - pK * vK + ps * alpha_m) * rden;
+    for (int q = 1; q < NDIM; ++q) v2 = fma_rn(wK[1 + q], wK[1 + q], v2);
+    const T GK = fma_rn(half_of(wK[0]), v2, wK[NV - 1]);
+    const T r = frcp(sub_rn(SK, a));
+    const T ps = fma_rn(aK, sub_rn(a, vK), pK);
+    const T Gs = mul_rn(fma_rn(dK, GK, fma_rn(ps, a, -mul_rn(pK, vK))), r);
+    const T m = mul_rn(mul_rn(aK, r), a);  // D* alpha_m
+    F[0] = m;
 #pragma unroll
-    for (int v = 0; v < NV; ++v) F[v] = fK[v] + SK * (us[v] - uK[v]);
+    for (int q = 0; q < NDIM; ++q) F[1 + q] = q == Q ? fma_rn(m, a, ps) : mul_rn(m, wK[1 + q]);
+    F[NV - 1] = mul_rn(add_rn(Gs, ps), a);
   }
 }
 
@@ -341,13 +424,12 @@ struct ColumnSum<float> {
   float hi = 0.0f, lo = 0.0f;
   // add u * (dz_hi + dz_lo)
   __device__ __forceinline__ void add_product(float u, float dz_hi, float dz_lo) {
-    const float p = u * dz_hi;
-    const float pe = fmaf(u, dz_hi, -p) + u * dz_lo;
-    const float t = hi + p;
-    const float bp = t - hi;
-    const float err = (hi - (t - bp)) + (p - bp);
+    const float p = mul_rn(u, dz_hi);
+    const float pe = fma_rn(u, dz_lo, fma_rn(u, dz_hi, -p));
+    float t, err;
+    two_sum(hi, p, t, err);
     hi = t;
-    lo += err + pe;
+    lo = add_rn(lo, add_rn(err, pe));
   }
   __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };

@@ -6,7 +6,7 @@
 // HLLC flux; the paper has no counterpart.)
 #pragma once
 
-#include "hydro_device.cuh"
+#include "learned_arith.cuh"
 #include "mlp.cuh"
 
 namespace gh {
@@ -62,7 +62,7 @@ __device__ __forceinline__ void cell_prim(const Mesh2& M, const float* __restric
   }
   if (fx) u[1] = -u[1];
   if (fy) u[2] = -u[2];
-  recover<2>(u, w);
+  lf::recover(u, w);
 }
 
 __device__ __forceinline__ Geo<float> geo_at(const Mesh2& M, int q, int c) {
@@ -80,10 +80,10 @@ __device__ __forceinline__ void plain_face_flux(const Mesh2& M, const float (&w)
   float wl[4], wr[4];
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
-    wl[v] = fmaf(limited_slope(w[0][v], w[1][v], w[2][v], gl), gl.h, w[1][v]);
-    wr[v] = fmaf(-limited_slope(w[1][v], w[2][v], w[3][v], gr), gr.h, w[2][v]);
+    wl[v] = fmaf(lf::limited_slope(w[0][v], w[1][v], w[2][v], gl), gl.h, w[1][v]);
+    wr[v] = fmaf(-lf::limited_slope(w[1][v], w[2][v], w[3][v], gr), gr.h, w[2][v]);
   }
-  face_flux<float, 2, Q, SOLVER>(wl, wr, M.gamma, M.gm1, F);
+  lf::face_flux<Q, SOLVER>(wl, wr, M.gamma, M.gm1, F);
 }
 
 // Features (24) and flux scales (4) of a face from its six-cell primitive

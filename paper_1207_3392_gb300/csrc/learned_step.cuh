@@ -274,7 +274,7 @@ __device__ __forceinline__ void lf_update_cell(const UpdateArgs& A, long long c,
       A.out[v * ncell + c] = u[v];
     }
   }
-  recover<2>(u, w);
+  lf::recover(u, w);
   const bool ok = w[0] > 0.f && M.gm1 * w[3] > 0.f && fabsf(w[1]) < INFINITY && fabsf(w[2]) < INFINITY;
   if (A.fixup == 0) {
     A.flag_out[c] = ok ? 0 : 1;

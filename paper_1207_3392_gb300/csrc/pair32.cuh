@@ -82,24 +82,27 @@ __device__ __forceinline__ f2 sound_speed2(f2 gamma, f2 p, f2 n) {
   return mul2(gp, mk2(rsqrtf(q.x), rsqrtf(q.y)));
 }
 
-// Conserved -> primitive (3D): n = D, v = S / D, e = G - |S|^2 / (2D); a lane
-// whose kinetic energy exceeds half of G recomputes e in FP64, as the scalar
+// Conserved -> primitive (3D): n = D, v = S / D, e = G - S.v / 2; a lane whose
+// kinetic energy exceeds half of G takes the compensated form, as the scalar
 // FP32 path does.
+__device__ __forceinline__ float energy_lane(float n, float s1, float s2, float s3, float G, float v1, float v2, float v3,
+                                             float rn) {
+  const float u[5] = {n, s1, s2, s3, G}, v[3] = {v1, v2, v3};
+  return energy_compensated<3>(u, v, rn);
+}
 __device__ __forceinline__ void recover2(const f2 (&u)[5], f2 (&w)[5]) {
   const f2 rn = frcp2(u[0]);
-  f2 s2 = mul2(u[1], u[1]);
-  s2 = fma2(u[2], u[2], s2);
-  s2 = fma2(u[3], u[3], s2);
-  const f2 ke = mul2(mul2(bc2(0.5f), s2), rn);
-  f2 e = sub2(u[4], ke);
-  if (__builtin_expect(!(ke.x <= 0.5f * u[4].x), 0))
-    e.x = energy_density_times_n_fp64(u[0].x, u[1].x, u[2].x, u[3].x, u[4].x) * rn.x;
-  if (__builtin_expect(!(ke.y <= 0.5f * u[4].y), 0))
-    e.y = energy_density_times_n_fp64(u[0].y, u[1].y, u[2].y, u[3].y, u[4].y) * rn.y;
+  const f2 v1 = mul2(u[1], rn), v2 = mul2(u[2], rn), v3 = mul2(u[3], rn);
+  const f2 sv = fma2(u[3], v3, fma2(u[2], v2, mul2(u[1], v1)));
+  f2 e = fma2(bc2(-0.5f), sv, u[4]);
+  if (__builtin_expect(!(e.x >= 0.5f * u[4].x), 0))
+    e.x = energy_lane(u[0].x, u[1].x, u[2].x, u[3].x, u[4].x, v1.x, v2.x, v3.x, rn.x);
+  if (__builtin_expect(!(e.y >= 0.5f * u[4].y), 0))
+    e.y = energy_lane(u[0].y, u[1].y, u[2].y, u[3].y, u[4].y, v1.y, v2.y, v3.y, rn.y);
   w[0] = u[0];
-  w[1] = mul2(u[1], rn);
-  w[2] = mul2(u[2], rn);
-  w[3] = mul2(u[3], rn);
+  w[1] = v1;
+  w[2] = v2;
+  w[3] = v3;
   w[4] = e;
 }
 

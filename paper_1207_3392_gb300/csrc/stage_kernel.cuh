@@ -280,7 +280,7 @@ struct StageKernel {
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       T x = ld(A.un + v * vs + c);
-      if (STAGE == 2) x = fma(dt, ld(A.k1 + v * vs + c), x);
+      if (STAGE == 2) x = fma_rn(dt, ld(A.k1 + v * vs + c), x);
       u[v] = x;
     }
     if (r.fa) u[1] = -u[1];
@@ -343,8 +343,8 @@ struct StageKernel {
       get_w(S, b, srow, sl + 2, w3);
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        wl[v] = fma(limited_slope(w0[v], w1[v], w2[v], gl), gl.h, w1[v]);
-        wr[v] = fma(-limited_slope(w1[v], w2[v], w3[v], gr), gr.h, w2[v]);
+        wl[v] = fma_rn(limited_slope(w0[v], w1[v], w2[v], gl), gl.h, w1[v]);
+        wr[v] = fma_rn(-limited_slope(w1[v], w2[v], w3[v], gr), gr.h, w2[v]);
       }
     }
     flux<0>(A, wl, wr, SW ? (unsigned)(S.fl[b][SW ? srow : 0][SW ? sl : 0] | S.fl[b][SW ? srow : 0][SW ? sl + 1 : 0]) : 0u,
@@ -367,8 +367,8 @@ struct StageKernel {
       get_w(S, b, sl + 2, scol, w3);
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        wl[v] = fma(limited_slope(w0[v], w1[v], w2[v], gl), gl.h, w1[v]);
-        wr[v] = fma(-limited_slope(w1[v], w2[v], w3[v], gr), gr.h, w2[v]);
+        wl[v] = fma_rn(limited_slope(w0[v], w1[v], w2[v], gl), gl.h, w1[v]);
+        wr[v] = fma_rn(-limited_slope(w1[v], w2[v], w3[v], gr), gr.h, w2[v]);
       }
     }
     flux<1>(A, wl, wr, SW ? (unsigned)(S.fl[b][SW ? sl : 0][SW ? scol : 0] | S.fl[b][SW ? sl + 1 : 0][SW ? scol : 0]) : 0u,
@@ -384,8 +384,8 @@ struct StageKernel {
     T wl[NV], wr[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-      wl[v] = fma(sa[v], ha, wa[v]);
-      wr[v] = fma(-sb[v], hb, wb[v]);
+      wl[v] = fma_rn(sa[v], ha, wa[v]);
+      wr[v] = fma_rn(-sb[v], hb, wb[v]);
     }
     flux<AM>(A, wl, wr, bits, f);
   }
@@ -410,8 +410,7 @@ struct StageKernel {
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         const T sv = limited_slope(wm[v], wc[v], wp[v], g);
-        lo[v] = fma(-sv, g.h, wc[v]);
-        hi[v] = fma(sv, g.h, wc[v]);
+        face_pair(sv, g.h, wc[v], lo[v], hi[v]);
       }
       put_xs(S, 0, ty, tx + 1, lo);
       put_xs(S, 1, ty, tx + 1, hi);
@@ -424,8 +423,7 @@ struct StageKernel {
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         const T sv = limited_slope(wm[v], wc[v], wp[v], g);
-        lo[v] = fma(-sv, g.h, wc[v]);
-        hi[v] = fma(sv, g.h, wc[v]);
+        face_pair(sv, g.h, wc[v], lo[v], hi[v]);
       }
       put_ys(S, 0, ty + 1, tx, lo);
       put_ys(S, 1, ty + 1, tx, hi);
@@ -446,7 +444,7 @@ struct StageKernel {
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         const T sv = limited_slope(wm[v], w1[v], wp[v], g);
-        o[v] = up ? fma(-sv, g.h, w1[v]) : fma(sv, g.h, w1[v]);
+        o[v] = up ? fma_rn(-sv, g.h, w1[v]) : fma_rn(sv, g.h, w1[v]);
       }
       if (up) put_xs(S, 0, r, TX + 1, o);
       else put_xs(S, 1, r, 0, o);
@@ -464,7 +462,7 @@ struct StageKernel {
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         const T sv = limited_slope(wm[v], w1[v], wp[v], g);
-        o[v] = up ? fma(-sv, g.h, w1[v]) : fma(sv, g.h, w1[v]);
+        o[v] = up ? fma_rn(-sv, g.h, w1[v]) : fma_rn(sv, g.h, w1[v]);
       }
       if (up) put_ys(S, 0, TY + 1, c, o);
       else put_ys(S, 1, 0, c, o);
@@ -699,9 +697,9 @@ struct StageKernel {
         }
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
-          T d = (fxr[v] - fxl[v]) * iwx;
-          if constexpr (HAS_Y) d += (fyt[v] - fyb[v]) * iwy;
-          if constexpr (MARCH) d += (fhi[v] - flo[v]) * iwm;
+          T d = mul_rn(sub_rn(fxr[v], fxl[v]), iwx);
+          if constexpr (HAS_Y) d = fma_rn(sub_rn(fyt[v], fyb[v]), iwy, d);
+          if constexpr (MARCH) d = fma_rn(sub_rn(fhi[v], flo[v]), iwm, d);
           L[v] = -d;
         }
         if (A.has_source) {
@@ -710,10 +708,10 @@ struct StageKernel {
           T power = T(0);
 #pragma unroll
           for (int q = 0; q < NDIM; ++q) {
-            L[1 + q] -= wown[0] * A.grad_phi[q];
-            power = fma(wown[0] * wown[1 + q], A.grad_phi[q], power);
+            L[1 + q] = fma_rn(-wown[0], A.grad_phi[q], L[1 + q]);
+            power = fma_rn(mul_rn(wown[0], wown[1 + q]), A.grad_phi[q], power);
           }
-          L[NV - 1] -= power;
+          L[NV - 1] = sub_rn(L[NV - 1], power);
         }
         const size_t c = cell(A, ca, cb, m);
         bad |= nonphysical(wown, A.gm1);
@@ -736,7 +734,7 @@ struct StageKernel {
 #pragma unroll
           for (int v = 0; v < NV; ++v) {
             const T u0 = ld(A.un + v * vs + c), k = ld(A.k1 + v * vs + c);
-            A.out[v * vs + c] = fma(hdt, add_rn(k, L[v]), u0);
+            A.out[v * vs + c] = fma_rn(hdt, add_rn(k, L[v]), u0);
           }
         }
       }

@@ -396,19 +396,19 @@ struct StageTma {
         T L[NV];
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
-          T d = (S.fx[v][ty][tx + 1] - S.fx[v][ty][tx]) * iwx;
-          d += (S.fy[v][ty + 1][tx] - S.fy[v][ty][tx]) * iwy;
-          d += (fhi[v] - flo[v]) * iwm;
+          T d = mul_rn(sub_rn(S.fx[v][ty][tx + 1], S.fx[v][ty][tx]), iwx);
+          d = fma_rn(sub_rn(S.fy[v][ty + 1][tx], S.fy[v][ty][tx]), iwy, d);
+          d = fma_rn(sub_rn(fhi[v], flo[v]), iwm, d);
           L[v] = -d;
         }
         if (A.has_source) {
           T power = T(0);
 #pragma unroll
           for (int q = 0; q < 3; ++q) {
-            L[1 + q] -= wk[0] * A.grad_phi[q];
-            power = fma(wk[0] * wk[1 + q], A.grad_phi[q], power);
+            L[1 + q] = fma_rn(-wk[0], A.grad_phi[q], L[1 + q]);
+            power = fma_rn(mul_rn(wk[0], wk[1 + q]), A.grad_phi[q], power);
           }
-          L[NV - 1] -= power;
+          L[NV - 1] = sub_rn(L[NV - 1], power);
         }
         const size_t c = ((size_t)m * ny + cb) * nx + ca;
         bad |= Base::nonphysical(wk, A.gm1);
@@ -430,7 +430,7 @@ struct StageTma {
 #pragma unroll
           for (int v = 0; v < NV; ++v) {
             const T u0 = __ldg(A.un + v * vs + c), k = __ldg(A.k1 + v * vs + c);
-            A.out[v * vs + c] = fma(hdt, add_rn(k, L[v]), u0);
+            A.out[v * vs + c] = fma_rn(hdt, add_rn(k, L[v]), u0);
           }
         }
       }
