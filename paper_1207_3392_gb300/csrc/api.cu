@@ -172,6 +172,8 @@ int configure(genasis_hydro* h, int tile, int kchunk_req) {
   if ((v1.tma || v2.tma) && !tma_usable(h))
     return fail(GENASIS_EINVAL, "tile %d stages the state with TMA, which needs a 3D FP32 mesh with n[0] a multiple of 4",
                 tile);
+  for (StageVariant* v : {&v1, &v2})
+    if (v->fn_wide && h->ncell > ((size_t)1 << 30)) v->fn = v->fn_wide;
   const int gx = (h->n[0] + v1.tx - 1) / v1.tx;
   const int gy = h->ndim == 3 ? (h->n[1] + v1.ty - 1) / v1.ty : 1;
   const int gx2 = (h->n[0] + v2.tx - 1) / v2.tx;
@@ -181,6 +183,15 @@ int configure(genasis_hydro* h, int tile, int kchunk_req) {
   if (h->ndim >= 2) {
     if (kchunk_req > 0) {
       kchunk = kchunk_req;
+    } else if (v1.fn_wide) {
+      // strips on their own warps: about 16 warps per SM, 4 to 32 rows each (a
+      // chunk re-reads four rows; stages 1 and 2 at 1024^2 take 28.2 and 26.6 us
+      // with 16 rows, 33.1 and 30.7 with 24, 31.6 and 28.7 with 4; at 256 x 768
+      // 13.2 and 12.3 us with 4, 16.4 and 14.3 with 8; at 4096^2 293 and 278 us
+      // with 32, 300 and 287 with 64)
+      const long strips = (h->n[0] + 27) / 28;
+      const long rows = (strips * nm + 16L * h->num_sms - 1) / (16L * h->num_sms);
+      kchunk = (int)(rows < 4 ? 4 : rows > 32 ? 32 : rows);
     } else {
       // about four CTAs per SM per stage, at least 8 planes per CTA
       const long target = 4L * h->num_sms;

@@ -139,6 +139,10 @@ int configure(genasis_batch* b, int tile, int chunk) {
                                       : batch_variant_dw(b->solver, 1, tile, &v1) && batch_variant_dw(b->solver, 2, tile, &v2);
   if (!ok) return fail(GENASIS_EINVAL, "no compiled batch kernel for this configuration");
   const int cols = v1.cols;
+  size_t most = 0;
+  for (const HostProblem& h : b->hp) most = std::max(most, h.ncell);
+  for (BatchVariant* v : {&v1, &v2})
+    if (v->fn_wide && most > ((size_t)1 << 30)) v->fn = v->fn_wide;
   if (chunk == 0) chunk = 32;
   // work items: (problem, x tile, y chunk), largest first
   struct Item {
@@ -148,11 +152,12 @@ int configure(genasis_batch* b, int tile, int chunk) {
   std::vector<Item> items;
   for (int p = 0; p < b->nprob; ++p) {
     const HostProblem& h = b->hp[p];
-    const int gx = (h.n[0] + cols - 1) / cols;
+    const int width = h.ndim == 1 ? cols * v1.group_1d : cols;
+    const int gx = (h.n[0] + width - 1) / width;
     const int gz = h.ndim == 2 ? (h.n[1] + chunk - 1) / chunk : 1;
     for (int x = 0; x < gx; ++x)
       for (int z = 0; z < gz; ++z) {
-        const long w = std::min(cols, h.n[0] - x * cols);
+        const long w = std::min(width, h.n[0] - x * width);
         const long rows = h.ndim == 2 ? std::min(chunk, h.n[1] - z * chunk) + 4 : 1;
         items.push_back({w * rows, {p, x, z, 0}});
       }
@@ -171,7 +176,7 @@ int configure(genasis_batch* b, int tile, int chunk) {
   GH_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ1, v1.fn, v1.tx, v1.smem));
   GH_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ2, v2.fn, v2.tx, v2.smem));
   int occ = std::max(1, std::min(occ1, occ2));
-  b->ctas = std::min(b->nitems, occ * b->num_sms);
+  b->ctas = std::min((b->nitems + v1.warps - 1) / v1.warps, occ * b->num_sms);
   if (b->ctas < 1) b->ctas = 1;
   b->v1 = v1;
   b->v2 = v2;

@@ -94,8 +94,8 @@ __device__ __forceinline__ dw minmod3(dw a, dw b, dw c) {
   return lo.hi > 0.0f ? lo : (hi.hi < 0.0f ? hi : dw(0.0f, 0.0f));
 }
 
-// max(0, a, b), x == 0 and x >= 0 for the wave speeds and the HLLC branch:
-// plain for float and double word, on the integer pipe for double.
+// max(0, a, b) for the wave speeds: plain for float and double word, on the
+// integer pipe for double.
 template <class T>
 __device__ __forceinline__ T max0(T a, T b) { return fmax(T(0), fmax(a, b)); }
 __device__ __forceinline__ double max0(double a, double b) {
@@ -103,12 +103,12 @@ __device__ __forceinline__ double max0(double a, double b) {
   const double m = ka < kb ? b : a;
   return (ka < kb ? kb : ka) > 0 ? m : 0.0;
 }
-template <class T>
-__device__ __forceinline__ bool is_zero(T x) { return x == T(0); }
+
+// x == 0 and x >= 0; FP64 tests run on the integer pipe.
+__device__ __forceinline__ bool is_zero(float x) { return x == 0.0f; }
 __device__ __forceinline__ bool is_zero(dw x) { return x.hi == 0.0f; }
 __device__ __forceinline__ bool is_zero(double x) { return ((unsigned long long)__double_as_longlong(x) << 1) == 0; }
-template <class T>
-__device__ __forceinline__ bool nonneg(T x) { return x >= T(0); }
+__device__ __forceinline__ bool nonneg(float x) { return x >= 0.0f; }
 __device__ __forceinline__ bool nonneg(dw x) { return x.hi >= 0.0f; }
 __device__ __forceinline__ bool nonneg(double x) { return okey(x) >= -1; }
 
@@ -321,6 +321,8 @@ __device__ __forceinline__ void recover(const float (&u)[NDIM + 2], float (&w)[N
 //                  D* = a_K / (S_K - alpha_m)
 //                  p* = p_K + a_K (alpha_m - v_K)
 //                  G* = (d_K G_K - p_K v_K + p* alpha_m) / (S_K - alpha_m)
+//                     = (d_K G_K + (alpha_m - v_K)(p_K + a_K alpha_m))
+//                       / (S_K - alpha_m)
 //                which are the outer jump conditions of Sec. 3.2 solved for the
 //                middle state (this form satisfies p*_L = p*_R).  The middle
 //                state moves with alpha_m, so its flux is
@@ -390,13 +392,14 @@ __device__ __forceinline__ void face_flux(const T (&wl)[NDIM + 2], const T (&wr)
     for (int v = 0; v < NV; ++v) wK[v] = left ? wl[v] : wr[v];
     const T vK = wK[1 + Q];
     const T a = is_zero(SK) ? vK : alpha;
+    const T dv = sub_rn(a, vK);
     T v2 = mul_rn(wK[1], wK[1]);
 #pragma unroll
     for (int q = 1; q < NDIM; ++q) v2 = fma_rn(wK[1 + q], wK[1 + q], v2);
     const T GK = fma_rn(half_of(wK[0]), v2, wK[NV - 1]);
     const T r = frcp(sub_rn(SK, a));
-    const T ps = fma_rn(aK, sub_rn(a, vK), pK);
-    const T Gs = mul_rn(fma_rn(dK, GK, fma_rn(ps, a, -mul_rn(pK, vK))), r);
+    const T ps = fma_rn(aK, dv, pK);
+    const T Gs = mul_rn(fma_rn(dK, GK, mul_rn(dv, fma_rn(aK, a, pK))), r);
     const T m = mul_rn(mul_rn(aK, r), a);  // D* alpha_m
     F[0] = m;
 #pragma unroll

@@ -14,6 +14,7 @@ struct StageVariant {
   int threads;         // threads per CTA
   int tma = 0;         // 1: takes TmaStageArgs (state planes staged by TMA), see stage_tma.cuh
   int box_x = 0, box_y = 0;  // TMA box of one plane (cells along x and y)
+  const void* fn_wide = nullptr;  // the kernel for meshes of more than 2^30 cells, where it is another
   int pair = 0;        // 1: two march planes per thread (stage_pair.cuh); chunks of an even plane count
 };
 

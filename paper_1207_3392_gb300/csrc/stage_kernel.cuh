@@ -536,6 +536,18 @@ struct StageKernel {
     }
   }
 
+  // External force and power (Sec. 4.3.2): S_q -= D dPhi/dq,
+  // G -= sum_q S_q dPhi/dq, from the cell's stage-input state w.
+  static __device__ __forceinline__ void add_source(const StageArgs<T>& A, const T (&w)[NV], T (&L)[NV]) {
+    T power = T(0);
+#pragma unroll
+    for (int q = 0; q < NDIM; ++q) {
+      L[1 + q] = fma_rn(-w[0], A.grad_phi[q], L[1 + q]);
+      power = fma_rn(mul_rn(w[0], w[1 + q]), A.grad_phi[q], power);
+    }
+    L[NV - 1] = sub_rn(L[NV - 1], power);
+  }
+
   static __device__ __forceinline__ bool nonphysical(const T (&w)[NV], T gm1) {
     bool bad = !(w[0] > T(0)) || !(gm1 * w[NV - 1] > T(0));
 #pragma unroll
@@ -697,22 +709,11 @@ struct StageKernel {
         }
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
-          T d = mul_rn(sub_rn(fxr[v], fxl[v]), iwx);
-          if constexpr (HAS_Y) d = fma_rn(sub_rn(fyt[v], fyb[v]), iwy, d);
-          if constexpr (MARCH) d = fma_rn(sub_rn(fhi[v], flo[v]), iwm, d);
-          L[v] = -d;
+          L[v] = mul_rn(sub_rn(fxl[v], fxr[v]), iwx);  // minus the divergence
+          if constexpr (HAS_Y) L[v] = fma_rn(sub_rn(fyb[v], fyt[v]), iwy, L[v]);
+          if constexpr (MARCH) L[v] = fma_rn(sub_rn(flo[v], fhi[v]), iwm, L[v]);
         }
-        if (A.has_source) {
-          // external force and power (Sec. 4.3.2): S_q -= D dPhi/dq,
-          // G -= sum_q S_q dPhi/dq, from this cell's stage-input state
-          T power = T(0);
-#pragma unroll
-          for (int q = 0; q < NDIM; ++q) {
-            L[1 + q] = fma_rn(-wown[0], A.grad_phi[q], L[1 + q]);
-            power = fma_rn(mul_rn(wown[0], wown[1 + q]), A.grad_phi[q], power);
-          }
-          L[NV - 1] = sub_rn(L[NV - 1], power);
-        }
+        if (A.has_source) add_source(A, wown, L);
         const size_t c = cell(A, ca, cb, m);
         bad |= nonphysical(wown, A.gm1);
         if (STAGE == 1) {

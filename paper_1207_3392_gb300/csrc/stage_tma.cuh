@@ -396,10 +396,9 @@ struct StageTma {
         T L[NV];
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
-          T d = mul_rn(sub_rn(S.fx[v][ty][tx + 1], S.fx[v][ty][tx]), iwx);
-          d = fma_rn(sub_rn(S.fy[v][ty + 1][tx], S.fy[v][ty][tx]), iwy, d);
-          d = fma_rn(sub_rn(fhi[v], flo[v]), iwm, d);
-          L[v] = -d;
+          T d = mul_rn(sub_rn(S.fx[v][ty][tx], S.fx[v][ty][tx + 1]), iwx);  // minus the divergence
+          d = fma_rn(sub_rn(S.fy[v][ty][tx], S.fy[v][ty + 1][tx]), iwy, d);
+          L[v] = fma_rn(sub_rn(flo[v], fhi[v]), iwm, d);
         }
         if (A.has_source) {
           T power = T(0);

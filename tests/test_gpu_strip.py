@@ -1,0 +1,92 @@
+"""The 2D FP32 strips (one warp per 28 columns) and the FP32 batch built on them,
+against the oracle at the sizes where a strip can go wrong: meshes narrower than
+a strip, its edges and remainders, chunks of rows and their remainders, every
+boundary rule, groups of 1D strips; and one mesh of more than 2^30 cells (64-bit
+offsets)."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_1207_3392_gb300 import hydro as H
+from paper_1207_3392_gb300 import problems as P
+from parity_util import TOL_FP32, check, oracle_run
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_1207_3392_gb300 import build
+    build.build()
+    yield
+
+
+@pytest.mark.parametrize("bc", [P.PERIODIC, P.REFLECT, P.OUTFLOW])
+@pytest.mark.parametrize("n", [(2, 2), (3, 9), (27, 5), (28, 33), (29, 4), (56, 3), (57, 38), (226, 7)])
+def test_strip_edges_match_the_oracle(n, bc):
+    pr = P.random_blocks(2, n, seed=40 + n[0], bc=bc).with_(grad_phi=(0.2, -0.3, 0.0))
+    for solver in (H.HLL, H.HLLC):
+        Uo, to = oracle_run(pr, solver=solver, steps=3)
+        ref = None
+        for tile in (0, 1, 2):
+            for kc in (0, 1, 4, 5):
+                h = H.Hydro.from_problem(pr, precision=H.FP32_MIXED, solver=solver)
+                h.set_tile(tile, kc)
+                t = h.advance(3, pr.cfl)
+                U = h.get_conserved(precision=H.FP64)
+                tot = h.step_totals()
+                h.close()
+                assert t == pytest.approx(to, rel=1e-5)
+                if ref is None:
+                    ref, ref_tot = U, tot
+                    check(U, Uo, 2, TOL_FP32, f"{n} bc={bc} solver={solver}")
+                np.testing.assert_array_equal(U, ref, err_msg=f"tile {tile} kchunk {kc}")
+                # the same cells summed in another grouping: 48-bit sums
+                np.testing.assert_allclose(tot, ref_tot, rtol=1e-12, atol=1e-12 * np.max(np.abs(ref_tot)))
+
+
+def test_batch_of_edge_sizes_matches_the_oracle():
+    probs = [P.random_blocks(1, (m,), seed=m, bc=bc) for m in (2, 27, 28, 29, 223, 224, 225, 449)
+             for bc in (P.PERIODIC, P.REFLECT, P.OUTFLOW)]
+    probs += [P.random_blocks(2, m, seed=m[0], bc=P.REFLECT) for m in ((2, 2), (28, 31), (29, 33), (57, 65))]
+    b = H.Batch(probs, precision=H.FP32_MIXED)
+    for i, pr in enumerate(probs):
+        b.set_primitive(i, pr.rho, pr.vel, pr.p)
+    b.run(4, 0.4)
+    assert b.status() == -1
+    for i, pr in enumerate(probs):
+        Uo, _ = oracle_run(pr.with_(cfl=0.4), steps=4)
+        check(b.get_conserved(i), Uo, pr.ndim, TOL_FP32, f"problem {i} {pr.n}")
+    b.close()
+
+
+def test_mesh_beyond_2_30_cells():
+    """A Sod tube along x on 65536 x 16400 cells: sampled rows, up to the last,
+    are bitwise the first row and match the 1D oracle step."""
+    import torch
+    nx, ny = 65536, 16400
+    if torch.cuda.mem_get_info()[0] < 90e9:
+        pytest.skip("needs 90 GB of device memory")
+    pr = P.sod(nx)
+    g = O.Grid(pr)
+    U1 = O.initial_state(pr, g).astype(np.float32)
+    U = torch.zeros((4, ny, nx), dtype=torch.float32, device="cuda")
+    for v, a in zip((0, 1, 3), U1):
+        U[v] = torch.from_numpy(a).cuda()
+    h = H.Hydro(2, (nx, ny), [pr.widths[0], np.full(ny, 1.0)], (P.OUTFLOW,) * 2, (P.OUTFLOW,) * 2, 1.4, H.HLLC,
+                precision=H.FP32_MIXED)
+    torch.cuda.synchronize()
+    h.set_conserved(U)
+    dt = h.compute_dt(0.4)
+    h.step(dt)
+    h.get_conserved(U)
+    h.close()
+    rows = U[:, [0, 1, ny // 2, ny - 2, ny - 1]].cpu().numpy()
+    del U
+    torch.cuda.empty_cache()
+    for k in range(1, rows.shape[1]):
+        np.testing.assert_array_equal(rows[:, k], rows[:, 0])
+    Uo = O.step(g, U1.astype(np.float64), dt)
+    check(rows[[0, 1, 3], 0].astype(np.float64), Uo, 1, TOL_FP32, "wide mesh")
