@@ -247,12 +247,15 @@ struct StripKernel {
     }
     if (STAGE == 1 && own) {
       if (A.want_totals) {
+        // the width as three floats: the pair alone would leave 2^-49 of it out
         const dw dx = dw(A.wdh[0][col], A.wdl[0][col]);
+        const float dx3 = (float)((A.wd[0][col] - (double)dx.hi) - (double)dx.lo);
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
           dw c;
           fast_two_sum(tcol[v].hi, tcol[v].lo, c.hi, c.lo);
-          tot[v] = c * dx;
+          const dw r = c * dx;
+          fast_two_sum(r.hi, fma_rn(c.hi, dx3, r.lo), tot[v].hi, tot[v].lo);
         }
       }
       speed_out = fmaxf(speed_out, speed_max);
