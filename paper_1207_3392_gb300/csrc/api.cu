@@ -62,6 +62,17 @@ bool stage_variant(int ndim, int prec, int solver, int stage, int tile, StageVar
 
 int stage_tile_count(int ndim, int prec) { return tile_count(ndim, prec); }
 
+// Independent warps wherever they are compiled: 3D FP32 (tile 14), 2D and 3D
+// double word (tiles 1 and 4).  A strip owns 28 columns, a tile 32: with 29 to
+// 32 columns along x in 3D two half-empty strips lose to one tile (29 x 160 x
+// 160: 96 to 99 us a step against 88 in FP32, 562 against 499 in double word).
+int stage_tile_default(int ndim, int prec, int solver, int nx) {
+  if (ndim == 3 && nx > 28 && nx <= 32) return 0;
+  if (prec == GENASIS_FP64_DW) return ndim == 3 ? 4 : ndim == 2 ? 1 : 0;
+  if (prec == GENASIS_FP32_MIXED && ndim == 3 && solver != GENASIS_HLLC_SWITCH) return 14;
+  return 0;
+}
+
 }  // namespace gh
 
 using namespace gh;
@@ -173,17 +184,37 @@ int configure(genasis_hydro* h, int tile, int kchunk_req) {
     return fail(GENASIS_EINVAL, "tile %d stages the state with TMA, which needs a 3D FP32 mesh with n[0] a multiple of 4",
                 tile);
   for (StageVariant* v : {&v1, &v2})
-    if (v->fn_wide && h->ncell > ((size_t)1 << 30)) v->fn = v->fn_wide;
-  const int gx = (h->n[0] + v1.tx - 1) / v1.tx;
-  const int gy = h->ndim == 3 ? (h->n[1] + v1.ty - 1) / v1.ty : 1;
-  const int gx2 = (h->n[0] + v2.tx - 1) / v2.tx;
-  const int gy2 = h->ndim == 3 ? (h->n[1] + v2.ty - 1) / v2.ty : 1;
+    if (h->ncell > ((size_t)1 << 30) && v->fn_wide) {
+      v->fn = v->fn_wide;
+      v->xy_fn = v->xy_fn_wide;
+      v->smem = 0;
+    } else if (v->fn_odd && ((size_t)h->n[0] * h->n[1]) % 4) {
+      v->fn = v->fn_odd;
+      v->smem = 0;
+    }
+  const bool split = v1.xy_fn != nullptr;  // 3D on independent warps: threads over the (x, y) plane
+  const size_t plane = (size_t)h->n[0] * h->n[1];
+  const int gx = split ? (int)((plane + v1.tx - 1) / v1.tx) : (h->n[0] + v1.tx - 1) / v1.tx;
+  const int gy = split ? 1 : h->ndim == 3 ? (h->n[1] + v1.ty - 1) / v1.ty : 1;
+  const int gx2 = split ? gx : (h->n[0] + v2.tx - 1) / v2.tx;
+  const int gy2 = split ? 1 : h->ndim == 3 ? (h->n[1] + v2.ty - 1) / v2.ty : 1;
   const int nm = h->ndim >= 2 ? h->n[h->ndim - 1] : 1;
   int kchunk = 1, gz = 1;
+  // independent warps: least rows or planes of a chunk, and the warps wanted in 3D
+  const long least = h->prec == GENASIS_FP64_DW ? 2 : 4;
+  const long wanted = (h->prec == GENASIS_FP64_DW ? 24L : 36L) * h->num_sms;
   if (h->ndim >= 2) {
     if (kchunk_req > 0) {
       kchunk = kchunk_req;
-    } else if (v1.fn_wide) {
+    } else if (split) {
+      // columns of threads: one and a half times the warps that fit, 4 (double
+      // word 2) to 48 planes each (a chunk re-reads four planes; stage 1 + 2 of
+      // 256^3 with 32, 48 and 64 planes: 1020, 1028 and 1041 us; a step of 16^3
+      // takes 27 us with 4 planes, 48 with 16; of 128^3 162 us with 16, 168 with 8)
+      const long warps = (long)((plane + 31) / 32);
+      const long rows = (warps * nm + wanted - 1) / wanted;
+      kchunk = (int)(rows < least ? least : rows > 48 ? 48 : rows);
+    } else if (v1.strips) {
       // strips on their own warps: about 16 warps per SM, 4 to 32 rows each (a
       // chunk re-reads four rows; stages 1 and 2 at 1024^2 take 28.2 and 26.6 us
       // with 16 rows, 33.1 and 30.7 with 24, 31.6 and 28.7 with 4; at 256 x 768
@@ -191,7 +222,7 @@ int configure(genasis_hydro* h, int tile, int kchunk_req) {
       // with 32, 300 and 287 with 64)
       const long strips = (h->n[0] + 27) / 28;
       const long rows = (strips * nm + 16L * h->num_sms - 1) / (16L * h->num_sms);
-      kchunk = (int)(rows < 4 ? 4 : rows > 32 ? 32 : rows);
+      kchunk = (int)(rows < least ? least : rows > 32 ? 32 : rows);
     } else {
       // about four CTAs per SM per stage, at least 8 planes per CTA
       const long target = 4L * h->num_sms;
@@ -204,6 +235,17 @@ int configure(genasis_hydro* h, int tile, int kchunk_req) {
     if (kchunk > nm) kchunk = nm;
     if ((v1.pair || v2.pair) && (kchunk & 1)) ++kchunk;  // whole plane pairs per chunk
     gz = (nm + kchunk - 1) / kchunk;
+  }
+  h->xy_strips = 0;
+  if (split) {
+    // strips along y: the same rule, up to 64 rows
+    h->xy_strips = (h->n[0] + 27) / 28;
+    const long units = (long)h->xy_strips * h->n[2];
+    long rows = (units * h->n[1] + wanted - 1) / wanted;
+    rows = rows < least ? least : rows > 64 ? 64 : rows;
+    if ((h->n[1] + rows - 1) / rows > 65535) rows = (h->n[1] + 65534) / 65535;
+    h->xy_rows = (int)rows;
+    h->xy_grid = dim3((unsigned)((units + v1.xy_warps - 1) / v1.xy_warps), (unsigned)((h->n[1] + rows - 1) / rows), 1);
   }
   const size_t nblk = (size_t)gx * gy * gz;
   for (const StageVariant* v : {&v1, &v2}) {
@@ -303,6 +345,10 @@ int launch_stage(genasis_hydro* h, int stage, cudaStream_t st) {
   }
   StageArgs<T> A = stage_args<T>(h, stage);
   void* p[] = {&A};
+  if (v.xy_fn) {
+    void* q[] = {&A, &h->xy_strips, &h->xy_rows};
+    GH_CK(cudaLaunchKernel(v.xy_fn, h->xy_grid, dim3(32 * v.xy_warps), q, 0, st));
+  }
   GH_CK(cudaLaunchKernel(v.fn, grid, dim3(v.threads), p, v.smem, st));
   return GENASIS_OK;
 }
@@ -609,7 +655,7 @@ int genasis_hydro_create(const genasis_hydro_desc* d, genasis_hydro_t* out) {
   rc = h->prec == GENASIS_FP64         ? upload_geometry<double>(h, d)
        : h->prec == GENASIS_FP32_MIXED ? upload_geometry<float>(h, d)
                                        : upload_geometry<dw>(h, d);
-  if (!rc) rc = configure(h, 0, 0);
+  if (!rc) rc = configure(h, stage_tile_default(h->ndim, h->prec, h->solver, h->n[0]), 0);
   if (rc) {
     free_all(h);
     return rc;
@@ -938,7 +984,7 @@ int genasis_hydro_launches_per_step(genasis_hydro_t h) {
     const int n = genasis_learned_launches_per_step(h->lf);
     return n < 0 ? n : n + 1;
   }
-  return h->solver == GENASIS_HLLC_SWITCH ? 5 : 3;
+  return (h->solver == GENASIS_HLLC_SWITCH ? 5 : 3) + (h->v1.xy_fn ? 2 : 0);
 }
 
 int genasis_hydro_profile_step(genasis_hydro_t h, double cfl, float* ms) {

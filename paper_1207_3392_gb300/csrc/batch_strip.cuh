@@ -19,8 +19,8 @@ constexpr int STRIP_GROUP_1D = 8;  // strips of a 1D item: one has a single row,
 
 template <int SOLVER, int STAGE, int NW, bool WIDE>
 __global__ void __launch_bounds__(32 * NW, 32 / NW) hydro_batch_strip_kernel(const BatchArgs<float> B) {
-  using K1 = StripKernel<1, SOLVER, STAGE, WIDE>;
-  using K2 = StripKernel<2, SOLVER, STAGE, WIDE>;
+  using K1 = StripKernel<1, float, SOLVER, STAGE, WIDE>;
+  using K2 = StripKernel<2, float, SOLVER, STAGE, WIDE>;
   using Args = BatchKernel<float, SOLVER, STAGE, 128>;
   const int lane = threadIdx.x & 31;
   for (;;) {
@@ -38,13 +38,13 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) hydro_batch_strip_kernel(con
       for (int k = 0; k < STRIP_GROUP_1D; ++k) {
         const int x0 = (w.tx * STRIP_GROUP_1D + k) * STRIP_OWN;
         if (x0 >= A.n[0]) break;
-        K1::strip(A, x0, 0, 1, speed, tot, bad);
+        K1::strip(A, x0, 0, 1, 0, speed, tot, bad);
       }
     } else {
       dw tot[4];
       const StageArgs<float> A = Args::template args_for<2>(B, P, w.prob);
       const int m0 = w.chunk * B.kchunk;
-      K2::strip(A, w.tx * STRIP_OWN, m0, min(A.n[1], m0 + B.kchunk), speed, tot, bad);
+      K2::strip(A, w.tx * STRIP_OWN, m0, min(A.n[1], m0 + B.kchunk), 0, speed, tot, bad);
     }
     if (bad) atomicOr(B.status + w.prob, STATUS_NONPHYS);
     if (STAGE == 1) {

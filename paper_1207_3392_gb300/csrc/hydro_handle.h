@@ -40,6 +40,9 @@ struct genasis_hydro {
   int tile = 0, kchunk_req = 0, kchunk = 1;
   gh::StageVariant v1{}, v2{};
   dim3 grid, grid2;  // stage 1 / stage 2 (the two may use different tile shapes)
+  // 3D on independent warps: strips per row, rows per warp and grid of the x/y launch
+  int xy_strips = 0, xy_rows = 0;
+  dim3 xy_grid;
   // tensor maps of U[0], U[1] and K for TMA variants (valid when v1.tma or v2.tma)
   CUtensorMap tmap[3];
   CUtensorMap fmap[2];     // U[0], U[1] with the box of the TMA shock-flag pass

@@ -39,22 +39,49 @@ inline bool pick_switch(int stage, StageVariant* out) {
   return true;
 }
 
-// 2D FP32 on independent warps (stage_strip.cuh), NW strips per CTA.
-template <int SOLVER, int STAGE, int NW>
+// 2D on independent warps (stage_strip.cuh), NW strips per CTA.
+template <class T, int SOLVER, int STAGE, int NW>
 inline void fill_strip(StageVariant* out) {
-  out->fn = reinterpret_cast<const void*>(&hydro_strip_kernel<SOLVER, STAGE, NW, false>);
-  out->fn_wide = reinterpret_cast<const void*>(&hydro_strip_kernel<SOLVER, STAGE, NW, true>);
+  out->fn = reinterpret_cast<const void*>(&hydro_strip_kernel<T, SOLVER, STAGE, NW, false>);
+  out->fn_wide = reinterpret_cast<const void*>(&hydro_strip_kernel<T, SOLVER, STAGE, NW, true>);
   out->smem = 0;
   out->tx = STRIP_OWN * NW;
   out->ty = 1;
   out->threads = 32 * NW;
+  out->strips = 1;
 }
-template <int NW>
+template <class T, int NW>
 inline bool pick_strip(int solver, int stage, StageVariant* out) {
-  if (solver == SOLVER_HLL && stage == 1) fill_strip<SOLVER_HLL, 1, NW>(out);
-  else if (solver == SOLVER_HLL && stage == 2) fill_strip<SOLVER_HLL, 2, NW>(out);
-  else if (solver == SOLVER_HLLC && stage == 1) fill_strip<SOLVER_HLLC, 1, NW>(out);
-  else if (solver == SOLVER_HLLC && stage == 2) fill_strip<SOLVER_HLLC, 2, NW>(out);
+  if (solver == SOLVER_HLL && stage == 1) fill_strip<T, SOLVER_HLL, 1, NW>(out);
+  else if (solver == SOLVER_HLL && stage == 2) fill_strip<T, SOLVER_HLL, 2, NW>(out);
+  else if (solver == SOLVER_HLLC && stage == 1) fill_strip<T, SOLVER_HLLC, 1, NW>(out);
+  else if (solver == SOLVER_HLLC && stage == 2) fill_strip<T, SOLVER_HLLC, 2, NW>(out);
+  else return false;
+  return true;
+}
+
+// 3D on independent warps: the strips' launch (x and y parts), then ZMarch's.
+template <class T, int SOLVER, int STAGE>
+inline void fill_split(StageVariant* out) {
+  constexpr int NW = 4;
+  out->xy_fn = reinterpret_cast<const void*>(&hydro_strip_xy_kernel<T, SOLVER, STAGE, NW, false>);
+  out->xy_fn_wide = reinterpret_cast<const void*>(&hydro_strip_xy_kernel<T, SOLVER, STAGE, NW, true>);
+  out->xy_warps = NW;
+  constexpr bool RING = std::is_same<T, float>::value;
+  out->fn = reinterpret_cast<const void*>(&hydro_march_z_kernel<T, SOLVER, STAGE, false, RING>);
+  out->smem = ZMarch<T, SOLVER, STAGE, false, RING>::SMEM;
+  if (RING) out->fn_odd = reinterpret_cast<const void*>(&hydro_march_z_kernel<T, SOLVER, STAGE, false, false>);
+  out->fn_wide = reinterpret_cast<const void*>(&hydro_march_z_kernel<T, SOLVER, STAGE, true, false>);
+  out->tx = 128;
+  out->ty = 1;
+  out->threads = 128;
+}
+template <class T>
+inline bool pick_split(int solver, int stage, StageVariant* out) {
+  if (solver == SOLVER_HLL && stage == 1) fill_split<T, SOLVER_HLL, 1>(out);
+  else if (solver == SOLVER_HLL && stage == 2) fill_split<T, SOLVER_HLL, 2>(out);
+  else if (solver == SOLVER_HLLC && stage == 1) fill_split<T, SOLVER_HLLC, 1>(out);
+  else if (solver == SOLVER_HLLC && stage == 2) fill_split<T, SOLVER_HLLC, 2>(out);
   else return false;
   return true;
 }

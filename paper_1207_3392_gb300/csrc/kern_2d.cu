@@ -12,9 +12,9 @@ bool stage_variant_2d(bool fp64, int solver, int stage, int tile, StageVariant* 
   if (solver == SOLVER_HLLC_SW)
     return tile == 0 && (fp64 ? pick_switch<2, double, 128, 1>(stage, out) : pick_switch<2, float, 128, 1>(stage, out));
   switch (tile) {
-    case 0: return fp64 ? pick_variant<2, double, 128, 1>(solver, stage, out) : pick_strip<2>(solver, stage, out);
-    case 1: return fp64 ? pick_variant<2, double, 64, 1>(solver, stage, out) : pick_strip<4>(solver, stage, out);
-    case 2: return fp64 ? pick_variant<2, double, 256, 1>(solver, stage, out) : pick_strip<8>(solver, stage, out);
+    case 0: return fp64 ? pick_variant<2, double, 128, 1>(solver, stage, out) : pick_strip<float, 2>(solver, stage, out);
+    case 1: return fp64 ? pick_variant<2, double, 64, 1>(solver, stage, out) : pick_strip<float, 4>(solver, stage, out);
+    case 2: return fp64 ? pick_variant<2, double, 256, 1>(solver, stage, out) : pick_strip<float, 8>(solver, stage, out);
   }
   return false;
 }

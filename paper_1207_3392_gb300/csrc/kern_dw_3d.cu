@@ -12,6 +12,7 @@ bool stage_variant_dw_3d(int solver, int stage, int tile, StageVariant* out) {
     case 1: return pick_variant<3, dw, 32, 4, 2>(solver, stage, out);
     case 2: return pick_variant<3, dw, 32, 8, 1>(solver, stage, out);
     case 3: return pick_variant<3, dw, 32, 4, 4>(solver, stage, out);
+    case 4: return stage_variant_dw_split(solver, stage, out);
   }
   return false;
 }

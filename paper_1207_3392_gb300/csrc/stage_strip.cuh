@@ -1,21 +1,33 @@
-// stage_strip.cuh -- one RK stage of a 1D or 2D FP32 mesh on independent warps.
+// stage_strip.cuh -- RK stages on independent warps.
 //
-// A warp takes a strip of 28 columns (lane l holds column x0 + l - 2: two
-// neighbours on each side) and marches along y.  The march axis lives in a
-// register ring, as in stage_kernel.cuh; along x the warp's own shuffles move
-// what neighbouring columns need: W of the two neighbours for the slope, the
-// upper face value of the lower neighbour, and the flux of the upper face.
-// Each slope and each face flux is computed once per lane, nothing goes
-// through shared memory, and no warp waits for another.
+// 1D and 2D (StripKernel): a warp takes a strip of 28 columns (lane l holds
+// column x0 + l - 2: two neighbours on each side) and marches along y.  The
+// march axis lives in a register ring, as in stage_kernel.cuh; along x the
+// warp's own shuffles move what neighbouring columns need: W of the two
+// neighbours for the slope, the upper face value of the lower neighbour, and
+// the flux of the upper face.  Each slope and each face flux is computed once
+// per lane, nothing goes through shared memory, and no warp waits for another.
 //
-// What bounds it, and why this split: the 2D row tiles it replaced (one row of
-// a CTA per plane, two barriers a row, every x slope formed twice) ran about
+// 3D: two launches a stage.  The strips march along y in every plane and leave
+// minus the x and y parts of the divergence in the stage's output array; then
+// every thread takes one (x, y) column and marches along z (ZMarch): it adds
+// the z part and finishes the cell (source, output, CFL speed, totals).
+//
+// What bounds it, and why this split.  2D: the row tiles it replaced (one row
+// of a CTA per plane, two barriers a row, every x slope formed twice) ran about
 // 640 instructions a cell at 47-67% of the issue slots, their warps waiting at
-// the barriers.
-// Stages 1 and 2 of the row tiles and of the strips, HLLC with totals: 40.0 and
-// 36.9 -> 28.2 and 26.6 us at 1024^2, 22.7 and 18.4 -> 13.2 and 12.3 us at
-// 256 x 768.  565 and 523 instructions a cell at 1024^2 (of them 54 and 0 for
-// the compensated totals), 78% of the issue slots at 4096^2.
+// the barriers.  Stages 1 and 2 of the row tiles and of the strips, HLLC with
+// totals: 40.0 and 36.9 -> 28.2 and 26.6 us at 1024^2, 22.7 and 18.4 -> 13.2
+// and 12.3 us at 256 x 768.  565 and 523 instructions a cell at 1024^2 (of them
+// 54 and 0 for the compensated totals), 78% of the issue slots at 4096^2.
+// 3D, FP32 HLLC at 256^3: the 32 x 8 tiles ran 981 and 894 instructions a cell at
+// 64% of the issue slots, held back by two barriers a plane, 24 warps and 160
+// halo cells recovered for 256 own ones: stages 1 and 2 685 and 660 us.  Here
+// the strips run 485 and 512 (of 32 lanes 25.6 own a column at nx = 256) at 77%,
+// and ZMarch 440 and 324 at 79% and 66%: 493 and 490 us together.  The price is
+// memory traffic, 100 and 140 algorithmic bytes a cell for 40 and 60, half of
+// what the launches' times could move.  Double word at 128^3: 558 and 549 ->
+// 464 and 530 us.
 #pragma once
 
 #include <type_traits>
@@ -24,182 +36,227 @@
 
 namespace gh {
 
+// The march loops take two rows an iteration in FP32, so that half of the
+// register ring's moves go (256^3: stages 1 and 2 508 and 502 -> 493 and 490
+// us; three rows: 505 and 506).  The double-word body is too large for that.
+template <class T>
+constexpr int march_unroll() { return sizeof(T) == 4 ? 2 : 1; }
 constexpr int STRIP_OWN = 28;  // columns a warp owns
 
-// Sum of four double-word values per lane over the warp: lanes 8 v .. 8 v + 7
-// of the result hold variable v.  Halving the variables with the lanes takes six
-// additions instead of twenty, and on FP32 pairs: as FP64 additions this tail
-// took 2-5 us of a stage on a mesh of 0.2 to 1 million cells.
-__device__ __forceinline__ dw shfl_xor_dw(dw x, int o) {
+__device__ __forceinline__ float lane_up(float x) { return __shfl_up_sync(0xffffffffu, x, 1); }
+__device__ __forceinline__ float lane_down(float x) { return __shfl_down_sync(0xffffffffu, x, 1); }
+__device__ __forceinline__ double lane_up(double x) { return __shfl_up_sync(0xffffffffu, x, 1); }
+__device__ __forceinline__ double lane_down(double x) { return __shfl_down_sync(0xffffffffu, x, 1); }
+__device__ __forceinline__ dw lane_up(dw x) { return dw(lane_up(x.hi), lane_up(x.lo)); }
+__device__ __forceinline__ dw lane_down(dw x) { return dw(lane_down(x.hi), lane_down(x.lo)); }
+
+// A lane's share of the conserved totals and their sum over the warp.  FP32 and
+// double-word states: double word, reduced on the FP32 pipes (as FP64 additions
+// this tail took 2-5 us of a stage on a mesh of 0.2 to 1 million cells); FP64:
+// FP64.
+template <class T>
+struct TotalSum {
+  using type = dw;
+};
+template <>
+struct TotalSum<double> {
+  using type = double;
+};
+
+// column sum times `area` (the FP64 product of the other axes' widths) as three
+// floats: the pair alone would leave 2^-49 of it out
+__device__ __forceinline__ dw share_of(dw c, double area) {
+  const float a1 = (float)area;
+  const double r1 = area - (double)a1;
+  const float a2 = (float)r1, a3 = (float)(r1 - (double)a2);
+  const dw r = c * dw(a1, a2);
+  dw s;
+  fast_two_sum(r.hi, __fmaf_rn(c.hi, a3, r.lo), s.hi, s.lo);
+  return s;
+}
+__device__ __forceinline__ dw share_of(const ColumnSum<float>& t, double area) {
+  dw c;
+  fast_two_sum(t.hi, t.lo, c.hi, c.lo);
+  return share_of(c, area);
+}
+__device__ __forceinline__ dw share_of(const ColumnSum<dw>& t, double area) { return share_of(t.s, area); }
+__device__ __forceinline__ double share_of(const ColumnSum<double>& t, double area) { return t.s * area; }
+
+__device__ __forceinline__ dw shfl_xor(dw x, int o) {
   return dw(__shfl_xor_sync(0xffffffffu, x.hi, o), __shfl_xor_sync(0xffffffffu, x.lo, o));
 }
-__device__ __forceinline__ dw warp_sum4(const dw (&s)[4]) {
+__device__ __forceinline__ double shfl_xor(double x, int o) { return __shfl_xor_sync(0xffffffffu, x, o); }
+// Sums of the NV shares over the warp into red[0 .. NV - 1].  Halving the first
+// four variables with the lanes takes six additions instead of twenty.
+template <int NV, class S>
+__device__ __forceinline__ void warp_totals(const S (&s)[NV], double* red) {
+  static_assert(NV == 4 || NV == 5, "2D or 3D");
   const int lane = threadIdx.x & 31;
   const bool h = lane & 16, q = lane & 8;
   // lanes 0..15 keep variables 0, 1; lanes 16..31 keep 2, 3
-  const dw a = (h ? s[2] : s[0]) + shfl_xor_dw(h ? s[0] : s[2], 16);
-  const dw b = (h ? s[3] : s[1]) + shfl_xor_dw(h ? s[1] : s[3], 16);
-  dw r = (q ? b : a) + shfl_xor_dw(q ? a : b, 8);
-  for (int o = 4; o > 0; o >>= 1) r += shfl_xor_dw(r, o);
-  return r;
+  const S a = (h ? s[2] : s[0]) + shfl_xor(h ? s[0] : s[2], 16);
+  const S b = (h ? s[3] : s[1]) + shfl_xor(h ? s[1] : s[3], 16);
+  S r = (q ? b : a) + shfl_xor(q ? a : b, 8);
+  for (int o = 4; o > 0; o >>= 1) r += shfl_xor(r, o);
+  if ((lane & 7) == 0) red[lane >> 3] = (double)r;  // lane 8 v holds variable v
+  if constexpr (NV == 5) {
+    S e = s[4];
+    for (int o = 16; o > 0; o >>= 1) e += shfl_xor(e, o);
+    if (lane == 0) red[4] = (double)e;
+  }
 }
 
 // WIDE: 64-bit cell offsets, for meshes of more than 2^30 cells.
-template <int NDIM, int SOLVER, int STAGE, bool WIDE>
-struct StripKernel {
-  static_assert(NDIM == 1 || NDIM == 2, "strips are 1D rows or 2D columns of rows");
-  using Base = StageKernel<NDIM, float, SOLVER, STAGE, 32, 1, false>;
+template <class T, bool WIDE>
+struct CellAccess {
   using Off = typename std::conditional<WIDE, size_t, unsigned>::type;
+  static __device__ __forceinline__ T at(const T* p, Off c) { return __ldg(p + c); }
+};
+
+// The march-axis step shared by the strips (along y) and ZMarch (along z):
+// limited slope and lower face value of the cell above from W of three
+// neighbours and the scaled difference dlo across the face below it, which
+// moves on to the face above (a cell's upper scaled difference and its upper
+// neighbour's lower one are the same number).
+template <int NV, class T>
+__device__ __forceinline__ void march_slope(const T (&wm)[NV], const T (&wc)[NV], const T (&wp)[NV], const Geo<T>& g,
+                                            T (&dlo)[NV], T (&s)[NV], T (&wr)[NV]) {
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    const T dhi = mul_rn(sub_rn(wp[v], wc[v]), g.tipc);
+    s[v] = minmod3(dlo[v], mul_rn(sub_rn(wp[v], wm[v]), g.ipm), dhi);
+    wr[v] = fma_rn(-s[v], g.h, wc[v]);
+    dlo[v] = dhi;
+  }
+}
+
+template <int NDIM, class T, int SOLVER, int STAGE, bool WIDE>
+struct StripKernel {
+  using Base = StageKernel<NDIM, T, SOLVER, STAGE, 32, 1, false>;
+  using Acc = CellAccess<T, WIDE>;
+  using Off = typename Acc::Off;
+  using Tot = typename TotalSum<T>::type;
   static constexpr int NV = NDIM + 2;
   static_assert(!Base::SW, "the switch runs on the row tiles");
 
-  static __device__ __forceinline__ float left_of(float x) { return __shfl_up_sync(0xffffffffu, x, 1); }
-  static __device__ __forceinline__ float right_of(float x) { return __shfl_down_sync(0xffffffffu, x, 1); }
-  // element c of a plane: the 32-bit byte offset is added to a base that is the
-  // same for the whole warp
-  static __device__ __forceinline__ float at(const float* p, Off c) {
-    return __ldg(reinterpret_cast<const float*>(reinterpret_cast<const char*>(p) + (Off)(c * 4)));
-  }
-  static __device__ __forceinline__ void set(float* p, Off c, float x) {
-    *reinterpret_cast<float*>(reinterpret_cast<char*>(p) + (Off)(c * 4)) = x;
-  }
-
   // minus the x part of the flux divergence of the lanes' cells of one row
   // (valid on the owned lanes), from W of the row
-  static __device__ __forceinline__ void x_part(const StageArgs<float>& A, const float (&w)[NV], const Geo<float>& g,
-                                                float iwx, float (&d)[NV]) {
-    float wl[NV], wr[NV], f[NV];
+  static __device__ __forceinline__ void x_part(const StageArgs<T>& A, const T (&w)[NV], const Geo<T>& g, T iwx,
+                                                T (&d)[NV]) {
+    T wl[NV], wr[NV], f[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-      float hi;
-      face_pair(limited_slope(left_of(w[v]), w[v], right_of(w[v]), g), g.h, w[v], wr[v], hi);
-      wl[v] = left_of(hi);
+      T hi;
+      face_pair(limited_slope(lane_up(w[v]), w[v], lane_down(w[v]), g), g.h, w[v], wr[v], hi);
+      wl[v] = lane_up(hi);
     }
-    face_flux<float, NDIM, 0, SOLVER>(wl, wr, A.gamma, A.gm1, f);  // the face below each column
+    face_flux<T, NDIM, 0, SOLVER>(wl, wr, A.gamma, A.gm1, f);  // the face below each column
 #pragma unroll
-    for (int v = 0; v < NV; ++v) d[v] = mul_rn(sub_rn(f[v], right_of(f[v])), iwx);
+    for (int v = 0; v < NV; ++v) d[v] = mul_rn(sub_rn(f[v], lane_down(f[v])), iwx);
   }
 
-  // Strip of columns x0 .. x0 + 27, rows m0 .. m1 - 1 (2D; 1D: the one row).
-  // Accumulates the lane's CFL speed and, with totals, its column's sum of
-  // U dy dx (stage 1), and the non-physical flag.  The whole warp calls it.
-  static __device__ __forceinline__ void strip(const StageArgs<float>& A, int x0, int m0, int m1, float& speed_out,
-                                               dw (&tot)[NV], bool& bad) {
+  // Strip of columns x0 .. x0 + 27, rows m0 .. m1 - 1 (1D: the one row; 3D: of
+  // plane k, and only minus the x and y parts of the divergence go to A.out).
+  // Accumulates the lane's CFL speed and, with totals, its share of them
+  // (stage 1), and the non-physical flag.  The whole warp calls it.
+  static __device__ __forceinline__ void strip(const StageArgs<T>& A, int x0, int m0, int m1, int k, T& speed_out,
+                                               Tot (&tot)[NV], bool& bad) {
     const int lane = threadIdx.x & 31;
-    const int nx = A.n[0], ny = NDIM == 2 ? A.n[1] : 1;
-    const size_t vs = (size_t)nx * ny;
-    const float dt = STAGE == 2 ? (float)(*A.dt) : 0.0f;
+    const int nx = A.n[0], ny = NDIM >= 2 ? A.n[1] : 1;
+    const size_t vs = NDIM == 3 ? (size_t)nx * ny * A.n[2] : (size_t)nx * ny;
+    const T dt = STAGE == 2 ? (T)(*A.dt) : T(0);
     const int col = x0 + lane - 2;
     const bool own = lane >= 2 && lane < 2 + STRIP_OWN && col < nx;
     bool fa;
-    const Off off = (Off)bc_map(col, nx, A.bc_lo[0], A.bc_hi[0], fa);
-    const Geo<float> gx = Base::geo(A, 0, col);
-    const float iwx = A.iw[0][min(col, nx + 1) + 2];
-    const float *un[NV], *k1[NV];
-    float* out[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      un[v] = A.un + v * vs;
-      k1[v] = A.k1 + v * vs;
-      out[v] = A.out + v * vs;
-    }
-    ColumnSum<float> tcol[NV];
-    float speed_max = 0.0f;
+    Off off = (Off)bc_map(col, nx, A.bc_lo[0], A.bc_hi[0], fa);
+    if constexpr (NDIM == 3) off += (Off)k * ((Off)nx * (Off)ny);
+    const Geo<T> gx = Base::geo(A, 0, col);
+    const T iwx = A.iw[0][min(col, nx + 1) + 2];
+    ColumnSum<T> tcol[NV];
+    T speed_max = T(0);
 
     // state of the cell at offset c (stage 2: U^n + dt K), x mirrored
-    auto load = [&](Off c, float (&u)[NV]) {
+    auto load = [&](Off c, T (&u)[NV]) {
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        u[v] = at(un[v], c);
-        if (STAGE == 2) u[v] = fma_rn(dt, at(k1[v], c), u[v]);
+        u[v] = Acc::at(A.un + v * vs, c);
+        if (STAGE == 2) u[v] = fma_rn(dt, Acc::at(A.k1 + v * vs, c), u[v]);
       }
     };
     // Epilogue of the own cell at offset c: L = minus the divergence, source,
     // output, and in stage 1 the CFL speed.
-    auto finish = [&](Off c, float (&L)[NV], const float (&w)[NV], float iwm) {
-      if (A.has_source) Base::add_source(A, w, L);
-      const float p = mul_rn(A.gm1, w[NV - 1]);
-      float vsum = fabsf(w[1]);
-      if constexpr (NDIM == 2) vsum = add_rn(vsum, fabsf(w[2]));
-      const bool ok = fminf(w[0], p) > 0.0f && w[0] == w[0] && p == p && vsum < INFINITY;
-      bad |= own && !ok;
-      if (STAGE == 1) {
-        const float cs = sound_speed(A.gamma, p, w[0]);
-        float s = mul_rn(add_rn(fabsf(w[1]), cs), iwx);
-        if constexpr (NDIM == 2) s = fmaxf(s, mul_rn(add_rn(fabsf(w[NDIM]), cs), iwm));
-        speed_max = fmaxf(speed_max, s);
+    auto finish = [&](Off c, T (&L)[NV], const T (&w)[NV], T iwm) {
+      if constexpr (NDIM == 3) {
         if (own) {
 #pragma unroll
-          for (int v = 0; v < NV; ++v) set(out[v], c, L[v]);
+          for (int v = 0; v < NV; ++v) A.out[v * vs + c] = L[v];
+        }
+        return;
+      }
+      if (A.has_source) Base::add_source(A, w, L);
+      bad |= own && Base::nonphysical(w, A.gm1);
+      if (STAGE == 1) {
+        const T cs = sound_speed(A.gamma, mul_rn(A.gm1, w[NV - 1]), w[0]);
+        T s = mul_rn(add_rn(fabs(w[1]), cs), iwx);
+        if constexpr (NDIM == 2) s = fmax(s, mul_rn(add_rn(fabs(w[NDIM]), cs), iwm));
+        speed_max = fmax(speed_max, s);
+        if (own) {
+#pragma unroll
+          for (int v = 0; v < NV; ++v) A.out[v * vs + c] = L[v];
         }
       } else {
-        const float hdt = 0.5f * dt;
-        float r[NV];
+        const T hdt = half_of(dt);
+        T r[NV];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) r[v] = fma_rn(hdt, add_rn(at(k1[v], c), L[v]), at(un[v], c));
+        for (int v = 0; v < NV; ++v)
+          r[v] = fma_rn(hdt, add_rn(Acc::at(A.k1 + v * vs, c), L[v]), Acc::at(A.un + v * vs, c));
         if (own) {
 #pragma unroll
-          for (int v = 0; v < NV; ++v) set(out[v], c, r[v]);
+          for (int v = 0; v < NV; ++v) A.out[v * vs + c] = r[v];
         }
       }
     };
 
     if constexpr (NDIM == 1) {
-      float u[NV], w[NV], L[NV];
+      T u[NV], w[NV], L[NV];
       load(off, u);
-      if (STAGE == 1 && A.want_totals) {
-#pragma unroll
-        for (int v = 0; v < NV; ++v) tcol[v].add_product(u[v], 1.0f, 0.0f);
-      }
       if (fa) u[1] = -u[1];
       recover<NDIM>(u, w);
       x_part(A, w, gx, iwx, L);
-      finish(off, L, w, 0.0f);
+      finish(off, L, w, T(0));
     } else {
       // W of row m (boundary-mapped); with totals also the row's share of the
       // column sums when it is one of the strip's own
-      auto row = [&](int m, float (&u)[NV]) {
-        bool fm;
-        const int sm = bc_map(m, ny, A.bc_lo[1], A.bc_hi[1], fm);
+      // (AHEAD: m >= 0, so that only the upper end needs the boundary rule)
+      auto row = [&](int m, T (&u)[NV], auto ahead) {
+        bool fm = false;
+        int sm = m;
+        if (!decltype(ahead)::value || m >= ny) sm = bc_map(m, ny, A.bc_lo[1], A.bc_hi[1], fm);
         load(off + (Off)sm * (Off)nx, u);
-        if (STAGE == 1 && A.want_totals && m >= m0 && m < m1) {
-          const float hi = A.wdh[1][m], lo = A.wdl[1][m];
+        if (NDIM == 2 && STAGE == 1 && A.want_totals && m >= m0 && m < m1) {
+          const T hi = A.wdh[1][m], lo = A.wdl[1][m];
 #pragma unroll
           for (int v = 0; v < NV; ++v) tcol[v].add_product(u[v], hi, lo);
         }
         if (fa) u[1] = -u[1];
         if (fm) u[2] = -u[2];
       };
-      // Limited slope and lower face value of row m + 1 from W(m), W(m + 1),
-      // W(m + 2) and the scaled difference dlo across face m + 1/2, which moves
-      // on to face m + 3/2 (a cell's upper scaled difference and its upper
-      // neighbour's lower one are the same number).
-      auto slope = [&](const float (&wk)[NV], const float (&wk1)[NV], const float (&w2)[NV], const Geo<float>& g,
-                       float (&dlo)[NV], float (&s)[NV], float (&wr)[NV]) {
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-          const float dhi = mul_rn(sub_rn(w2[v], wk1[v]), g.tipc);
-          s[v] = minmod3(dlo[v], mul_rn(sub_rn(w2[v], wk[v]), g.ipm), dhi);
-          wr[v] = fma_rn(-s[v], g.h, wk1[v]);
-          dlo[v] = dhi;
-        }
-      };
       // At the top of iteration m: wk = W(m), wk1 = W(m + 1), dlo = the scaled
       // difference across face m + 1/2, hi = the upper face value of cell m,
       // flo = the flux through face m - 1/2.
-      float wk[NV], wk1[NV], w2[NV], dlo[NV], hi[NV], flo[NV], u[NV], s[NV], wr[NV];
-      row(m0 - 2, u);
+      T wk[NV], wk1[NV], w2[NV], dlo[NV], hi[NV], flo[NV], u[NV], s[NV], wr[NV];
+      row(m0 - 2, u, std::false_type());
       recover<NDIM>(u, wk);
-      row(m0 - 1, u);
+      row(m0 - 1, u, std::false_type());
       recover<NDIM>(u, wk1);
-      row(m0, u);
+      row(m0, u, std::false_type());
       recover<NDIM>(u, w2);
       {
-        const float t = Base::geo(A, 1, m0 - 2).tipc;
+        const T t = Base::geo(A, 1, m0 - 2).tipc;
 #pragma unroll
         for (int v = 0; v < NV; ++v) dlo[v] = mul_rn(sub_rn(wk1[v], wk[v]), t);
-        const Geo<float> g = Base::geo(A, 1, m0 - 1);
-        slope(wk, wk1, w2, g, dlo, s, wr);
+        const Geo<T> g = Base::geo(A, 1, m0 - 1);
+        march_slope<NV, T>(wk, wk1, w2, g, dlo, s, wr);
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
           hi[v] = fma_rn(s[v], g.h, wk1[v]);
@@ -207,12 +264,12 @@ struct StripKernel {
           wk1[v] = w2[v];
         }
       }
-      row(m0 + 1, u);
+      row(m0 + 1, u, std::false_type());
       recover<NDIM>(u, w2);
       {
-        const Geo<float> g = Base::geo(A, 1, m0);
-        slope(wk, wk1, w2, g, dlo, s, wr);
-        face_flux<float, NDIM, NDIM - 1, SOLVER>(hi, wr, A.gamma, A.gm1, flo);
+        const Geo<T> g = Base::geo(A, 1, m0);
+        march_slope<NV, T>(wk, wk1, w2, g, dlo, s, wr);
+        face_flux<T, NDIM, 1, SOLVER>(hi, wr, A.gamma, A.gm1, flo);
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
           hi[v] = fma_rn(s[v], g.h, wk1[v]);
@@ -220,17 +277,17 @@ struct StripKernel {
           wk1[v] = w2[v];
         }
       }
-#pragma unroll 1
+#pragma unroll march_unroll<T>()
       for (int m = m0; m < m1; ++m) {
-        float L[NV], fhi[NV];
-        row(m + 2, u);  // lands during the x part
+        T L[NV], fhi[NV];
+        row(m + 2, u, std::true_type());  // lands during the x part
         x_part(A, wk, gx, iwx, L);
         recover<NDIM>(u, w2);
-        const Geo<float> g = Base::geo(A, 1, m + 1);
-        const float iwm = A.iw[1][m + 2];
-        slope(wk, wk1, w2, g, dlo, s, wr);
+        const Geo<T> g = A.geo[1][m + 3];  // of row m + 1
+        const T iwm = A.iw[1][m + 2];
+        march_slope<NV, T>(wk, wk1, w2, g, dlo, s, wr);
         // face m + 1/2 between the upper value of m and the lower of m + 1
-        face_flux<float, NDIM, NDIM - 1, SOLVER>(hi, wr, A.gamma, A.gm1, fhi);
+        face_flux<T, NDIM, 1, SOLVER>(hi, wr, A.gamma, A.gm1, fhi);
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
           L[v] = fma_rn(sub_rn(flo[v], fhi[v]), iwm, L[v]);
@@ -245,62 +302,318 @@ struct StripKernel {
         }
       }
     }
-    if (STAGE == 1 && own) {
-      if (A.want_totals) {
-        // the width as three floats: the pair alone would leave 2^-49 of it out
-        const dw dx = dw(A.wdh[0][col], A.wdl[0][col]);
-        const float dx3 = (float)((A.wd[0][col] - (double)dx.hi) - (double)dx.lo);
+    if (NDIM < 3 && STAGE == 1 && own) {
+      if (NDIM == 2 && A.want_totals) {
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-          dw c;
-          fast_two_sum(tcol[v].hi, tcol[v].lo, c.hi, c.lo);
-          const dw r = c * dx;
-          fast_two_sum(r.hi, fma_rn(c.hi, dx3, r.lo), tot[v].hi, tot[v].lo);
-        }
+        for (int v = 0; v < NV; ++v) tot[v] = share_of(tcol[v], A.wd[0][col]);
       }
-      speed_out = fmaxf(speed_out, speed_max);
+      speed_out = fmax(speed_out, speed_max);
     }
   }
 };
 
-// 2D single mesh: CTA (x, chunk) of NW warps, each its own strip.  64
-// registers, so that 32 warps stay resident on an SM.
-template <int SOLVER, int STAGE, int NW, bool WIDE>
-__global__ void __launch_bounds__(32 * NW, 32 / NW) hydro_strip_kernel(const StageArgs<float> A) {
-  using K = StripKernel<2, SOLVER, STAGE, WIDE>;
+// Fixed-order reduction of the warps' speeds and totals into CTA blk's partials.
+template <int NV, int NW, class T, class S>
+__device__ __forceinline__ void write_warp_partials(const StageArgs<T>& A, size_t blk, int warp, T speed,
+                                                    const S (&tot)[NV], double (&red)[NW][NV + 1]) {
+  double s;
+  if constexpr (std::is_same<T, float>::value) s = (double)warp_max(speed);
+  else s = warp_max((double)speed);
+  if ((threadIdx.x & 31) == 0) red[warp][0] = s;
+  if (A.want_totals) warp_totals<NV, S>(tot, &red[warp][1]);
+  else if ((threadIdx.x & 31) < NV) red[warp][1 + (threadIdx.x & 31)] = 0.0;
+  __syncthreads();
+  const int t = threadIdx.x;
+  if (t <= NV) {
+    double acc = red[0][t];
+    for (int w = 1; w < NW; ++w) acc = t == 0 ? fmax(acc, red[w][0]) : acc + red[w][t];
+    if (t == 0) A.part_speed[blk] = acc;
+    else A.part_tot[blk * NV + (t - 1)] = acc;
+  }
+}
+
+// Registers: FP32 2D 64 (32 warps per SM), 3D 80 (24 warps); double word 128
+// (16 warps).
+template <class T, int NDIM>
+constexpr int strip_warps() { return sizeof(T) == 8 ? 16 : NDIM == 3 ? 24 : 32; }
+
+// 2D single mesh: CTA (x, chunk) of NW warps, each its own strip.
+template <class T, int SOLVER, int STAGE, int NW, bool WIDE>
+__global__ void __launch_bounds__(32 * NW, (strip_warps<T, 2>() / NW)) hydro_strip_kernel(const StageArgs<T> A) {
+  using K = StripKernel<2, T, SOLVER, STAGE, WIDE>;
   constexpr int NV = 4;
   __shared__ double red[NW][NV + 1];
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
   const int x0 = (blockIdx.x * NW + warp) * STRIP_OWN;
   const int m0 = blockIdx.z * A.kchunk, m1 = min(A.n[1], m0 + A.kchunk);
-  float speed = 0.0f;
-  dw tot[NV];
+  T speed = T(0);
+  typename K::Tot tot[NV];
 #pragma unroll
-  for (int v = 0; v < NV; ++v) tot[v] = dw(0.0f, 0.0f);
+  for (int v = 0; v < NV; ++v) tot[v] = typename K::Tot(0.0);
   bool bad = false;
-  if (x0 < A.n[0]) K::strip(A, x0, m0, m1, speed, tot, bad);
+  if (x0 < A.n[0]) K::strip(A, x0, m0, m1, 0, speed, tot, bad);
   if (bad) atomicOr(A.status, STATUS_NONPHYS);
-  if (STAGE == 1) {
-    // fixed-order reduction into this CTA's partials
+  if (STAGE == 1)
+    write_warp_partials<NV, NW>(A, (size_t)blockIdx.z * gridDim.x + blockIdx.x, warp, speed, tot, red);
+}
+
+// 3D, x and y parts: one warp per (strip, plane, chunk of ychunk rows); strips
+// and planes are numbered along grid x, chunks along grid y.
+template <class T, int SOLVER, int STAGE, int NW, bool WIDE>
+__global__ void __launch_bounds__(32 * NW, (strip_warps<T, 3>() / NW))
+    hydro_strip_xy_kernel(const StageArgs<T> A, int strips, int ychunk) {
+  using K = StripKernel<3, T, SOLVER, STAGE, WIDE>;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+  const int id = blockIdx.x * NW + warp;
+  const int k = id / strips;
+  if (k >= A.n[2]) return;
+  const int x0 = (id - k * strips) * STRIP_OWN;
+  const int m0 = blockIdx.y * ychunk, m1 = min(A.n[1], m0 + ychunk);
+  T speed = T(0);
+  typename K::Tot tot[5];
+  bool bad = false;
+  K::strip(A, x0, m0, m1, k, speed, tot, bad);
+}
+
+// 3D, z part and epilogue: one thread per (x, y) column and chunk of planes.
+//
+// ASYNC (FP32, planes of a multiple of 4 cells): every warp keeps its own ring
+// of SLOTS planes in shared memory, filled ahead of the march by 16-byte
+// cp.async copies (a lane moves a quarter of a row of a quarter of the arrays:
+// 3 or 4 copies a plane for U, K and the strips' L), so that a plane's loads
+// have 3 or 4 planes of arithmetic to land in, and the plane's second use (U and
+// K of the stage combine) reads shared memory again.  Only __syncwarp separates
+// filling from reading.
+template <class T, int SOLVER, int STAGE, bool WIDE, bool ASYNC>
+struct ZMarch {
+  static_assert(!ASYNC || (std::is_same<T, float>::value && !WIDE), "the ring moves FP32 rows");
+  using Base = StageKernel<3, T, SOLVER, STAGE, 32, 1, false>;
+  using Acc = CellAccess<T, WIDE>;
+  using Off = typename Acc::Off;
+  using Tot = typename TotalSum<T>::type;
+  static constexpr int NV = 5;
+  static constexpr int NARR = STAGE == 1 ? 10 : 15;        // U, (K,) L
+  static constexpr int SLOTS = STAGE == 1 ? 7 : 6;
+  static constexpr int COPIES = (NARR * 8 + 31) / 32;      // 16-byte copies a lane and plane
+  struct Ring {
+    float a[SLOTS][NARR][32];
+  };
+  static constexpr size_t SMEM = ASYNC ? 4 * sizeof(Ring) : 0;  // four warps a CTA
+
+  static __device__ __forceinline__ void march(const StageArgs<T>& A, Ring* ring, unsigned j, int m0, int m1,
+                                               T& speed_max, Tot (&tot)[NV], bool& bad) {
     const int lane = threadIdx.x & 31;
-    const float s = warp_max(speed);
-    if (lane == 0) red[warp][0] = (double)s;
-    if (A.want_totals) {
-      const dw t = warp_sum4(tot);
-      if ((lane & 7) == 0) red[warp][1 + (lane >> 3)] = (double)t;
-    } else if ((lane & 7) == 0) {
-      red[warp][1 + (lane >> 3)] = 0.0;
+    const int nx = A.n[0], ny = A.n[1], nz = A.n[2];
+    const unsigned plane = (unsigned)nx * (unsigned)ny;
+    const size_t vs = (size_t)plane * nz;
+    const bool own = j < plane;
+    const unsigned jc = own ? j : plane - 1;
+    const int x = (int)(jc % (unsigned)nx), y = (int)(jc / (unsigned)nx);
+    const T dt = STAGE == 2 ? (T)(*A.dt) : T(0);
+    const T iwx = A.iw[0][x + 2], iwy = A.iw[1][y + 2];
+    ColumnSum<T> tcol[NV];
+
+    // ring: source (array, quarter row) and destination of the lane's copies
+    const char* src[ASYNC ? COPIES : 1];
+    unsigned dst = 0;
+    bool quarter = false;  // the lane's quarter rows lie inside the mesh
+    if constexpr (ASYNC) {
+      const unsigned j0 = j - lane;
+      quarter = j0 + 4u * (lane & 7) < plane;
+      dst = (unsigned)__cvta_generic_to_shared(&ring->a[0][0][0]) + 16u * lane;
+#pragma unroll
+      for (int i = 0; i < COPIES; ++i) {
+        const int idx = i * 32 + lane, arr = idx >> 3;
+        // columns past the mesh repeat its last four of U and K (L: left as it is)
+        const unsigned col = min(j0 + 4u * (lane & 7), plane - 4u);
+        const T* base = arr < 5 ? A.un + arr * vs
+                        : STAGE == 2 && arr < 10 ? A.k1 + (arr - 5) * vs
+                                                 : A.out + (size_t)min(arr - (NARR - 5), 4) * vs;
+        src[i] = reinterpret_cast<const char*>(base + col);
+      }
     }
-    __syncthreads();
-    const int t = threadIdx.x;
-    const size_t blk = (size_t)blockIdx.z * gridDim.x + blockIdx.x;
-    if (t <= NV) {
-      double acc = red[0][t];
-      for (int w = 1; w < NW; ++w) acc = t == 0 ? fmax(acc, red[w][0]) : acc + red[w][t];
-      if (t == 0) A.part_speed[blk] = acc;
-      else A.part_tot[blk * NV + (t - 1)] = acc;
+    // Fill slot `slot` with plane m (boundary-mapped; L only for the chunk's own
+    // planes); planes past the march leave an empty group.
+    auto fill = [&](int m, int slot) {
+      if constexpr (ASYNC) {
+        if (m < m1 + 2) {
+          bool fm;
+          int sm = m;
+          if (m < 0 || m >= nz) sm = bc_map(m, nz, A.bc_lo[2], A.bc_hi[2], fm);
+          const size_t off = (size_t)sm * plane * sizeof(T);
+          const bool inner = m >= m0 && m < m1 && quarter;
+#pragma unroll
+          for (int i = 0; i < COPIES; ++i) {
+            const int arr = (i * 32 + lane) >> 3;
+            if (arr < NARR - 5 || (inner && arr < NARR))
+              asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + slot * (unsigned)sizeof(ring->a[0]) +
+                                                                            i * 512u),
+                           "l"(src[i] + off)
+                           : "memory");
+          }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+      }
+    };
+    auto row = [&](int m, int slot, T (&u)[NV], auto ahead) {
+      bool fm = false;
+      int sm = m;
+      if (!decltype(ahead)::value || m >= nz) sm = bc_map(m, nz, A.bc_lo[2], A.bc_hi[2], fm);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        if constexpr (ASYNC) {
+          u[v] = ring->a[slot][v][lane];
+          if (STAGE == 2) u[v] = fma_rn(dt, ring->a[slot][5 + v][lane], u[v]);
+        } else {
+          const Off c = (Off)sm * (Off)plane + (Off)jc;
+          u[v] = Acc::at(A.un + v * vs, c);
+          if (STAGE == 2) u[v] = fma_rn(dt, Acc::at(A.k1 + v * vs, c), u[v]);
+        }
+      }
+      if (STAGE == 1 && A.want_totals && m >= m0 && m < m1) {
+        const T hi = A.wdh[2][m], lo = A.wdl[2][m];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) tcol[v].add_product(u[v], hi, lo);
+      }
+      if (fm) u[3] = -u[3];
+    };
+    T wk[NV], wk1[NV], w2[NV], dlo[NV], hi[NV], flo[NV], u[NV], s[NV], wr[NV];
+    // the first SLOTS planes; the four below are consumed before the march
+    if constexpr (ASYNC) {
+      for (int i = 0; i < SLOTS; ++i) fill(m0 - 2 + i, i);
+      asm volatile("cp.async.wait_group %0;" ::"n"(SLOTS - 4) : "memory");
+      __syncwarp();
+    }
+    row(m0 - 2, 0, u, std::false_type());
+    recover<3>(u, wk);
+    row(m0 - 1, 1, u, std::false_type());
+    recover<3>(u, wk1);
+    row(m0, 2, u, std::false_type());
+    recover<3>(u, w2);
+    {
+      const T t = Base::geo(A, 2, m0 - 2).tipc;
+#pragma unroll
+      for (int v = 0; v < NV; ++v) dlo[v] = mul_rn(sub_rn(wk1[v], wk[v]), t);
+      const Geo<T> g = Base::geo(A, 2, m0 - 1);
+      march_slope<NV, T>(wk, wk1, w2, g, dlo, s, wr);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        hi[v] = fma_rn(s[v], g.h, wk1[v]);
+        wk[v] = wk1[v];
+        wk1[v] = w2[v];
+      }
+    }
+    row(m0 + 1, 3, u, std::false_type());
+    recover<3>(u, w2);
+    {
+      const Geo<T> g = Base::geo(A, 2, m0);
+      march_slope<NV, T>(wk, wk1, w2, g, dlo, s, wr);
+      face_flux<T, 3, 2, SOLVER>(hi, wr, A.gamma, A.gm1, flo);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        hi[v] = fma_rn(s[v], g.h, wk1[v]);
+        wk[v] = wk1[v];
+        wk1[v] = w2[v];
+      }
+    }
+    if constexpr (ASYNC) {
+      __syncwarp();
+      fill(m0 - 2 + SLOTS, 0);
+    }
+    // slots of planes m - 1 (free in iteration m), m, m + 1 and m + 2
+    int slf = 1, sl0 = 2, sl1 = 3, sl2 = 4;
+#pragma unroll march_unroll<T>()
+    for (int m = m0; m < m1; ++m) {
+      const Off c = (Off)m * (Off)plane + (Off)jc;
+      T L[NV], fhi[NV];
+      if constexpr (ASYNC) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(SLOTS - 4) : "memory");  // plane m + 2 has landed
+        __syncwarp();  // for every lane, and every lane is done with plane m - 1
+        fill(m - 1 + SLOTS, slf);
+      }
+      row(m + 2, sl2, u, std::true_type());
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {  // the strips' x and y parts
+        if constexpr (ASYNC) L[v] = ring->a[sl0][NARR - 5 + v][lane];
+        else L[v] = own ? A.out[v * vs + c] : T(0);
+      }
+      recover<3>(u, w2);
+      const Geo<T> g = A.geo[2][m + 3];  // of plane m + 1
+      const T iwm = A.iw[2][m + 2];
+      march_slope<NV, T>(wk, wk1, w2, g, dlo, s, wr);
+      face_flux<T, 3, 2, SOLVER>(hi, wr, A.gamma, A.gm1, fhi);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        L[v] = fma_rn(sub_rn(flo[v], fhi[v]), iwm, L[v]);
+        flo[v] = fhi[v];
+      }
+      if (A.has_source) Base::add_source(A, wk, L);
+      bad |= own && Base::nonphysical(wk, A.gm1);
+      if (STAGE == 1) {
+        const T cs = sound_speed(A.gamma, mul_rn(A.gm1, wk[4]), wk[0]);
+        T sp = mul_rn(add_rn(fabs(wk[1]), cs), iwx);
+        sp = fmax(sp, mul_rn(add_rn(fabs(wk[2]), cs), iwy));
+        sp = fmax(sp, mul_rn(add_rn(fabs(wk[3]), cs), iwm));
+        speed_max = fmax(speed_max, sp);
+      } else {
+        const T hdt = half_of(dt);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          T u0, k;
+          if constexpr (ASYNC) {
+            u0 = ring->a[sl0][v][lane];
+            k = ring->a[sl0][5 + v][lane];
+          } else {
+            u0 = Acc::at(A.un + v * vs, c);
+            k = Acc::at(A.k1 + v * vs, c);
+          }
+          L[v] = fma_rn(hdt, add_rn(k, L[v]), u0);
+        }
+      }
+      if (own) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) A.out[v * vs + c] = L[v];
+      }
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        hi[v] = fma_rn(s[v], g.h, wk1[v]);
+        wk[v] = wk1[v];
+        wk1[v] = w2[v];
+      }
+      slf = sl0;
+      sl0 = sl1;
+      sl1 = sl2;
+      sl2 = sl2 + 1 == SLOTS ? 0 : sl2 + 1;
+    }
+    if constexpr (ASYNC) asm volatile("cp.async.wait_group 0;" ::: "memory");
+    if (STAGE == 1 && A.want_totals && own) {
+      const double area = A.wd[0][x] * A.wd[1][y];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) tot[v] = share_of(tcol[v], area);
     }
   }
+};
+
+template <class T, int SOLVER, int STAGE, bool WIDE, bool ASYNC>
+__global__ void __launch_bounds__(128, (sizeof(T) == 8 ? 4 : ASYNC && STAGE == 2 ? 4 : 6))
+    hydro_march_z_kernel(const StageArgs<T> A) {
+  using K = ZMarch<T, SOLVER, STAGE, WIDE, ASYNC>;
+  constexpr int NV = 5, NW = 4;
+  extern __shared__ __align__(16) unsigned char smem_z[];
+  __shared__ double red[NW][NV + 1];
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+  // chunks in descending order: the strips' last planes are still in L2
+  const int chunk = gridDim.z - 1 - blockIdx.z;
+  const int m0 = chunk * A.kchunk, m1 = min(A.n[2], m0 + A.kchunk);
+  T speed = T(0);
+  typename K::Tot tot[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) tot[v] = typename K::Tot(0.0);
+  bool bad = false;
+  K::march(A, reinterpret_cast<typename K::Ring*>(smem_z) + warp, blockIdx.x * 128u + threadIdx.x, m0, m1, speed, tot,
+           bad);
+  if (bad) atomicOr(A.status, STATUS_NONPHYS);
+  if (STAGE == 1) write_warp_partials<NV, NW>(A, (size_t)chunk * gridDim.x + blockIdx.x, warp, speed, tot, red);
 }
 
 }  // namespace gh

@@ -9,7 +9,7 @@ import pytest
 import oracle as O
 from paper_1207_3392_gb300 import hydro as H
 from paper_1207_3392_gb300 import problems as P
-from parity_util import TOL_FP32, check, oracle_run
+from parity_util import TOL_FP32, TOL_FP64, check, oracle_run
 
 pytestmark = pytest.mark.gpu
 
@@ -90,3 +90,47 @@ def test_mesh_beyond_2_30_cells():
         np.testing.assert_array_equal(rows[:, k], rows[:, 0])
     Uo = O.step(g, U1.astype(np.float64), dt)
     check(rows[[0, 1, 3], 0].astype(np.float64), Uo, 1, TOL_FP32, "wide mesh")
+
+
+@pytest.mark.parametrize("precision,tol,tile", [(H.FP32_MIXED, TOL_FP32, 14), (H.FP64_DW, TOL_FP64, 4)])
+@pytest.mark.parametrize("bc", [P.PERIODIC, P.REFLECT, P.OUTFLOW])
+@pytest.mark.parametrize("n", [(2, 2, 2), (3, 5, 3), (27, 4, 5), (28, 7, 4), (29, 3, 9), (57, 9, 11), (226, 3, 14)])
+def test_split_stages_match_the_oracle_and_the_tiles(n, bc, precision, tol, tile):
+    """3D on independent warps (a launch for x and y, one for z): planes of 4 k
+    cells (the shared-memory ring) and of other counts, chunks of planes and
+    their remainders; bitwise the state of tile 0."""
+    pr = P.random_blocks(3, n, seed=60 + n[0], bc=bc).with_(grad_phi=(0.2, -0.3, 0.1))
+    for solver in (H.HLL, H.HLLC):
+        Uo, to = oracle_run(pr, solver=solver, steps=2)
+        ref = None
+        for t, kc in ((tile, 0), (tile, 1), (tile, 3), (tile, 8), (0, 0)):
+            h = H.Hydro.from_problem(pr, precision=precision, solver=solver)
+            h.set_tile(t, kc)
+            time = h.advance(2, pr.cfl)
+            U = h.get_conserved(precision=H.FP64)
+            tot = h.step_totals()
+            h.close()
+            if ref is None:
+                ref, ref_tot = U, tot
+                assert time == pytest.approx(to, rel=1e-5 if tol == TOL_FP32 else 1e-10)
+                check(U, Uo, 3, tol, f"{n} bc={bc} solver={solver}")
+            np.testing.assert_array_equal(U, ref, err_msg=f"tile {t} kchunk {kc}")
+            np.testing.assert_allclose(tot, ref_tot, rtol=1e-12, atol=1e-12 * np.max(np.abs(ref_tot)))
+
+
+@pytest.mark.parametrize("n", [(2, 2), (27, 5), (29, 33), (57, 38)])
+def test_double_word_strips_match_the_oracle_and_the_tiles(n):
+    for bc in (P.PERIODIC, P.REFLECT, P.OUTFLOW):
+        pr = P.random_blocks(2, n, seed=80 + n[0], bc=bc)
+        Uo, _ = oracle_run(pr, steps=3)
+        ref = None
+        for t, kc in ((1, 0), (1, 1), (1, 5), (0, 0)):
+            h = H.Hydro.from_problem(pr, precision=H.FP64_DW)
+            h.set_tile(t, kc)
+            h.advance(3, pr.cfl)
+            U = h.get_conserved()
+            h.close()
+            if ref is None:
+                ref = U
+                check(U, Uo, 2, TOL_FP64, f"dw {n} bc={bc}")
+            np.testing.assert_array_equal(U, ref, err_msg=f"tile {t} kchunk {kc}")
