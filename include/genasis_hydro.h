@@ -197,11 +197,12 @@ int genasis_hydro_autotune(genasis_hydro_t h, int trial_steps, const char *cache
 #define GENASIS_OPT_STEP_TOTALS 1
 /* GENASIS_OPT_ONE_LAUNCH: 1 (default) runs genasis_hydro_step and
  * genasis_hydro_advance of a 1D FP64 or FP32-mixed HLL/HLLC mesh of at most
- * 4088 cells as one cooperative kernel launch (one CTA per tile, bounded grid
- * barriers between the phases) for all the steps of the call
- * (the same tile arithmetic and dt fold as the three launches per step, so
+ * 4088 cells as one kernel launch for all the steps of the call, on one
+ * thread-block cluster that keeps the state on chip (or, where the device
+ * cannot place it, as a cooperative launch with bounded grid barriers)
+ * (the same cell and face arithmetic and dt fold as the three launches per step, so
  * bitwise the same states, dt and time; the step totals sum the cells in
- * tiles of another width and agree to rounding); 0 keeps three launches per
+ * another grouping and agree to rounding); 0 keeps three launches per
  * step.  With a network attached (genasis_hydro_set_flux_mlp) the option is
  * passed on to its corrected scheme (genasis_learned_set_option), as is
  * GENASIS_OPT_MLP_TCGEN05 (defined with genasis_learned_set_option), which

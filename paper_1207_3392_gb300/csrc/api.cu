@@ -360,8 +360,9 @@ template int launch_stage<dw>(genasis_hydro*, int, cudaStream_t);
 
 namespace {
 
-// Small 1D meshes: every step of a call in one cooperative launch of one CTA
-// per tile (kern_1d_advance.cu): 32 threads (31 cells) per CTA in FP64, so
+// Small 1D meshes: every step of a call in one launch, on one thread-block
+// cluster (kern_1d_cluster.cu) or, where the device cannot place it, as a
+// cooperative launch of one CTA per tile (kern_1d_advance.cu): 32 threads (31 cells) per CTA in FP64, so
 // the FP64 work spreads over as many SMs as possible (an SM retires ~2 FP64
 // operations per clock), 256 (255 cells) in FP32.
 constexpr int ADV1D_MAX_CELLS = 4088;
@@ -372,8 +373,41 @@ bool use_1d_advance(const genasis_hydro* h) {
          (h->solver == GENASIS_HLL || h->solver == GENASIS_HLLC) && h->n[0] <= ADV1D_MAX_CELLS;
 }
 
+// On one cluster of CTAs where the device can place it (faster at every size,
+// see kern_1d_cluster.cu), else on a cooperative grid.
+bool use_1d_cluster(genasis_hydro* h) {
+  if (h->cluster_state == 0)
+    h->cluster_state = cluster_1d_plan(h->prec == GENASIS_FP64, h->solver, h->n[0], &h->cluster) ? 1 : -1;
+  return h->cluster_state == 1;
+}
+
+template <class T>
+int launch_1d_cluster_t(genasis_hydro* h, int nsteps, int mode, double cfl, double fixed_dt, double t_end) {
+  StageArgs<T> A = stage_args<T>(h, 1);
+  FinalizeArgs F;
+  memset(&F, 0, sizeof(F));
+  F.part_tot = h->want_totals ? h->part_tot : nullptr;
+  F.nv = h->nv;
+  F.mode = mode;
+  F.cfl = cfl;
+  F.fixed_dt = fixed_dt;
+  F.t_end = t_end;
+  F.scal = h->scal;
+  F.status = h->status;
+  const T* uin = (const T*)h->U[h->cur];
+  T* uout = (T*)h->U[h->cur ^ (nsteps & 1)];
+  void* args[] = {&A, &F, &nsteps, &uin, &uout, &h->cluster.per};
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  cluster_1d_config(h->cluster, h->stream, &cfg, at);
+  GH_CK(cudaLaunchKernelExC(&cfg, h->cluster.fn, args));
+  h->cur ^= nsteps & 1;
+  return GENASIS_OK;
+}
+
 template <class T>
 int launch_1d_advance_t(genasis_hydro* h, int nsteps, int mode, double cfl, double fixed_dt, double t_end) {
+  if (use_1d_cluster(h)) return launch_1d_cluster_t<T>(h, nsteps, mode, cfl, fixed_dt, t_end);
   const int tx = sizeof(T) == 8 ? 32 : 256;
   size_t smem = 0;
   const void* fn = advance_1d_kernel(sizeof(T) == 8, h->solver, tx, &smem);

@@ -48,6 +48,15 @@ int tile_count_1d();
 // kernel for (precision, solver) on tx threads and its dynamic shared memory,
 // or nullptr if not compiled.
 const void* advance_1d_kernel(bool fp64, int solver, int tx, size_t* smem);
+// The same on one thread-block cluster (kern_1d_cluster.cu): the launch for n
+// cells; false if there is none on this device.
+struct Cluster1D {
+  const void* fn = nullptr;
+  int per = 0, ranks = 0, threads = 0;
+  size_t smem = 0;
+};
+bool cluster_1d_plan(bool fp64, int solver, int n, Cluster1D* out);
+void cluster_1d_config(const Cluster1D& c, cudaStream_t st, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at);
 int tile_count_2d();
 int tile_count_3d_f32();
 int tile_count_3d_f64();
