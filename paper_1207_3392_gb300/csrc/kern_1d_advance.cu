@@ -41,9 +41,8 @@ __global__ void __launch_bounds__(TX)
   constexpr int NV = 3;
   const int bx = blockIdx.x;
   const unsigned nb = gridDim.x;
-  unsigned my_gen = 0;
+  unsigned passed = 0;  // grid barriers
   bool failed = false;
-  if (threadIdx.x == 0) my_gen = atomicAdd(bar + 1, 0u);  // the generation at launch (no CTA can move it yet)
   // the time, kept by every CTA (CTA 0 also stores it): read before any CTA
   // of this launch writes it
   double t = __ldcg(F.scal + SCAL_T);
@@ -60,7 +59,7 @@ __global__ void __launch_bounds__(TX)
       if (bad) atomicOr(A.status, STATUS_NONPHYS);
       K1::write_partials(a1, S1, bx, speed, tot);
     }
-    if (!grid_barrier(bar, bar + 1, nb, my_gen, A.status, failed)) return;
+    if (!grid_barrier(bar, nb, passed, A.status, failed)) return;
     // every CTA folds the partials the same way and takes the same dt; CTA 0
     // also stores dt, t and the totals in the scalar block
     if (threadIdx.x < 32) {
@@ -82,7 +81,7 @@ __global__ void __launch_bounds__(TX)
       K2::tile(a2, S2, bx, 0, 0, speed, tot, bad);
       if (bad) atomicOr(A.status, STATUS_NONPHYS);
     }
-    if (!grid_barrier(bar, bar + 1, nb, my_gen, A.status, failed)) return;
+    if (!grid_barrier(bar, nb, passed, A.status, failed)) return;
     T* tmp = cur;
     cur = nxt;
     nxt = tmp;

@@ -96,9 +96,8 @@ __device__ __forceinline__ void lf_advance_body(const LfAdvanceArgs& P, typename
   constexpr int XSTRIDE = TC ? 8 : 1;
   unsigned phase = 0;    // of the group's mbarrier
   bool mlp_ok = true;    // the group's tensor-core waits have all completed
-  unsigned my_gen = 0;
+  unsigned passed = 0;  // grid barriers
   bool failed = false;
-  if (tid == 0) my_gen = atomicAdd(bar + 1, 0u);  // the generation at launch (no CTA can move it yet)
   // the time, kept by every CTA (CTA 0 also stores it): read before any CTA
   // of this launch writes it
   double t = __ldcg(P.Fa.scal + SCAL_T);
@@ -123,7 +122,7 @@ __device__ __forceinline__ void lf_advance_body(const LfAdvanceArgs& P, typename
         atomicMax(speed_slot + (s & 1), (unsigned long long)__double_as_longlong(acc));
       }
     }
-    if (!grid_barrier(bar, bar + 1, nb, my_gen, P.status, failed)) return;
+    if (!grid_barrier(bar, nb, passed, P.status, failed)) return;
     if (warp == 0) {
       // the largest speed of the step; the other slot is free again (its
       // last reads were before this barrier, its next writes come after the
@@ -192,7 +191,7 @@ __device__ __forceinline__ void lf_advance_body(const LfAdvanceArgs& P, typename
           __syncwarp();  // the rows are read before the next tile's features
         }
       }
-      if (!grid_barrier(bar, bar + 1, nb, my_gen, P.status, failed)) return;
+      if (!grid_barrier(bar, nb, passed, P.status, failed)) return;
       unsigned* ap = P.sync + 2 * stage;  // this stage's all-plain flags
       if (bx == 0 && tid == 0) {
         unsigned* other = P.sync + 2 * (3 - stage);
@@ -220,7 +219,7 @@ __device__ __forceinline__ void lf_advance_body(const LfAdvanceArgs& P, typename
       A.R = nullptr;
       if (corr && P.fct) {
         for (long long c = first + tid; c < ncell; c += stride) lf_fct_cell<true>(A, c, dt, P.Rfct);
-        if (!grid_barrier(bar, bar + 1, nb, my_gen, P.status, failed)) return;
+        if (!grid_barrier(bar, nb, passed, P.status, failed)) return;
         A.R = P.Rfct;
       }
       // the corrected pass, then only when some cell failed the widening
@@ -230,7 +229,7 @@ __device__ __forceinline__ void lf_advance_body(const LfAdvanceArgs& P, typename
 #pragma unroll 1
       for (int pass = 0;;) {
         for (long long c = first + tid; c < ncell; c += stride) lf_update_cell<true>(A, c, dt);
-        if (!grid_barrier(bar, bar + 1, nb, my_gen, P.status, failed)) return;
+        if (!grid_barrier(bar, nb, passed, P.status, failed)) return;
         if (!corr || pass < 0) break;
         if (pass == 0 && !__syncthreads_or(tid == 0 && __ldcg(ap + 1) != 0u)) break;
         if (pass == LFA_PASSES) {

@@ -19,9 +19,9 @@ namespace {
 
 __global__ void barrier_wait_probe(unsigned* words, unsigned* status) {
   if (blockIdx.x != 0) return;  // the second CTA never arrives
-  unsigned my_gen = 0;
+  unsigned passed = 0;  // grid barriers
   bool failed = false;
-  grid_barrier(words, words + 1, 2u, my_gen, status, failed);
+  grid_barrier(words, 2u, passed, status, failed);
 }
 
 __global__ void mbarrier_wait_probe(unsigned* status) {
@@ -47,7 +47,7 @@ extern "C" int genasis_check_bounded_waits(unsigned* status, double* seconds) {
   for (int i = 0; i < 3 && err == cudaSuccess; ++i) err = cudaEventCreate(&e[i]);
   if (err == cudaSuccess) err = cudaMemset(d, 0, 4 * sizeof(unsigned));
   if (err == cudaSuccess) {
-    // d[0..1]: barrier count and generation; d[2], d[3]: the two status words
+    // d[0]: barrier count; d[2], d[3]: the two status words
     cudaEventRecord(e[0]);
     barrier_wait_probe<<<2, 32>>>(d, d + 2);
     cudaEventRecord(e[1]);
