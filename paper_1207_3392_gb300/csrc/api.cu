@@ -223,6 +223,22 @@ int configure(genasis_hydro* h, int tile, int kchunk_req) {
       const long strips = (h->n[0] + 27) / 28;
       const long rows = (strips * nm + 16L * h->num_sms - 1) / (16L * h->num_sms);
       kchunk = (int)(rows < least ? least : rows > 32 ? 32 : rows);
+    } else if (h->prec == GENASIS_FP64) {
+      // FP64 is bound by its pipe on every SM: the chunk whose CTAs per SM, each
+      // its planes and half a plane of warm-up, come to the least
+      // (128^3: 19 planes in 448 CTAs, 2.95 per SM, 1.86 ms a stage; 13 in 640,
+      // 4.2 per SM, 2.03; 16 in 512 2.10.  A step of 32^3: one plane 0.11 ms, 8
+      // planes 0.66)
+      long best = -1;
+      for (int gzt = 1; gzt <= nm && gzt <= 65535; ++gzt) {
+        const int kc = (nm + gzt - 1) / gzt;
+        const long ctas = (long)gx * gy * ((nm + kc - 1) / kc);
+        const long cost = (ctas + h->num_sms - 1) / h->num_sms * (2L * kc + 1);
+        if (best < 0 || cost < best) {
+          best = cost;
+          kchunk = kc;
+        }
+      }
     } else {
       // about four CTAs per SM per stage, at least 8 planes per CTA
       const long target = 4L * h->num_sms;

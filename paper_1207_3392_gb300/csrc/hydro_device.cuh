@@ -104,7 +104,25 @@ __device__ __forceinline__ double max0(double a, double b) {
   return (ka < kb ? kb : ka) > 0 ? m : 0.0;
 }
 
-// x == 0 and x >= 0; FP64 tests run on the integer pipe.
+// max(a, b) of a CFL speed a >= 0 that ignores a NaN b, x > 0, |x| < infinity,
+// x == 0 and x >= 0; FP64: on the integer pipe.
+template <class T>
+__device__ __forceinline__ T max_speed(T a, T b) { return fmax(a, b); }
+__device__ __forceinline__ double max_speed(double a, double b) {
+  const long long ka = __double_as_longlong(a), kb = __double_as_longlong(b);
+  return kb > ka && kb <= 0x7ff0000000000000ll ? b : a;
+}
+template <class T>
+__device__ __forceinline__ bool positive(T x) { return x > T(0); }
+__device__ __forceinline__ bool positive(double x) {  // false for NaN, whose bits lie above infinity's
+  const long long b = __double_as_longlong(x);
+  return b > 0 && b <= 0x7ff0000000000000ll;
+}
+template <class T>
+__device__ __forceinline__ bool finite(T x) { return fabs(x) < T(INFINITY); }
+__device__ __forceinline__ bool finite(double x) {
+  return (__double_as_longlong(x) & 0x7fffffffffffffffll) < 0x7ff0000000000000ll;
+}
 __device__ __forceinline__ bool is_zero(float x) { return x == 0.0f; }
 __device__ __forceinline__ bool is_zero(dw x) { return x.hi == 0.0f; }
 __device__ __forceinline__ bool is_zero(double x) { return ((unsigned long long)__double_as_longlong(x) << 1) == 0; }
@@ -130,7 +148,11 @@ __device__ __forceinline__ dw mul_rn(dw a, dw b) { return a * b; }
 __device__ __forceinline__ dw fma_rn(dw a, dw b, dw c) { return fma(a, b, c); }
 // a / 2 (exact) and c - a / 2
 __device__ __forceinline__ float half_of(float a) { return __fmul_rn(0.5f, a); }
-__device__ __forceinline__ double half_of(double a) { return __dmul_rn(0.5, a); }
+__device__ __forceinline__ double half_of(double a) {  // normal numbers: one off the exponent, on the integer pipe
+  const long long b = __double_as_longlong(a);
+  const unsigned ex = (unsigned)((unsigned long long)b >> 52) & 0x7ffu;
+  return ex - 2u < 0x7fdu ? __longlong_as_double(b - (1ll << 52)) : __dmul_rn(0.5, a);
+}
 __device__ __forceinline__ dw half_of(dw a) { return dw(__fmul_rn(0.5f, a.hi), __fmul_rn(0.5f, a.lo)); }
 __device__ __forceinline__ float sub_half(float c, float a) { return __fmaf_rn(-0.5f, a, c); }
 __device__ __forceinline__ double sub_half(double c, double a) { return __fma_rn(-0.5, a, c); }
