@@ -66,10 +66,10 @@ int stage_tile_count(int ndim, int prec) { return tile_count(ndim, prec); }
 // double word (tiles 1 and 4).  A strip owns 28 columns, a tile 32: with 29 to
 // 32 columns along x in 3D two half-empty strips lose to one tile (29 x 160 x
 // 160: 96 to 99 us a step against 88 in FP32, 562 against 499 in double word).
-int stage_tile_default(int ndim, int prec, int solver, int nx) {
+int stage_tile_default(int ndim, int prec, int nx) {
   if (ndim == 3 && nx > 28 && nx <= 32) return 0;
   if (prec == GENASIS_FP64_DW) return ndim == 3 ? 4 : ndim == 2 ? 1 : 0;
-  if (prec == GENASIS_FP32_MIXED && ndim == 3 && solver != GENASIS_HLLC_SWITCH) return 14;
+  if (prec == GENASIS_FP32_MIXED && ndim == 3) return 14;
   return 0;
 }
 
@@ -705,7 +705,7 @@ int genasis_hydro_create(const genasis_hydro_desc* d, genasis_hydro_t* out) {
   rc = h->prec == GENASIS_FP64         ? upload_geometry<double>(h, d)
        : h->prec == GENASIS_FP32_MIXED ? upload_geometry<float>(h, d)
                                        : upload_geometry<dw>(h, d);
-  if (!rc) rc = configure(h, stage_tile_default(h->ndim, h->prec, h->solver, h->n[0]), 0);
+  if (!rc) rc = configure(h, stage_tile_default(h->ndim, h->prec, h->n[0]), 0);
   if (rc) {
     free_all(h);
     return rc;

@@ -51,6 +51,13 @@ inline void fill_strip(StageVariant* out) {
   out->strips = 1;
 }
 template <class T, int NW>
+inline bool pick_strip_switch(int stage, StageVariant* out) {
+  if (stage == 1) fill_strip<T, SOLVER_HLLC_SW, 1, NW>(out);
+  else if (stage == 2) fill_strip<T, SOLVER_HLLC_SW, 2, NW>(out);
+  else return false;
+  return true;
+}
+template <class T, int NW>
 inline bool pick_strip(int solver, int stage, StageVariant* out) {
   if (solver == SOLVER_HLL && stage == 1) fill_strip<T, SOLVER_HLL, 1, NW>(out);
   else if (solver == SOLVER_HLL && stage == 2) fill_strip<T, SOLVER_HLL, 2, NW>(out);
@@ -75,6 +82,13 @@ inline void fill_split(StageVariant* out) {
   out->tx = 128;
   out->ty = 1;
   out->threads = 128;
+}
+template <class T>
+inline bool pick_split_switch(int stage, StageVariant* out) {
+  if (stage == 1) fill_split<T, SOLVER_HLLC_SW, 1>(out);
+  else if (stage == 2) fill_split<T, SOLVER_HLLC_SW, 2>(out);
+  else return false;
+  return true;
 }
 template <class T>
 inline bool pick_split(int solver, int stage, StageVariant* out) {

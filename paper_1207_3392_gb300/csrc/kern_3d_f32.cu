@@ -20,6 +20,7 @@ bool stage_variant_3d_f32(int solver, int stage, int tile, StageVariant* out) {
   if (solver == SOLVER_HLLC_SW) {
     if (tile == 0) return pick_switch<3, float, 32, 8, 3>(stage, out);
     if (tile == 8) return pick_switch<3, float, 32, 7, 4>(stage, out);
+    if (tile == 14) return stage_variant_3d_f32_split(solver, stage, out);
     return false;
   }
   switch (tile) {

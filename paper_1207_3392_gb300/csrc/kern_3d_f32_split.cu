@@ -3,6 +3,9 @@
 
 namespace gh {
 
-bool stage_variant_3d_f32_split(int solver, int stage, StageVariant* out) { return pick_split<float>(solver, stage, out); }
+bool stage_variant_3d_f32_split(int solver, int stage, StageVariant* out) {
+  if (solver == SOLVER_HLLC_SW) return pick_split_switch<float>(stage, out);
+  return pick_split<float>(solver, stage, out);
+}
 
 }  // namespace gh

@@ -27,7 +27,8 @@
 // and ZMarch 440 and 324 at 79% and 66%: 493 and 490 us together.  The price is
 // memory traffic, 100 and 140 algorithmic bytes a cell for 40 and 60, half of
 // what the launches' times could move.  Double word at 128^3: 558 and 549 ->
-// 464 and 530 us.
+// 464 and 530 us.  With the shock switch (bits read beside U, HLLC and HLL both
+// compiled at every face), 203 x 91 x 61: 176 -> 148 us a step, 24^3 61 -> 39.
 #pragma once
 
 #include <type_traits>
@@ -137,12 +138,12 @@ struct StripKernel {
   using Off = typename Acc::Off;
   using Tot = typename TotalSum<T>::type;
   static constexpr int NV = NDIM + 2;
-  static_assert(!Base::SW, "the switch runs on the row tiles");
+  static constexpr bool SW = Base::SW;  // per-face HLLC/HLL choice from shock bits
 
   // minus the x part of the flux divergence of the lanes' cells of one row
   // (valid on the owned lanes), from W of the row
   static __device__ __forceinline__ void x_part(const StageArgs<T>& A, const T (&w)[NV], const Geo<T>& g, T iwx,
-                                                T (&d)[NV]) {
+                                                unsigned fl, T (&d)[NV]) {
     T wl[NV], wr[NV], f[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
@@ -150,7 +151,8 @@ struct StripKernel {
       face_pair(limited_slope(lane_up(w[v]), w[v], lane_down(w[v]), g), g.h, w[v], wr[v], hi);
       wl[v] = lane_up(hi);
     }
-    face_flux<T, NDIM, 0, SOLVER>(wl, wr, A.gamma, A.gm1, f);  // the face below each column
+    if constexpr (SW) fl |= __shfl_up_sync(0xffffffffu, fl, 1);
+    Base::template flux<0>(A, wl, wr, fl, f);  // the face below each column
 #pragma unroll
     for (int v = 0; v < NV; ++v) d[v] = mul_rn(sub_rn(f[v], lane_down(f[v])), iwx);
   }
@@ -222,17 +224,18 @@ struct StripKernel {
       load(off, u);
       if (fa) u[1] = -u[1];
       recover<NDIM>(u, w);
-      x_part(A, w, gx, iwx, L);
+      x_part(A, w, gx, iwx, 0u, L);
       finish(off, L, w, T(0));
     } else {
       // W of row m (boundary-mapped); with totals also the row's share of the
       // column sums when it is one of the strip's own
       // (AHEAD: m >= 0, so that only the upper end needs the boundary rule)
-      auto row = [&](int m, T (&u)[NV], auto ahead) {
+      auto row = [&](int m, T (&u)[NV], unsigned& fl, auto ahead) {
         bool fm = false;
         int sm = m;
         if (!decltype(ahead)::value || m >= ny) sm = bc_map(m, ny, A.bc_lo[1], A.bc_hi[1], fm);
         load(off + (Off)sm * (Off)nx, u);
+        if constexpr (SW) fl = A.flags[off + (Off)sm * (Off)nx];
         if (NDIM == 2 && STAGE == 1 && A.want_totals && m >= m0 && m < m1) {
           const T hi = A.wdh[1][m], lo = A.wdl[1][m];
 #pragma unroll
@@ -245,11 +248,12 @@ struct StripKernel {
       // difference across face m + 1/2, hi = the upper face value of cell m,
       // flo = the flux through face m - 1/2.
       T wk[NV], wk1[NV], w2[NV], dlo[NV], hi[NV], flo[NV], u[NV], s[NV], wr[NV];
-      row(m0 - 2, u, std::false_type());
+      unsigned fk = 0, fk1 = 0, fk2 = 0;  // shock bits of rows m, m + 1, m + 2
+      row(m0 - 2, u, fk, std::false_type());
       recover<NDIM>(u, wk);
-      row(m0 - 1, u, std::false_type());
+      row(m0 - 1, u, fk, std::false_type());
       recover<NDIM>(u, wk1);
-      row(m0, u, std::false_type());
+      row(m0, u, fk1, std::false_type());
       recover<NDIM>(u, w2);
       {
         const T t = Base::geo(A, 1, m0 - 2).tipc;
@@ -264,12 +268,14 @@ struct StripKernel {
           wk1[v] = w2[v];
         }
       }
-      row(m0 + 1, u, std::false_type());
+      row(m0 + 1, u, fk2, std::false_type());
       recover<NDIM>(u, w2);
       {
         const Geo<T> g = Base::geo(A, 1, m0);
         march_slope<NV, T>(wk, wk1, w2, g, dlo, s, wr);
-        face_flux<T, NDIM, 1, SOLVER>(hi, wr, A.gamma, A.gm1, flo);
+        Base::template flux<1>(A, hi, wr, fk | fk1, flo);
+        fk = fk1;
+        fk1 = fk2;
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
           hi[v] = fma_rn(s[v], g.h, wk1[v]);
@@ -280,14 +286,16 @@ struct StripKernel {
 #pragma unroll march_unroll<T>()
       for (int m = m0; m < m1; ++m) {
         T L[NV], fhi[NV];
-        row(m + 2, u, std::true_type());  // lands during the x part
-        x_part(A, wk, gx, iwx, L);
+        row(m + 2, u, fk2, std::true_type());  // lands during the x part
+        x_part(A, wk, gx, iwx, fk, L);
         recover<NDIM>(u, w2);
         const Geo<T> g = A.geo[1][m + 3];  // of row m + 1
         const T iwm = A.iw[1][m + 2];
         march_slope<NV, T>(wk, wk1, w2, g, dlo, s, wr);
         // face m + 1/2 between the upper value of m and the lower of m + 1
-        face_flux<T, NDIM, 1, SOLVER>(hi, wr, A.gamma, A.gm1, fhi);
+        Base::template flux<1>(A, hi, wr, fk | fk1, fhi);
+        fk = fk1;
+        fk1 = fk2;
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
           L[v] = fma_rn(sub_rn(flo[v], fhi[v]), iwm, L[v]);
@@ -455,7 +463,7 @@ struct ZMarch {
         asm volatile("cp.async.commit_group;" ::: "memory");
       }
     };
-    auto row = [&](int m, int slot, T (&u)[NV], auto ahead) {
+    auto row = [&](int m, int slot, T (&u)[NV], unsigned& fl, auto ahead) {
       bool fm = false;
       int sm = m;
       if (!decltype(ahead)::value || m >= nz) sm = bc_map(m, nz, A.bc_lo[2], A.bc_hi[2], fm);
@@ -470,6 +478,7 @@ struct ZMarch {
           if (STAGE == 2) u[v] = fma_rn(dt, Acc::at(A.k1 + v * vs, c), u[v]);
         }
       }
+      if constexpr (Base::SW) fl = A.flags[(Off)sm * (Off)plane + (Off)jc];
       if (STAGE == 1 && A.want_totals && m >= m0 && m < m1) {
         const T hi = A.wdh[2][m], lo = A.wdl[2][m];
 #pragma unroll
@@ -478,17 +487,18 @@ struct ZMarch {
       if (fm) u[3] = -u[3];
     };
     T wk[NV], wk1[NV], w2[NV], dlo[NV], hi[NV], flo[NV], u[NV], s[NV], wr[NV];
+    unsigned fk = 0, fk1 = 0, fk2 = 0;  // shock bits of planes m, m + 1, m + 2
     // the first SLOTS planes; the four below are consumed before the march
     if constexpr (ASYNC) {
       for (int i = 0; i < SLOTS; ++i) fill(m0 - 2 + i, i);
       asm volatile("cp.async.wait_group %0;" ::"n"(SLOTS - 4) : "memory");
       __syncwarp();
     }
-    row(m0 - 2, 0, u, std::false_type());
+    row(m0 - 2, 0, u, fk, std::false_type());
     recover<3>(u, wk);
-    row(m0 - 1, 1, u, std::false_type());
+    row(m0 - 1, 1, u, fk, std::false_type());
     recover<3>(u, wk1);
-    row(m0, 2, u, std::false_type());
+    row(m0, 2, u, fk1, std::false_type());
     recover<3>(u, w2);
     {
       const T t = Base::geo(A, 2, m0 - 2).tipc;
@@ -503,12 +513,14 @@ struct ZMarch {
         wk1[v] = w2[v];
       }
     }
-    row(m0 + 1, 3, u, std::false_type());
+    row(m0 + 1, 3, u, fk2, std::false_type());
     recover<3>(u, w2);
     {
       const Geo<T> g = Base::geo(A, 2, m0);
       march_slope<NV, T>(wk, wk1, w2, g, dlo, s, wr);
-      face_flux<T, 3, 2, SOLVER>(hi, wr, A.gamma, A.gm1, flo);
+      Base::template flux<2>(A, hi, wr, fk | fk1, flo);
+      fk = fk1;
+      fk1 = fk2;
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         hi[v] = fma_rn(s[v], g.h, wk1[v]);
@@ -531,7 +543,7 @@ struct ZMarch {
         __syncwarp();  // for every lane, and every lane is done with plane m - 1
         fill(m - 1 + SLOTS, slf);
       }
-      row(m + 2, sl2, u, std::true_type());
+      row(m + 2, sl2, u, fk2, std::true_type());
 #pragma unroll
       for (int v = 0; v < NV; ++v) {  // the strips' x and y parts
         if constexpr (ASYNC) L[v] = ring->a[sl0][NARR - 5 + v][lane];
@@ -541,7 +553,9 @@ struct ZMarch {
       const Geo<T> g = A.geo[2][m + 3];  // of plane m + 1
       const T iwm = A.iw[2][m + 2];
       march_slope<NV, T>(wk, wk1, w2, g, dlo, s, wr);
-      face_flux<T, 3, 2, SOLVER>(hi, wr, A.gamma, A.gm1, fhi);
+      Base::template flux<2>(A, hi, wr, fk | fk1, fhi);
+      fk = fk1;
+      fk1 = fk2;
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         L[v] = fma_rn(sub_rn(flo[v], fhi[v]), iwm, L[v]);
