@@ -103,6 +103,7 @@ __global__ void totals_kernel(ReduceArgs<T> A) {
 // waits for another: the last one to take a ticket does the fold.
 __global__ void __launch_bounds__(32) finalize_kernel(FinalizeArgs A) {
   static_assert(FIN_CTAS <= 32, "one slice result per lane in the last fold");
+  chain_wait();
   const int lane = threadIdx.x, g = blockIdx.x;
   double* work = A.scal + SCAL_COUNT;  // [FIN_CTAS][6]: totals 0..4, speed bits 5
   unsigned* ticket = reinterpret_cast<unsigned*>(A.scal + SCAL_COUNT + FIN_CTAS * 6);
@@ -146,6 +147,7 @@ __global__ void __launch_bounds__(TX * TY) shock_flags_kernel(FlagArgs<T> A, int
   static_assert(NDIM == 2 || NDIM == 3, "the switch runs in 2D and 3D");
   static_assert(2 * (TX + TY) <= TX * TY, "one ring cell per thread at most");
   __shared__ T sp[TY + 2][TX + 2], svx[TY + 2][TX + 2], svy[TY + 2][TX + 2];
+  chain_wait();
   const T gm1 = (T)(A.gamma - 1.0);
   const T dt = A.stage == 2 ? (T)(*A.dt) : T(0);
   const int nx = A.n[0], ny = A.n[1], nz = A.n[2];
@@ -229,6 +231,21 @@ static int grid_for(size_t count, int block, int max_blocks) {
   return (int)(g > (size_t)max_blocks ? max_blocks : g);
 }
 
+cudaError_t launch_chained(const void* fn, dim3 grid, int threads, void** args, size_t smem, cudaStream_t s,
+                           bool chained) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = chained ? 1 : 0;
+  return cudaLaunchKernelExC(&cfg, fn, args);
+}
+
 template <class T>
 cudaError_t launch_init_from_primitive(int ndim, size_t ncell, double gamma, const double* rho, const double* vel,
                                        const double* p, T* U, cudaStream_t s) {
@@ -263,13 +280,16 @@ cudaError_t launch_totals(int ndim, const ReduceArgs<T>& A, cudaStream_t s) {
 }
 
 template <class T>
-cudaError_t launch_shock_flags(int ndim, const FlagArgs<T>& A, cudaStream_t s) {
+cudaError_t launch_shock_flags(int ndim, const FlagArgs<T>& A, cudaStream_t s, bool chained) {
   if (ndim == 2) {
     constexpr int TX = 32, TY = 8;
     const long long bx = (A.n[0] + TX - 1) / TX, by = (A.n[1] + TY - 1) / TY;
     if (by > 65535) return cudaErrorInvalidConfiguration;
-    shock_flags_kernel<T, 2, TX, TY><<<dim3((unsigned)bx, (unsigned)by, 1), TX * TY, 0, s>>>(A, 1);
-    return cudaGetLastError();
+    int kz = 1;
+    FlagArgs<T> a = A;
+    void* p[] = {&a, &kz};
+    return launch_chained(reinterpret_cast<const void*>(&shock_flags_kernel<T, 2, TX, TY>),
+                          dim3((unsigned)bx, (unsigned)by, 1), TX * TY, p, 0, s, chained);
   }
   if (ndim != 3) return cudaErrorInvalidValue;  // 1D runs plain HLLC
   // 32 x 4 tiles (many small CTAs keep the most loads in flight); z chunks
@@ -285,15 +305,19 @@ cudaError_t launch_shock_flags(int ndim, const FlagArgs<T>& A, cudaStream_t s) {
   const int nz = A.n[2];
   long long chunks = (target + bx * by - 1) / (bx * by);
   chunks = chunks < 1 ? 1 : (chunks > nz ? nz : (chunks > 65535 ? 65535 : chunks));
-  const int kz = (int)((nz + chunks - 1) / chunks);
+  int kz = (int)((nz + chunks - 1) / chunks);
   chunks = (nz + kz - 1) / kz;
-  shock_flags_kernel<T, 3, TX, TY><<<dim3((unsigned)bx, (unsigned)by, (unsigned)chunks), TX * TY, 0, s>>>(A, kz);
-  return cudaGetLastError();
+  FlagArgs<T> a = A;
+  void* p[] = {&a, &kz};
+  return launch_chained(reinterpret_cast<const void*>(&shock_flags_kernel<T, 3, TX, TY>),
+                        dim3((unsigned)bx, (unsigned)by, (unsigned)chunks), TX * TY, p, 0, s, chained);
 }
 
-cudaError_t launch_finalize(const FinalizeArgs& A, cudaStream_t s) {
-  finalize_kernel<<<A.nblk <= 512 ? 1 : FIN_CTAS, 32, 0, s>>>(A);
-  return cudaGetLastError();
+cudaError_t launch_finalize(const FinalizeArgs& A, cudaStream_t s, bool chained) {
+  FinalizeArgs a = A;
+  void* p[] = {&a};
+  return launch_chained(reinterpret_cast<const void*>(&finalize_kernel), dim3(A.nblk <= 512 ? 1 : FIN_CTAS), 32, p, 0, s,
+                        chained);
 }
 
 template cudaError_t launch_init_from_primitive<float>(int, size_t, double, const double*, const double*,
@@ -314,7 +338,7 @@ template cudaError_t launch_convert<dw, double>(size_t, const dw*, double*, cuda
 template cudaError_t launch_convert<dw, float>(size_t, const dw*, float*, cudaStream_t);
 template cudaError_t launch_speed<dw>(int, const ReduceArgs<dw>&, cudaStream_t);
 template cudaError_t launch_totals<dw>(int, const ReduceArgs<dw>&, cudaStream_t);
-template cudaError_t launch_shock_flags<float>(int, const FlagArgs<float>&, cudaStream_t);
-template cudaError_t launch_shock_flags<double>(int, const FlagArgs<double>&, cudaStream_t);
+template cudaError_t launch_shock_flags<float>(int, const FlagArgs<float>&, cudaStream_t, bool);
+template cudaError_t launch_shock_flags<double>(int, const FlagArgs<double>&, cudaStream_t, bool);
 
 }  // namespace gh

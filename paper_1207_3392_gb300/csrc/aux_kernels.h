@@ -7,6 +7,12 @@
 
 namespace gh {
 
+// Launch of a kernel that begins with chain_wait() (hydro_device.cuh): it may be
+// placed while the kernel before it on the stream drains
+// (chained; else an ordinary launch).
+cudaError_t launch_chained(const void* fn, dim3 grid, int threads, void** args, size_t smem, cudaStream_t s,
+                           bool chained);
+
 // Slots of the per-handle device scalar block.
 enum { SCAL_DT = 0, SCAL_T = 1, SCAL_DTCFL = 2, SCAL_TOT = 3, SCAL_COUNT = 8 };
 enum { FIN_FIXED = 0, FIN_CFL = 1, FIN_REDUCE = 2 };
@@ -59,7 +65,7 @@ struct FlagArgs {
 };
 
 template <class T>
-cudaError_t launch_shock_flags(int ndim, const FlagArgs<T>& A, cudaStream_t s);
+cudaError_t launch_shock_flags(int ndim, const FlagArgs<T>& A, cudaStream_t s, bool chained);
 
 // The detector of Runge-Kutta stage 1 on 3D FP32 meshes with the state
 // planes staged by TMA (flags_tma.cu).  Usable when n[0] is a multiple of 4
@@ -78,6 +84,6 @@ template <class T>
 cudaError_t launch_speed(int ndim, const ReduceArgs<T>& A, cudaStream_t s);
 template <class T>
 cudaError_t launch_totals(int ndim, const ReduceArgs<T>& A, cudaStream_t s);
-cudaError_t launch_finalize(const FinalizeArgs& A, cudaStream_t s);
+cudaError_t launch_finalize(const FinalizeArgs& A, cudaStream_t s, bool chained = false);
 
 }  // namespace gh

@@ -17,6 +17,16 @@ enum : int { BC_PERIODIC = 0, BC_REFLECT = 1, BC_OUTFLOW = 2 };
 enum : int { SOLVER_HLL = 0, SOLVER_HLLC = 1, SOLVER_HLLC_SW = 2 };
 enum : unsigned { STATUS_NONPHYS = 1u, STATUS_TIMEOUT = 2u };
 
+// Programmatic dependent launch: a kernel of a step's chain is launched while
+// its predecessor's last CTAs still run.  chain_wait() returns when the
+// predecessor has finished and its writes are visible, and lets the successor's
+// CTAs be placed; a kernel of the chain calls it before any access to memory
+// that a kernel writes.  Without the launch attribute it is a no-op.
+__device__ __forceinline__ void chain_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Per-cell reconstruction geometry along one axis (Eq. MinMod with
 // non-uniform centre distances): theta / (q_c - q_-), 1 / (q_+ - q_-),
 // theta / (q_+ - q_c), and the half width (face offset from the geometric

@@ -40,6 +40,7 @@ struct genasis_hydro {
   int tile = 0, kchunk_req = 0, kchunk = 1;
   gh::StageVariant v1{}, v2{};
   dim3 grid, grid2;  // stage 1 / stage 2 (the two may use different tile shapes)
+  bool chained = false;  // the step's kernels overlap their predecessors' ends (launch_chained)
   // 3D on independent warps: strips per row, rows per warp and grid of the x/y launch
   int xy_strips = 0, xy_rows = 0;
   dim3 xy_grid;

@@ -821,6 +821,7 @@ struct StageKernel {
 // MINB: CTAs per SM the register allocation must allow (__launch_bounds__).
 template <int NDIM, class T, int SOLVER, int STAGE, int TX, int TY, int MINB, bool PRE>
 __global__ void __launch_bounds__(TX * TY, MINB) hydro_stage_kernel(const StageArgs<T> A) {
+  chain_wait();
   StageKernel<NDIM, T, SOLVER, STAGE, TX, TY, PRE>::run(A);
 }
 

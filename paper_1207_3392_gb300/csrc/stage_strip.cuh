@@ -351,6 +351,7 @@ __global__ void __launch_bounds__(32 * NW, (strip_warps<T, 2>() / NW)) hydro_str
   using K = StripKernel<2, T, SOLVER, STAGE, WIDE>;
   constexpr int NV = 4;
   __shared__ double red[NW][NV + 1];
+  chain_wait();
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
   const int x0 = (blockIdx.x * NW + warp) * STRIP_OWN;
   const int m0 = blockIdx.z * A.kchunk, m1 = min(A.n[1], m0 + A.kchunk);
@@ -371,6 +372,7 @@ template <class T, int SOLVER, int STAGE, int NW, bool WIDE>
 __global__ void __launch_bounds__(32 * NW, (strip_warps<T, 3>() / NW))
     hydro_strip_xy_kernel(const StageArgs<T> A, int strips, int ychunk) {
   using K = StripKernel<3, T, SOLVER, STAGE, WIDE>;
+  chain_wait();
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
   const int id = blockIdx.x * NW + warp;
   const int k = id / strips;
@@ -615,6 +617,7 @@ __global__ void __launch_bounds__(128, (sizeof(T) == 8 ? 4 : ASYNC && STAGE == 2
   constexpr int NV = 5, NW = 4;
   extern __shared__ __align__(16) unsigned char smem_z[];
   __shared__ double red[NW][NV + 1];
+  chain_wait();
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
   // chunks in descending order: the strips' last planes are still in L2
   const int chunk = gridDim.z - 1 - blockIdx.z;
