@@ -157,6 +157,7 @@ struct TrainSmem {
   __nv_bfloat16 d1t[mlp::NH][TSP];   // (dL/dz1)^T
   __nv_bfloat16 d2t[mlp::NH][TSP];   // (dL/dz2)^T
   __nv_bfloat16 dyt[16][TSP];        // (dL/dy)^T, rows >= 4 zero
+  __nv_bfloat16 ones[8][TSP];        // row 0 ones: a product with it sums over the samples
   float red[256];
 };
 
@@ -197,12 +198,14 @@ __global__ void __launch_bounds__(256) mlp_train_kernel(const float* __restrict_
                                                         float* __restrict__ part, float* __restrict__ part_loss) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TrainSmem& S = *reinterpret_cast<TrainSmem*>(smem_raw);
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // the reduction is placed, and waits
   mlp::load_weights(S.W, P);
   for (int i = threadIdx.x; i < 16 * TSP; i += blockDim.x) (&S.dyt[0][0])[i] = __float2bfloat16(0.0f);
+  for (int i = threadIdx.x; i < 8 * TSP; i += blockDim.x) (&S.ones[0][0])[i] = __float2bfloat16(i < TSP ? 1.0f : 0.0f);
   __syncthreads();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   float gw1[2][4] = {}, gw2[4][4] = {}, gw3[4] = {};
-  float gb = 0.0f, loss = 0.0f;
+  float gb[4] = {}, gb3[4] = {}, loss = 0.0f;
   for (long long base = (long long)blockIdx.x * TS; base < n; base += (long long)gridDim.x * TS) {
     const long long s0 = base + 16 * warp;
     const int rows = (int)(n - s0 <= 0 ? 0 : (n - s0 < 16 ? n - s0 : 16));
@@ -279,18 +282,12 @@ __global__ void __launch_bounds__(256) mlp_train_kernel(const float* __restrict_
       grad_tile(gw2[i], S.d2t, 16 * (tile / 8), S.h1t, 8 * (tile % 8));
     }
     grad_tile(gw3, S.dyt, 0, S.h2t, 8 * warp);
-    // bias gradients: row sums of the transposed derivative tables
-    {
-      const __nv_bfloat16* row = tid < 64 ? S.d1t[tid] : tid < 128 ? S.d2t[tid - 64] : S.dyt[(tid - 128) & 15];
-      if (tid < 132) {
-        float s = 0.f;
-        for (int k = 0; k < TS; k += 2) {
-          const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162*>(row + k);
-          s += __bfloat162float(v.x) + __bfloat162float(v.y);
-        }
-        gb += s;
-      }
-    }
+    // bias gradients: the sums of the derivatives over the samples, as products
+    // with a row of ones (one more tile a warp; a thread per bias summing its
+    // row of 128 values took longer than all the tiles)
+    if (warp < 4) grad_tile(gb, S.d1t, 16 * warp, S.ones, 0);
+    else grad_tile(gb, S.d2t, 16 * (warp - 4), S.ones, 0);
+    if (warp == 0) grad_tile(gb3, S.dyt, 0, S.ones, 0);
     __syncthreads();
   }
   // write this CTA's partial gradient
@@ -318,9 +315,12 @@ __global__ void __launch_bounds__(256) mlp_train_kernel(const float* __restrict_
     const int r = g + (e >= 2 ? 8 : 0), c = 8 * warp + 2 * t + (e & 1);
     if (r < mlp::NOUT) G[mlp::OW3 + r * mlp::NH + c] = gw3[e];
   }
-  if (tid < 64) G[mlp::OB1 + tid] = gb;
-  else if (tid < 128) G[mlp::OB2 + tid - 64] = gb;
-  else if (tid < 132) G[mlp::OB3 + tid - 128] = gb;
+  if (t == 0) {  // column 0 of the tile: rows g and g + 8
+    float* B = G + (warp < 4 ? mlp::OB1 + 16 * warp : mlp::OB2 + 16 * (warp - 4));
+    B[g] = gb[0];
+    B[g + 8] = gb[2];
+    if (warp == 0 && g < mlp::NOUT) G[mlp::OB3 + g] = gb3[0];
+  }
   // loss: fixed-order block sum
   S.red[tid] = loss;
   __syncthreads();
@@ -331,20 +331,53 @@ __global__ void __launch_bounds__(256) mlp_train_kernel(const float* __restrict_
   if (tid == 0) part_loss[blockIdx.x] = S.red[0];
 }
 
-// Sum the per-CTA partials in order (gradient, loss); optionally one Adam step
-// on the FP32 parameters (Kingma & Ba, bias-corrected).
-__global__ void mlp_reduce_adam_kernel(const float* __restrict__ part, const float* __restrict__ part_loss, int nblk,
-                                       float* __restrict__ grad_out, float* __restrict__ loss_out, float* P, float* m,
-                                       float* v, int step, float lr, float b1, float b2, float eps) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p == 0 && loss_out) {
-    float s = 0.f;
-    for (int b = 0; b < nblk; ++b) s += part_loss[b];
-    *loss_out = s;
+// Sum the per-CTA partials in a fixed order (gradient, loss); optionally one
+// Adam step on the FP32 parameters (Kingma & Ba, bias-corrected).  A CTA takes
+// RED_PARAMS parameters; RED_SLICES threads per parameter sum every
+// RED_SLICES-th partial, so that the loads of all partials are in flight at
+// once (one thread per parameter walked 152 partials in 13 us), and the slices
+// are added in order.  The CTA after the last parameter sums the loss.  The
+// kernel is placed while the training kernel runs.  A gradient of 32,768
+// samples with this, the weights staged in one pass and the bias sums as
+// products: 30.5 -> 20.4 us; of 512 samples 21.2 -> 14.8.
+constexpr int RED_PARAMS = 32, RED_SLICES = 8;
+constexpr int RED_CTAS = (mlp::NPARAM + RED_PARAMS - 1) / RED_PARAMS + 1;
+
+__global__ void __launch_bounds__(RED_PARAMS * RED_SLICES)
+    mlp_reduce_adam_kernel(const float* __restrict__ part, const float* __restrict__ part_loss, int nblk,
+                           float* __restrict__ grad_out, float* __restrict__ loss_out, float* P, float* m, float* v,
+                           int step, float lr, float b1, float b2, float eps) {
+  __shared__ float sums[RED_SLICES][RED_PARAMS];
+  chain_wait();
+  const int col = threadIdx.x % RED_PARAMS, slice = threadIdx.x / RED_PARAMS;
+  if (blockIdx.x == RED_CTAS - 1) {
+    if (!loss_out || slice != 0) return;
+    double s = 0.0;
+    for (int b = col; b < nblk; b += 32) s += (double)part_loss[b];
+    s = warp_sum(s);
+    if (col == 0) *loss_out = (float)s;
+    return;
   }
-  if (p >= mlp::NPARAM) return;
+  const int p = blockIdx.x * RED_PARAMS + col;
   float g = 0.f;
-  for (int b = 0; b < nblk; ++b) g += part[(size_t)b * mlp::NPARAM + p];
+  if (p < mlp::NPARAM) {
+    constexpr int BATCH = 20;  // reads in flight: all of them up to 160 partials
+    for (int b0 = slice; b0 < nblk; b0 += BATCH * RED_SLICES) {
+      float x[BATCH];
+#pragma unroll
+      for (int k = 0; k < BATCH; ++k) {
+        const int b = b0 + k * RED_SLICES;
+        x[k] = b < nblk ? part[(size_t)b * mlp::NPARAM + p] : 0.f;
+      }
+#pragma unroll
+      for (int k = 0; k < BATCH; ++k) g += x[k];
+    }
+  }
+  sums[slice][col] = g;
+  __syncthreads();
+  if (slice != 0 || p >= mlp::NPARAM) return;
+#pragma unroll
+  for (int k = 1; k < RED_SLICES; ++k) g += sums[k][col];
   if (grad_out) grad_out[p] = g;
   if (step > 0) {
     const float mm = b1 * m[p] + (1.f - b1) * g;
@@ -530,7 +563,9 @@ int mlp_grad_impl(const float* P, const void* X, const float* T, long long n, fl
   GH_CK(cudaGetDevice(&dev));
   GH_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   long long iters = (n + TS - 1) / TS;
-  int nblk = (int)(iters < (long long)sms ? iters : (long long)sms);
+  // the fewest CTAs that keep the number of rounds: each leaves a partial
+  const long long rounds = (iters + sms - 1) / sms;
+  const int nblk = (int)((iters + rounds - 1) / rounds);
   float* part = nullptr;
   float* part_loss = nullptr;
   GH_CK(cudaMallocAsync((void**)&part, (size_t)nblk * mlp::NPARAM * sizeof(float), st));
@@ -539,9 +574,11 @@ int mlp_grad_impl(const float* P, const void* X, const float* T, long long n, fl
   mlp_train_kernel<<<nblk, 256, sizeof(TrainSmem), st>>>(P, (const __nv_bfloat16*)X, T, n, inv, part, part_loss);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) {
-    mlp_reduce_adam_kernel<<<(mlp::NPARAM + 255) / 256, 256, 0, st>>>(part, part_loss, nblk, grad, loss, Pupd, m, v, step,
-                                                                       lr, 0.9f, 0.999f, 1e-8f);
-    e = cudaGetLastError();
+    float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+    int blocks = nblk;
+    void* p[] = {&part, &part_loss, &blocks, &grad, &loss, &Pupd, &m, &v, &step, &lr, &b1, &b2, &eps};
+    e = launch_chained(reinterpret_cast<const void*>(&mlp_reduce_adam_kernel), dim3(RED_CTAS), RED_PARAMS * RED_SLICES, p,
+                       0, st, true);
   }
   cudaFreeAsync(part, st);
   cudaFreeAsync(part_loss, st);

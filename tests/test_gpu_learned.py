@@ -111,6 +111,30 @@ def test_mlp_gradient_matches_reference():
     assert float(loss.item()) == pytest.approx(le, rel=2e-3)
 
 
+@pytest.mark.parametrize("n", [1, 15, 128, 129, 19456, 19457, 41000])
+def test_mlp_gradient_over_partial_and_many_tiles(n):
+    """One sample, a ragged and a full 128-sample tile, one round of CTAs filled
+    and passed by one tile, three rounds: each layer's gradient (weights and
+    biases) and the loss against the emulated BF16 gradient, with the bars of
+    the test above."""
+    import torch
+    rng = np.random.default_rng(n)
+    th = _random_net(4)
+    X = M.bf16(rng.normal(0, 0.7, (n, 24)))
+    T = rng.normal(0, 0.3, (n, 4))
+    g = torch.empty(M.NPARAM, device="cuda")
+    loss = torch.empty(1, device="cuda")
+    H.mlp_gradient(_dev(th, torch.float32), _x_bf16(X), _dev(T, torch.float32), g, loss)
+    gg = g.cpu().numpy().astype(np.float64)
+    ge, le = _emulated_grad(th, X, T)
+    o = 0
+    for name, shp in M.SHAPES:
+        k = int(np.prod(shp))
+        assert _rel(gg[o:o + k], ge[o:o + k]) < 2e-2, name
+        o += k
+    assert float(loss.item()) == pytest.approx(le, rel=2e-3)
+
+
 def test_adam_training_fits_a_teacher():
     import torch
     rng = np.random.default_rng(5)
