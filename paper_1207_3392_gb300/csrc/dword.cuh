@@ -15,7 +15,14 @@
 //   residual; the approximate reciprocal of the hardware suffices because the
 //   residual corrects q1;
 //   square root is one Newton correction of an approximate float root s from
-//   the exact residual x - s^2.
+//   the exact residual x - s^2;
+//   fma takes the product's high part and error into the sum without normalising
+//   in between, three operations fewer: the distance to the FP64 update after
+//   12 steps goes from 3.2 - 3.4e-15 to 2.2 - 2.4e-15 in 2D, from 1.7 - 3.0e-15
+//   to 1.6 - 2.7e-15 in 3D, and stays at 2.0e-15 in 1D.
+// The FP32 pipes bound the double-word update; with this fma, the sound speed
+// with one correction and one product for both face values, 6 steps of 128^3
+// went from 6005 to 5624 us.
 // The operations are hidden friends (found by argument-dependent lookup), so
 // they add to, rather than hide, the float and double overloads of fma,
 // fmax, fmin, fabs and __ldg.  Every float operation is an explicitly rounded
@@ -42,6 +49,14 @@ __device__ __forceinline__ void fast_two_sum(float a, float b, float& s, float& 
 __device__ __forceinline__ void two_prod(float a, float b, float& p, float& e) {
   p = __fmul_rn(a, b);
   e = __fmaf_rn(a, b, -p);
+}
+
+// hardware reciprocal (relative error about 2^-23); infinite for a subnormal x,
+// whose residual x - q1 y would have no bits left below it in any case
+__device__ __forceinline__ float approx_rcp(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
 }
 
 struct __align__(8) dw {
@@ -75,7 +90,7 @@ struct __align__(8) dw {
   }
 
   friend __device__ __forceinline__ dw operator/(dw x, dw y) {
-    const float r0 = __fdividef(1.0f, y.hi);  // hardware reciprocal, a few ulp
+    const float r0 = approx_rcp(y.hi);
     const float q1 = __fmul_rn(x.hi, r0);
     float ph, pl, zh, zl;
     two_prod(q1, y.hi, ph, pl);
@@ -96,7 +111,16 @@ struct __align__(8) dw {
   friend __device__ __forceinline__ bool operator==(dw x, dw y) { return x.hi == y.hi && x.lo == y.lo; }
   friend __device__ __forceinline__ bool operator!=(dw x, dw y) { return !(x == y); }
 
-  friend __device__ __forceinline__ dw fma(dw a, dw b, dw c) { return a * b + c; }
+  // a b + c: the product's high part and its error enter the sum without being
+  // normalised in between (three operations fewer; the same low-order terms)
+  friend __device__ __forceinline__ dw fma(dw a, dw b, dw c) {
+    float ch, cl1, sh, sl, zh, zl;
+    two_prod(a.hi, b.hi, ch, cl1);
+    const float cl = __fadd_rn(cl1, __fmaf_rn(a.lo, b.hi, __fmaf_rn(a.hi, b.lo, __fmul_rn(a.lo, b.lo))));
+    two_sum(ch, c.hi, sh, sl);
+    fast_two_sum(sh, __fadd_rn(sl, __fadd_rn(cl, c.lo)), zh, zl);
+    return dw(zh, zl);
+  }
   friend __device__ __forceinline__ dw fabs(dw x) { return x.hi < 0.0f ? -x : x; }
   friend __device__ __forceinline__ dw fmax(dw x, dw y) { return x < y ? y : x; }
   friend __device__ __forceinline__ dw fmin(dw x, dw y) { return y < x ? y : x; }

@@ -168,11 +168,18 @@ __device__ __forceinline__ float sub_half(float c, float a) { return __fmaf_rn(-
 __device__ __forceinline__ double sub_half(double c, double a) { return __fma_rn(-0.5, a, c); }
 __device__ __forceinline__ dw sub_half(dw c, dw a) { return c - half_of(a); }
 
-// Values a distance h s below and above wc (the two faces of a cell).
+// Values a distance h s below and above wc (the two faces of a cell), alone and
+// as a pair; double word forms h s once for both.
+template <class T>
+__device__ __forceinline__ T face_lo(T s, T h, T wc) { return fma_rn(-s, h, wc); }
+template <class T>
+__device__ __forceinline__ T face_hi(T s, T h, T wc) { return fma_rn(s, h, wc); }
+__device__ __forceinline__ dw face_lo(dw s, dw h, dw wc) { return wc - s * h; }
+__device__ __forceinline__ dw face_hi(dw s, dw h, dw wc) { return wc + s * h; }
 template <class T>
 __device__ __forceinline__ void face_pair(T s, T h, T wc, T& lo, T& hi) {
-  lo = fma_rn(-s, h, wc);
-  hi = fma_rn(s, h, wc);
+  lo = face_lo(s, h, wc);
+  hi = face_hi(s, h, wc);
 }
 __device__ __forceinline__ void face_pair(dw s, dw h, dw wc, dw& lo, dw& hi) {
   const dw d = s * h;
@@ -252,8 +259,23 @@ __device__ __forceinline__ dw frcp(dw x) { return dw(1.0f, 0.0f) / x; }
 // then x^(-1/2) = r (1 - e)^(-1/2) = r (1 + e/2 + 3 e^2/8 + ...), which leaves
 // 5 e^3/16 ~ 2^-65: seven FP64 operations; CUDA's rsqrt outside the seed range,
 // and 0 where gamma p is not positive.  FP32: the hardware approximation.
-// Double word: the quotient and square root of dword.cuh.
-__device__ __forceinline__ dw sound_speed(dw gamma, dw p, dw n) { return sqrt(gamma * (p / n)); }
+// Double word: the same form with one correction (34 -> 26 operations), the
+// quotient and square root of dword.cuh where gp n nears the ends of FP32.
+__device__ __forceinline__ dw sound_speed(dw gamma, dw p, dw n) {
+  const dw gp = gamma * p;
+  const float x = mul_rn(gp.hi, n.hi);
+  if (!(x > 1e-30f && x < 1e30f)) return sqrt(gamma * (p / n));
+  // c0 = gp rsqrt(gp n) and one Newton correction (gp - n c0^2) / (2 n c0) from
+  // the exact residual, 1 / (n c0) = rsqrt(gp n)
+  const float r = frsqrt(x), c0 = mul_rn(gp.hi, r);
+  float q, qe, ph, pl, zh, zl;
+  two_prod(c0, c0, q, qe);
+  two_prod(n.hi, q, ph, pl);
+  pl = fma_rn(n.hi, qe, fma_rn(n.lo, q, pl));
+  const float res = add_rn(sub_rn(sub_rn(gp.hi, ph), pl), gp.lo);  // gp.hi - ph exact
+  fast_two_sum(c0, mul_rn(res, mul_rn(0.5f, r)), zh, zl);
+  return dw(zh, zl);
+}
 __device__ __forceinline__ float sound_speed(float gamma, float p, float n) {
   const float gp = mul_rn(gamma, p);
   return mul_rn(gp, frsqrt(mul_rn(gp, n)));

@@ -343,8 +343,8 @@ struct StageKernel {
       get_w(S, b, srow, sl + 2, w3);
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        wl[v] = fma_rn(limited_slope(w0[v], w1[v], w2[v], gl), gl.h, w1[v]);
-        wr[v] = fma_rn(-limited_slope(w1[v], w2[v], w3[v], gr), gr.h, w2[v]);
+        wl[v] = face_hi(limited_slope(w0[v], w1[v], w2[v], gl), gl.h, w1[v]);
+        wr[v] = face_lo(limited_slope(w1[v], w2[v], w3[v], gr), gr.h, w2[v]);
       }
     }
     flux<0>(A, wl, wr, SW ? (unsigned)(S.fl[b][SW ? srow : 0][SW ? sl : 0] | S.fl[b][SW ? srow : 0][SW ? sl + 1 : 0]) : 0u,
@@ -367,8 +367,8 @@ struct StageKernel {
       get_w(S, b, sl + 2, scol, w3);
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        wl[v] = fma_rn(limited_slope(w0[v], w1[v], w2[v], gl), gl.h, w1[v]);
-        wr[v] = fma_rn(-limited_slope(w1[v], w2[v], w3[v], gr), gr.h, w2[v]);
+        wl[v] = face_hi(limited_slope(w0[v], w1[v], w2[v], gl), gl.h, w1[v]);
+        wr[v] = face_lo(limited_slope(w1[v], w2[v], w3[v], gr), gr.h, w2[v]);
       }
     }
     flux<1>(A, wl, wr, SW ? (unsigned)(S.fl[b][SW ? sl : 0][SW ? scol : 0] | S.fl[b][SW ? sl + 1 : 0][SW ? scol : 0]) : 0u,
@@ -384,8 +384,8 @@ struct StageKernel {
     T wl[NV], wr[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-      wl[v] = fma_rn(sa[v], ha, wa[v]);
-      wr[v] = fma_rn(-sb[v], hb, wb[v]);
+      wl[v] = face_hi(sa[v], ha, wa[v]);
+      wr[v] = face_lo(sb[v], hb, wb[v]);
     }
     flux<AM>(A, wl, wr, bits, f);
   }
@@ -444,7 +444,7 @@ struct StageKernel {
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         const T sv = limited_slope(wm[v], w1[v], wp[v], g);
-        o[v] = up ? fma_rn(-sv, g.h, w1[v]) : fma_rn(sv, g.h, w1[v]);
+        o[v] = up ? face_lo(sv, g.h, w1[v]) : face_hi(sv, g.h, w1[v]);
       }
       if (up) put_xs(S, 0, r, TX + 1, o);
       else put_xs(S, 1, r, 0, o);
@@ -462,7 +462,7 @@ struct StageKernel {
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         const T sv = limited_slope(wm[v], w1[v], wp[v], g);
-        o[v] = up ? fma_rn(-sv, g.h, w1[v]) : fma_rn(sv, g.h, w1[v]);
+        o[v] = up ? face_lo(sv, g.h, w1[v]) : face_hi(sv, g.h, w1[v]);
       }
       if (up) put_ys(S, 0, TY + 1, c, o);
       else put_ys(S, 1, 0, c, o);

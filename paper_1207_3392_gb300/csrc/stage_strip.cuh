@@ -126,7 +126,7 @@ __device__ __forceinline__ void march_slope(const T (&wm)[NV], const T (&wc)[NV]
   for (int v = 0; v < NV; ++v) {
     const T dhi = mul_rn(sub_rn(wp[v], wc[v]), g.tipc);
     s[v] = minmod3(dlo[v], mul_rn(sub_rn(wp[v], wm[v]), g.ipm), dhi);
-    wr[v] = fma_rn(-s[v], g.h, wc[v]);
+    wr[v] = face_lo(s[v], g.h, wc[v]);
     dlo[v] = dhi;
   }
 }
@@ -263,7 +263,7 @@ struct StripKernel {
         march_slope<NV, T>(wk, wk1, w2, g, dlo, s, wr);
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
-          hi[v] = fma_rn(s[v], g.h, wk1[v]);
+          hi[v] = face_hi(s[v], g.h, wk1[v]);
           wk[v] = wk1[v];
           wk1[v] = w2[v];
         }
@@ -278,7 +278,7 @@ struct StripKernel {
         fk1 = fk2;
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
-          hi[v] = fma_rn(s[v], g.h, wk1[v]);
+          hi[v] = face_hi(s[v], g.h, wk1[v]);
           wk[v] = wk1[v];
           wk1[v] = w2[v];
         }
@@ -304,7 +304,7 @@ struct StripKernel {
         finish(off + (Off)m * (Off)nx, L, wk, iwm);
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
-          hi[v] = fma_rn(s[v], g.h, wk1[v]);
+          hi[v] = face_hi(s[v], g.h, wk1[v]);
           wk[v] = wk1[v];
           wk1[v] = w2[v];
         }
@@ -510,7 +510,7 @@ struct ZMarch {
       march_slope<NV, T>(wk, wk1, w2, g, dlo, s, wr);
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        hi[v] = fma_rn(s[v], g.h, wk1[v]);
+        hi[v] = face_hi(s[v], g.h, wk1[v]);
         wk[v] = wk1[v];
         wk1[v] = w2[v];
       }
@@ -525,7 +525,7 @@ struct ZMarch {
       fk1 = fk2;
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        hi[v] = fma_rn(s[v], g.h, wk1[v]);
+        hi[v] = face_hi(s[v], g.h, wk1[v]);
         wk[v] = wk1[v];
         wk1[v] = w2[v];
       }
@@ -592,7 +592,7 @@ struct ZMarch {
       }
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        hi[v] = fma_rn(s[v], g.h, wk1[v]);
+        hi[v] = face_hi(s[v], g.h, wk1[v]);
         wk[v] = wk1[v];
         wk1[v] = w2[v];
       }
