@@ -746,20 +746,19 @@ int genasis_hydro_set_primitive(genasis_hydro_t h, const double* rho, const doub
     const double* v = dev[1] ? dev[1] : vel;
     const double* pp = dev[2] ? dev[2] : p;
     void* U = h->U[h->cur];
+    double* t = h->scal + SCAL_T;
     cudaError_t e =
         h->prec == GENASIS_FP64
-            ? launch_init_from_primitive<double>(h->ndim, h->ncell, h->gamma, r, v, pp, (double*)U, h->stream)
+            ? launch_init_from_primitive<double>(h->ndim, h->ncell, h->gamma, r, v, pp, (double*)U, t, h->stream)
         : h->prec == GENASIS_FP32_MIXED
-            ? launch_init_from_primitive<float>(h->ndim, h->ncell, h->gamma, r, v, pp, (float*)U, h->stream)
-            : launch_init_from_primitive<dw>(h->ndim, h->ncell, h->gamma, r, v, pp, (dw*)U, h->stream);
+            ? launch_init_from_primitive<float>(h->ndim, h->ncell, h->gamma, r, v, pp, (float*)U, t, h->stream)
+            : launch_init_from_primitive<dw>(h->ndim, h->ncell, h->gamma, r, v, pp, (dw*)U, t, h->stream);
     if (e != cudaSuccess) rc = fail(GENASIS_ECUDA, "init kernel: %s", cudaGetErrorString(e));
   }
   for (int a = 0; a < 3; ++a)
     if (dev[a]) cudaFreeAsync(dev[a], h->stream);
-  if (!rc) {
-    GH_CK(cudaMemsetAsync(h->scal + SCAL_T, 0, sizeof(double), h->stream));
-    if (!is_device_ptr(rho) || !is_device_ptr(vel) || !is_device_ptr(p)) GH_CK(cudaStreamSynchronize(h->stream));
-  }
+  if (!rc && (!is_device_ptr(rho) || !is_device_ptr(vel) || !is_device_ptr(p)))
+    GH_CK(cudaStreamSynchronize(h->stream));
   return rc;
 }
 

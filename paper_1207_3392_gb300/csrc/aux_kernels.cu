@@ -10,11 +10,17 @@ namespace gh {
 
 // U = (D, S, G) from (rho, v, p): D = rho, S = rho v, G = p/(gamma-1) + rho |v|^2 / 2
 // (Sec. 3.5, m = 1), evaluated in FP64 and rounded once to the storage type.
+// U of primitive variables, and *t = 0.  Small meshes are bound by the launch:
+// the problems of a batch are set one call after the other, so the kernel is
+// placed while its predecessor drains and the time needs no operation of its own
+// (256 problems, 128 to 4096 and 64^2 to 512^2 cells, set in FP32: 2.16 -> 1.76 ms)
 template <class T>
 __global__ void init_from_primitive_kernel(int ndim, size_t ncell, double gamma, const double* __restrict__ rho,
                                            const double* __restrict__ vel, const double* __restrict__ p,
-                                           T* __restrict__ U) {
+                                           T* __restrict__ U, double* __restrict__ t) {
+  chain_wait();
   const int nv = ndim + 2;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *t = 0.0;
   for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < ncell; c += (size_t)gridDim.x * blockDim.x) {
     const double n = rho[c];
     double v2 = 0.0;
@@ -248,9 +254,10 @@ cudaError_t launch_chained(const void* fn, dim3 grid, int threads, void** args, 
 
 template <class T>
 cudaError_t launch_init_from_primitive(int ndim, size_t ncell, double gamma, const double* rho, const double* vel,
-                                       const double* p, T* U, cudaStream_t s) {
-  init_from_primitive_kernel<T><<<grid_for(ncell, 256, 4096), 256, 0, s>>>(ndim, ncell, gamma, rho, vel, p, U);
-  return cudaGetLastError();
+                                       const double* p, T* U, double* t, cudaStream_t s) {
+  void* a[] = {&ndim, &ncell, &gamma, &rho, &vel, &p, &U, &t};
+  return launch_chained(reinterpret_cast<const void*>(&init_from_primitive_kernel<T>),
+                        dim3(grid_for(ncell, 256, 4096)), 256, a, 0, s, true);
 }
 
 template <class Tin, class Tout>
@@ -321,9 +328,9 @@ cudaError_t launch_finalize(const FinalizeArgs& A, cudaStream_t s, bool chained)
 }
 
 template cudaError_t launch_init_from_primitive<float>(int, size_t, double, const double*, const double*,
-                                                       const double*, float*, cudaStream_t);
+                                                       const double*, float*, double*, cudaStream_t);
 template cudaError_t launch_init_from_primitive<double>(int, size_t, double, const double*, const double*,
-                                                        const double*, double*, cudaStream_t);
+                                                        const double*, double*, double*, cudaStream_t);
 template cudaError_t launch_convert<float, double>(size_t, const float*, double*, cudaStream_t);
 template cudaError_t launch_convert<double, float>(size_t, const double*, float*, cudaStream_t);
 template cudaError_t launch_speed<float>(int, const ReduceArgs<float>&, cudaStream_t);
@@ -331,7 +338,7 @@ template cudaError_t launch_speed<double>(int, const ReduceArgs<double>&, cudaSt
 template cudaError_t launch_totals<float>(int, const ReduceArgs<float>&, cudaStream_t);
 template cudaError_t launch_totals<double>(int, const ReduceArgs<double>&, cudaStream_t);
 template cudaError_t launch_init_from_primitive<dw>(int, size_t, double, const double*, const double*, const double*,
-                                                    dw*, cudaStream_t);
+                                                    dw*, double*, cudaStream_t);
 template cudaError_t launch_convert<double, dw>(size_t, const double*, dw*, cudaStream_t);
 template cudaError_t launch_convert<float, dw>(size_t, const float*, dw*, cudaStream_t);
 template cudaError_t launch_convert<dw, double>(size_t, const dw*, double*, cudaStream_t);

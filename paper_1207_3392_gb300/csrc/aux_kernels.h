@@ -77,7 +77,7 @@ cudaError_t launch_shock_flags_tma(const FlagArgs<float>& A, const CUtensorMap& 
 
 template <class T>
 cudaError_t launch_init_from_primitive(int ndim, size_t ncell, double gamma, const double* rho, const double* vel,
-                                       const double* p, T* U, cudaStream_t s);
+                                       const double* p, T* U, double* t, cudaStream_t s);
 template <class Tin, class Tout>
 cudaError_t launch_convert(size_t count, const Tin* in, Tout* out, cudaStream_t s);
 template <class T>

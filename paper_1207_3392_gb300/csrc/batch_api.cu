@@ -440,18 +440,17 @@ int genasis_batch_set_primitive(genasis_batch_t b, int iprob, const double* rho,
     cudaError_t e =
         b->prec == GENASIS_FP64
             ? launch_init_from_primitive<double>(h.ndim, h.ncell, h.gamma, use[0], use[1], use[2],
-                                                 (double*)b->U[b->cur] + h.off, b->stream)
+                                                 (double*)b->U[b->cur] + h.off, b->t + iprob, b->stream)
         : b->prec == GENASIS_FP32_MIXED
             ? launch_init_from_primitive<float>(h.ndim, h.ncell, h.gamma, use[0], use[1], use[2],
-                                                (float*)b->U[b->cur] + h.off, b->stream)
+                                                (float*)b->U[b->cur] + h.off, b->t + iprob, b->stream)
             : launch_init_from_primitive<dw>(h.ndim, h.ncell, h.gamma, use[0], use[1], use[2], (dw*)b->U[b->cur] + h.off,
-                                             b->stream);
+                                             b->t + iprob, b->stream);
     if (e != cudaSuccess) rc = fail(GENASIS_ECUDA, "init kernel: %s", cudaGetErrorString(e));
   }
   for (int a = 0; a < 3; ++a)
     if (tmp[a]) cudaFreeAsync(tmp[a], b->stream);
   if (rc) return rc;
-  GH_CK(cudaMemsetAsync(b->t + iprob, 0, sizeof(double), b->stream));
   if (host) GH_CK(cudaStreamSynchronize(b->stream));
   return GENASIS_OK;
 }

@@ -1094,13 +1094,12 @@ int genasis_learned_set_primitive(genasis_learned_t l, const double* rho, const 
   }
   if (!rc) {
     cudaError_t e = launch_init_from_primitive<float>(2, l->ncell, (double)l->M.gamma, use[0], use[1], use[2],
-                                                      (float*)l->U[l->cur], l->stream);
+                                                      (float*)l->U[l->cur], l->scal + SCAL_T, l->stream);
     if (e != cudaSuccess) rc = fail(GENASIS_ECUDA, "init kernel: %s", cudaGetErrorString(e));
   }
   for (int a = 0; a < 3; ++a)
     if (tmp[a]) cudaFreeAsync(tmp[a], l->stream);
   if (rc) return rc;
-  GH_CK(cudaMemsetAsync(l->scal + SCAL_T, 0, sizeof(double), l->stream));
   GH_CK(cudaStreamSynchronize(l->stream));
   return GENASIS_OK;
 }
