@@ -96,16 +96,31 @@ __device__ __forceinline__ void ring_cell(unsigned t, unsigned np, unsigned N, i
 
 // ---------------------------------------------------------------- transfers
 
+// A level's provisional forward-Euler state at its child's time, U + (t_child -
+// t_level) K, formed where it is read (the child's ring and the level's speed):
+// it is never stored, and the level's own buffers stay as they are.
+template <class T, bool PROV>
+struct CoarseState {
+  const T* U;
+  const T* K;
+  T dt;
+  __device__ __forceinline__ CoarseState(const T* u, const T* k, const double* ltime, int level)
+      : U(u), K(k), dt(PROV ? (T)(ltime[level + 1] - ltime[level]) : T(0)) {}
+  __device__ __forceinline__ T operator()(size_t c) const { return PROV ? fma_rn(dt, K[c], U[c]) : U[c]; }
+};
+
 // Exterior ring of fine level from the coarse level: child = coarse value +
 // minmod-limited conserved slopes x (-+ h_c / 4) per axis (added in axis order).
-template <class T, int NDIM>
-__global__ void fmr_prolong_kernel(const T* __restrict__ Uc, LevelGeo gc, T* __restrict__ Uf, LevelGeo gf) {
+template <class T, int NDIM, bool PROV>
+__global__ void fmr_prolong_kernel(const T* __restrict__ Uc, const T* __restrict__ Kc, const double* ltime, int coarse,
+                                   LevelGeo gc, T* __restrict__ Uf, LevelGeo gf) {
   constexpr int NV = NDIM + 2;
   const unsigned np = gf.npad;
   const int N = gf.N;
   const unsigned nf = np * (NDIM > 1 ? np : 1) * (NDIM > 2 ? np : 1);  // < 2^31 (n <= 1024)
   const size_t vsc = (size_t)gc.npad * (NDIM > 1 ? gc.npad : 1) * (NDIM > 2 ? gc.npad : 1);
   chain_wait();
+  const CoarseState<T, PROV> S(Uc, Kc, ltime, coarse);
   const unsigned cells = ring_count(NDIM, np, N);
   for (unsigned r = blockIdx.x * blockDim.x + threadIdx.x; r < cells; r += gridDim.x * blockDim.x) {
     int p[3];
@@ -115,14 +130,14 @@ __global__ void fmr_prolong_kernel(const T* __restrict__ Uc, LevelGeo gc, T* __r
     for (int q = 0; q < NDIM; ++q) c[q] = N / 4 + p[q] / 2 - 1 + gc.off;  // coarse stored index
     const size_t cc = lin(NDIM, gc.npad, c[0], c[1], c[2]);
     for (int v = 0; v < NV; ++v) {
-      const T u = Uc[v * vsc + cc];
+      const T u = S(v * vsc + cc);
       T out = u;
       for (int q = 0; q < NDIM; ++q) {
         int cm[3] = {c[0], c[1], c[2]}, cp[3] = {c[0], c[1], c[2]};
         cm[q] -= 1;
         cp[q] += 1;
-        const T um = Uc[v * vsc + lin(NDIM, gc.npad, cm[0], cm[1], cm[2])];
-        const T up = Uc[v * vsc + lin(NDIM, gc.npad, cp[0], cp[1], cp[2])];
+        const T um = S(v * vsc + lin(NDIM, gc.npad, cm[0], cm[1], cm[2]));
+        const T up = S(v * vsc + lin(NDIM, gc.npad, cp[0], cp[1], cp[2]));
         // minmod of the one-sided differences times the child offset (-+1/4 of a coarse cell)
         const T dm = u - um, dp = up - u;
         const T s = dm * dp > T(0) ? (fabs(dm) < fabs(dp) ? dm : dp) : T(0);
@@ -192,22 +207,14 @@ __global__ void fmr_ring_zero_kernel(T* __restrict__ K, LevelGeo g) {
   }
 }
 
-// Provisional coarse substep: out = U + (t_child - t_coarse) K (forward Euler).
-template <class T>
-__global__ void fmr_euler_kernel(const T* __restrict__ U, const T* __restrict__ K, T* __restrict__ out, size_t count,
-                                 const double* ltime, int child, int coarse) {
-  chain_wait();
-  const T dt = (T)(ltime[child] - ltime[coarse]);
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < count; t += (size_t)gridDim.x * blockDim.x)
-    out[t] = U[t] + dt * K[t];
-}
-
 // Per-block max over the interior of max_q (|v_q| + c_s).
-template <class T, int NDIM>
-__global__ void fmr_speed_kernel(const T* __restrict__ U, LevelGeo g, double gamma, double* __restrict__ part) {
+template <class T, int NDIM, bool PROV>
+__global__ void fmr_speed_kernel(const T* __restrict__ U, const T* __restrict__ K, const double* ltime, int level,
+                                 LevelGeo g, double gamma, double* __restrict__ part) {
   constexpr int NV = NDIM + 2;
   __shared__ double red[32];
   chain_wait();
+  const CoarseState<T, PROV> S(U, K, ltime, level);
   const unsigned N = g.N, np = g.npad;
   const unsigned ni = N * (NDIM > 1 ? N : 1) * (NDIM > 2 ? N : 1);
   const size_t vs = (size_t)np * (NDIM > 1 ? np : 1) * (NDIM > 2 ? np : 1);
@@ -218,7 +225,7 @@ __global__ void fmr_speed_kernel(const T* __restrict__ U, LevelGeo g, double gam
               k = NDIM > 2 ? (int)(t1 / N) + g.off : 0;
     const size_t c = lin(NDIM, np, i, j, k);
     T u[NV], w[NV];
-    for (int v = 0; v < NV; ++v) u[v] = U[v * vs + c];
+    for (int v = 0; v < NV; ++v) u[v] = S(v * vs + c);
     recover<NDIM>(u, w);
     const T cs = sound_speed((T)gamma, (T)(gamma - 1.0) * w[NV - 1], w[0]);
     for (int q = 0; q < NDIM; ++q) best = fmax(best, fabs(w[1 + q]) + cs);
@@ -280,9 +287,77 @@ __global__ void fmr_sync_times_kernel(double* ltime, int L) {
     for (int l = 1; l < L; ++l) ltime[l] = ltime[0];
 }
 
-// Heun-effective face flux (F(U^n) + F(U^n + dt K)) / 2 through the face of
+// K of the interior cells whose stencils reach the exterior ring (the two
+// outermost layers): a level with a child has K of its state already, from the
+// provisional substep, but with the ring of that time; nothing else it depends on
+// has changed when the level takes its own first stage.  One thread per cell with
+// its 13-cell stencil, the stage kernels' operations in their order (the values
+// are theirs bit for bit).  9% of the cells of a 128^3 level: about 13 us in place
+// of a whole first stage's 80.
+template <class T, int NDIM, int Q, int SOLVER>
+__device__ __forceinline__ void shell_axis(const StageArgs<T>& A, const T* __restrict__ U, size_t c, int i, size_t vs,
+                                           const T (&w)[NDIM + 2], T (&L)[NDIM + 2]) {
+  constexpr int NV = NDIM + 2;
+  const size_t st = Q == 0 ? 1 : Q == 1 ? (size_t)A.n[0] : (size_t)A.n[0] * A.n[1];
+  const Geo<T> gm = A.geo[Q][i + 1], g = A.geo[Q][i + 2], gp = A.geo[Q][i + 3];
+  auto prim = [&](size_t cc, T (&o)[NV]) {
+    T u[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) u[v] = U[v * vs + cc];
+    recover<NDIM>(u, o);
+  };
+  T wa[NV], wb[NV], wl[NV], wr[NV], lo[NV], hi[NV], up[NV];
+  prim(c - 2 * st, wa);
+  prim(c - st, wb);
+  T wc[NV], wd[NV];
+  prim(c + st, wc);
+  prim(c + 2 * st, wd);
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    wl[v] = face_hi(limited_slope(wa[v], wb[v], w[v], gm), gm.h, wb[v]);
+    face_pair(limited_slope(wb[v], w[v], wc[v], g), g.h, w[v], wr[v], up[v]);
+  }
+  face_flux<T, NDIM, Q, SOLVER>(wl, wr, A.gamma, A.gm1, lo);
+#pragma unroll
+  for (int v = 0; v < NV; ++v) wr[v] = face_lo(limited_slope(w[v], wc[v], wd[v], gp), gp.h, wc[v]);
+  face_flux<T, NDIM, Q, SOLVER>(up, wr, A.gamma, A.gm1, hi);
+  const T iw = A.iw[Q][i + 2];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    const T d = sub_rn(lo[v], hi[v]);
+    L[v] = Q == 0 ? mul_rn(d, iw) : fma_rn(d, iw, L[v]);
+  }
+}
+
+template <class T, int NDIM, int SOLVER>
+__global__ void __launch_bounds__(128) fmr_shell_kernel(StageArgs<T> A, const T* __restrict__ U, T* __restrict__ K,
+                                                        LevelGeo g) {
+  constexpr int NV = NDIM + 2;
+  chain_wait();
+  const unsigned N = g.N, inner = N - 2 * FNG, cells = ring_count(NDIM, N, inner);
+  const size_t vs = (size_t)A.n[0] * A.n[1] * A.n[2];
+  for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < cells; t += gridDim.x * blockDim.x) {
+    int p[3] = {0, 0, 0};
+    ring_cell<NDIM>(t, N, inner, p);
+    for (int q = 0; q < NDIM; ++q) p[q] += g.off;
+    const size_t c = lin(NDIM, g.npad, p[0], p[1], p[2]);
+    T u[NV], w[NV], L[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) u[v] = U[v * vs + c];
+    recover<NDIM>(u, w);
+    shell_axis<T, NDIM, 0, SOLVER>(A, U, c, p[0], vs, w, L);
+    shell_axis<T, NDIM, 1, SOLVER>(A, U, c, p[1], vs, w, L);
+    if constexpr (NDIM == 3) shell_axis<T, NDIM, 2, SOLVER>(A, U, c, p[2], vs, w, L);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) K[v * vs + c] = L[v];
+  }
+}
+
+// Twice the Heun-effective face flux, F(U^n) + F(U^n + dt K), through the face of
 // axis Q between stored cells c - e_Q and c (same reconstruction and Riemann
-// solver as the stage kernels, with the handle's geometry tables).
+// solver as the stage kernels, with the handle's geometry tables).  The factors
+// of two of this sum and of the means over fine faces are exact, so they are left
+// to the last product: FP64 operations are what the face kernels have most of.
 template <class T, int NDIM, int Q, int SOLVER>
 __device__ void face_eff(const StageArgs<T>& A, const T* U0, const T* K, T dt, int i, int j, int k, size_t vs,
                          double (&Fe)[NDIM + 2]) {
@@ -309,7 +384,7 @@ __device__ void face_eff(const StageArgs<T>& A, const T* U0, const T* K, T dt, i
       wr[v] = fma(-limited_slope(w[1][v], w[2][v], w[3][v], gr), gr.h, w[2][v]);
     }
     face_flux<T, NDIM, Q, SOLVER>(wl, wr, A.gamma, A.gm1, f);
-    for (int v = 0; v < NV; ++v) Fe[v] = s ? 0.5 * (Fe[v] + (double)f[v]) : (double)f[v];
+    for (int v = 0; v < NV; ++v) Fe[v] = s ? Fe[v] + (double)f[v] : (double)f[v];
   }
 }
 
@@ -331,17 +406,21 @@ __host__ __device__ inline size_t cf_index(int nd, int M, int q, int side, int v
   return (((size_t)q * 2 + side) * (nd + 2) + v) * per + tr;
 }
 
-// This level as parent: Heun-effective fluxes through the faces of its child's
-// box, one thread per coarse face -> fc.
+// This level as parent: flux replacement on the uncovered coarse cells next to
+// the child's box, U += sign (dt F_coarse - Phi) / h, sign +1 below the box, -1
+// above, with the Heun-effective flux of the coarse face.  One thread per coarse
+// face (a cell next to the box has one face on it, so no cell is written twice).
 template <class T, int NDIM, int SOLVER>
-__global__ void fmr_parent_faces_kernel(StageArgs<T> A, const T* __restrict__ U0, const T* __restrict__ K,
-                                        LevelGeo g, double* __restrict__ fc) {
+__global__ void __launch_bounds__(64) fmr_replace_kernel(StageArgs<T> A, const T* __restrict__ U0,
+                                                         const T* __restrict__ K, T* __restrict__ U, LevelGeo g,
+                                                         const double* __restrict__ phi, double h) {
   constexpr int NV = NDIM + 2;
   const int M = g.N / 2;
   const int per = NDIM == 1 ? 1 : NDIM == 2 ? M : M * M;
   const size_t vs = (size_t)A.n[0] * A.n[1] * A.n[2];
   chain_wait();
-  const T dt = (T)(*A.dt);
+  const double dtd = *A.dt;
+  const T dt = (T)dtd;
   const int total = NDIM * 2 * per;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
     const int tr = t % per, side = (t / per) % 2, q = t / (2 * per);
@@ -355,7 +434,13 @@ __global__ void fmr_parent_faces_kernel(StageArgs<T> A, const T* __restrict__ U0
     c[q] = g.off + (side == 0 ? g.N / 4 : 3 * g.N / 4);  // face between cells c - e_q and c
     double Fe[NV];
     face_eff_q<T, NDIM, SOLVER>(q, A, U0, K, dt, c[0], c[1], c[2], vs, Fe);
-    for (int v = 0; v < NV; ++v) fc[cf_index(NDIM, M, q, side, v, tr)] = Fe[v];
+    if (side == 0) c[q] -= 1;
+    const double sign = side == 0 ? 1.0 : -1.0, hdt = 0.5 * dtd;
+    const size_t cc = lin(NDIM, g.npad, c[0], c[1], c[2]);
+    for (int v = 0; v < NV; ++v) {
+      const double d = hdt * Fe[v] - phi[cf_index(NDIM, M, q, side, v, tr)];
+      U[v * vs + cc] = (T)((double)U[v * vs + cc] + sign * d / h);
+    }
   }
 }
 
@@ -402,46 +487,16 @@ __global__ void __launch_bounds__(128) fmr_child_faces_kernel(StageArgs<T> A, co
     face_eff_q<T, NDIM, SOLVER>(q, A, U0, K, dt, c[0], c[1], c[2], vs, m);
   }
   if constexpr (NDIM == 3) {
-    for (int v = 0; v < NV; ++v) m[v] = (m[v] + __shfl_xor_sync(0xffffffffu, m[v], 2)) / 2.0;  // slower axis
+    for (int v = 0; v < NV; ++v) m[v] = m[v] + __shfl_xor_sync(0xffffffffu, m[v], 2);  // slower axis
   }
   if constexpr (NDIM >= 2) {
-    for (int v = 0; v < NV; ++v) m[v] = (m[v] + __shfl_xor_sync(0xffffffffu, m[v], 1)) / 2.0;  // faster axis
+    for (int v = 0; v < NV; ++v) m[v] = m[v] + __shfl_xor_sync(0xffffffffu, m[v], 1);  // faster axis
   }
   if (act && sub == 0) {
+    const double share = dtd / (double)(2 * G);  // exact: m sums two fluxes of each of G faces
     for (int v = 0; v < NV; ++v) {
       const size_t o = cf_index(NDIM, M, q, side, v, tr);
-      acc[o] = acc[o] + dtd * m[v];
-    }
-  }
-}
-
-// Flux replacement on the uncovered coarse cells next to the child's box:
-// U += sign (dt F_coarse - Phi) / h, sign +1 below the box, -1 above.
-template <class T, int NDIM>
-__global__ void fmr_replace_kernel(T* __restrict__ U, LevelGeo g, const double* __restrict__ fc,
-                                   const double* __restrict__ phi, const double* __restrict__ dtp, double h) {
-  constexpr int NV = NDIM + 2;
-  const int M = g.N / 2;
-  const int per = NDIM == 1 ? 1 : NDIM == 2 ? M : M * M;
-  const size_t vs = (size_t)g.npad * (NDIM > 1 ? g.npad : 1) * (NDIM > 2 ? g.npad : 1);
-  chain_wait();
-  const double dt = *dtp;
-  const int total = NDIM * 2 * per;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
-    const int tr = t % per, side = (t / per) % 2, q = t / (2 * per);
-    int c[3] = {0, 0, 0};
-    int r0 = tr;
-    for (int r = 0; r < NDIM; ++r) {
-      if (r == q) continue;
-      c[r] = g.off + g.N / 4 + r0 % M;
-      r0 /= M;
-    }
-    c[q] = g.off + (side == 0 ? g.N / 4 - 1 : 3 * g.N / 4);
-    const double sign = side == 0 ? 1.0 : -1.0;
-    const size_t cc = lin(NDIM, g.npad, c[0], c[1], c[2]);
-    for (int v = 0; v < NV; ++v) {
-      const size_t o = cf_index(NDIM, M, q, side, v, tr);
-      U[v * vs + cc] = (T)((double)U[v * vs + cc] + sign * (dt * fc[o] - phi[o]) / h);
+      acc[o] = acc[o] + share * m[v];
     }
   }
 }
@@ -464,9 +519,7 @@ struct genasis_fmr {
   std::vector<genasis_hydro_t> lev;
   std::vector<LevelGeo> geo;
   std::vector<double> hcell;
-  std::vector<void*> save;
   std::vector<double*> acc;  // acc[l]: Phi accumulated by level l (>= 1) for its parent
-  std::vector<double*> fc;   // fc[l]: level l's fluxes through its child's box
   size_t cf_count = 0;       // doubles per face array
   int nblk = 0;
   double* part = nullptr;    // [L][nblk]
@@ -508,28 +561,41 @@ struct FmrRun {
   }
 
   static int evolve_level(genasis_fmr* f, int i, double* acc, double cfl) {
-    int rc = step_level(f, i, acc, cfl);
+    int rc = step_level(f, i, acc, cfl, false);
     if (rc || i == 0) return rc;
     genasis_hydro* c = f->lev[i - 1];
-    cudaStream_t st = f->stream;
     // provisional coarse substep (forward Euler by the child's first step), ring
-    // held: into the level's third buffer, which stands in for its state while
-    // the child takes its second step (nothing below writes level i - 1)
-    rc = launch_stage(c, 1, st);
+    // held: only K is stored, the child's ring and this speed form the state
+    rc = launch_stage(c, 1, f->stream);
     if (rc) return rc;
     if (i - 1 >= 1 && (rc = ring_zero(f, i - 1))) return rc;
-    GH_CK(chain(st, &fmr_euler_kernel<T>, grid_of(c->ncell * c->nv), 256, (const T*)c->U[c->cur], (const T*)c->K,
-                (T*)f->save[i - 1], c->ncell * c->nv, (const double*)f->ltime, i, i - 1));
-    std::swap(c->U[c->cur], f->save[i - 1]);
-    f->dirty[i - 1] = 1;
-    rc = step_level(f, i, acc, cfl);
-    std::swap(c->U[c->cur], f->save[i - 1]);
-    if (rc) return rc;
-    f->dirty[i - 1] = 1;
+    if ((rc = speed<true>(f, i - 1))) return rc;
+    if ((rc = step_level(f, i, acc, cfl, true))) return rc;
+    f->dirty[i - 1] = 1;  // its state is U again
     return GENASIS_OK;
   }
 
-  static int step_level(genasis_fmr* f, int i, double* acc, double cfl) {
+  // speed partials of a level's interior
+  template <bool PROV>
+  static int speed(genasis_fmr* f, int l) {
+    genasis_hydro* g = f->lev[l];
+    GH_CK(chain(f->stream, &fmr_speed_kernel<T, NDIM, PROV>, f->nblk, 256, (const T*)g->U[g->cur], (const T*)g->K,
+                (const double*)f->ltime, l, f->geo[l], f->gamma, f->part + (size_t)l * f->nblk));
+    f->dirty[l] = 0;
+    return GENASIS_OK;
+  }
+
+  template <bool PROV>
+  static int prolong(genasis_fmr* f, int i) {
+    genasis_hydro *h = f->lev[i], *c = f->lev[i - 1];
+    GH_CK(chain(f->stream, &fmr_prolong_kernel<T, NDIM, PROV>,
+                grid_of(ring_count(NDIM, f->geo[i].npad, f->geo[i].N)), 256, (const T*)c->U[c->cur], (const T*)c->K,
+                (const double*)f->ltime, i - 1, f->geo[i - 1], (T*)h->U[h->cur], f->geo[i]));
+    return GENASIS_OK;
+  }
+
+  // A step of level i, its parent's state provisional or not
+  static int step_level(genasis_fmr* f, int i, double* acc, double cfl, bool provisional) {
     genasis_hydro* h = f->lev[i];
     cudaStream_t st = f->stream;
     const int L = f->L;
@@ -538,20 +604,11 @@ struct FmrRun {
       GH_CK(cudaMemsetAsync(f->acc[i + 1], 0, f->cf_count * sizeof(double), st));
       if ((rc = evolve_level(f, i + 1, f->acc[i + 1], cfl))) return rc;
     }
-    if (i > 0) {
-      genasis_hydro* c = f->lev[i - 1];
-      GH_CK(chain(st, &fmr_prolong_kernel<T, NDIM>, grid_of(ring_count(NDIM, f->geo[i].npad, f->geo[i].N)), 256,
-                  (const T*)c->U[c->cur], f->geo[i - 1], (T*)h->U[h->cur], f->geo[i]));
-    }
+    if (i > 0 && (rc = provisional ? prolong<true>(f, i) : prolong<false>(f, i))) return rc;
     if (i == L - 1) {
       // speed partials of every level whose interior changed since they were taken
-      for (int l = 0; l < L; ++l) {
-        if (!f->dirty[l]) continue;
-        genasis_hydro* g = f->lev[l];
-        GH_CK(chain(st, &fmr_speed_kernel<T, NDIM>, f->nblk, 256, (const T*)g->U[g->cur], f->geo[l], f->gamma,
-                    f->part + (size_t)l * f->nblk));
-        f->dirty[l] = 0;
-      }
+      for (int l = 0; l < L; ++l)
+        if (f->dirty[l] && (rc = speed<false>(f, l))) return rc;
     }
     DtArgs D;
     D.L = L;
@@ -564,19 +621,24 @@ struct FmrRun {
     D.ldt = f->ldt;
     D.scal_dt = h->scal + SCAL_DT;
     GH_CK(chain(st, &fmr_dt_kernel, 1, 32 * L, D));
-    // the two RK stages with the exterior ring held
-    if ((rc = launch_stage(h, 1, st))) return rc;
-    if (i >= 1 && (rc = ring_zero(f, i))) return rc;
+    // the two RK stages with the exterior ring held; with a child, K is there from
+    // the provisional substep but for the cells next to the ring
+    const StageArgs<T> A = stage_args<T>(h, 1);  // geometry, gamma and the dt slot of this level
+    const T* U0 = (const T*)h->U[h->cur];
+    if (i + 1 == L) {
+      if ((rc = launch_stage(h, 1, st))) return rc;
+      if (i >= 1 && (rc = ring_zero(f, i))) return rc;
+    } else if (i >= 1) {
+      const size_t cells = ring_count(NDIM, f->geo[i].N, f->geo[i].N - 2 * FNG);
+      GH_CK(chain(st, &fmr_shell_kernel<T, NDIM, SOLVER>, (int)((cells + 127) / 128), 128, A, U0, (T*)h->K, f->geo[i]));
+    }
     if ((rc = launch_stage(h, 2, st))) return rc;
     h->cur = 1 - h->cur;
     f->dirty[i] = 1;
-    StageArgs<T> A = stage_args<T>(h, 1);  // geometry, gamma and the dt slot of this level
-    const T* U0 = (const T*)h->U[1 - h->cur];
-    const int nfc = grid_of(f->cf_count / (NDIM + 2));
     if (i + 1 < L) {
-      GH_CK(chain(st, &fmr_parent_faces_kernel<T, NDIM, SOLVER>, nfc, 128, A, U0, (const T*)h->K, f->geo[i], f->fc[i]));
-      GH_CK(chain(st, &fmr_replace_kernel<T, NDIM>, nfc, 128, (T*)h->U[h->cur], f->geo[i], (const double*)f->fc[i],
-                  (const double*)f->acc[i + 1], (const double*)f->ldt + i, f->hcell[i]));
+      const int faces = (int)(f->cf_count / (NDIM + 2));
+      GH_CK(chain(st, &fmr_replace_kernel<T, NDIM, SOLVER>, (faces + 63) / 64, 64, A, U0, (const T*)h->K,
+                  (T*)h->U[h->cur], f->geo[i], (const double*)f->acc[i + 1], f->hcell[i]));
       genasis_hydro* c = f->lev[i + 1];
       GH_CK(chain(st, &fmr_restrict_kernel<T, NDIM>, grid_of(h->ncell), 256, (const T*)c->U[c->cur], f->geo[i + 1],
                   (T*)h->U[h->cur], f->geo[i]));
@@ -612,9 +674,7 @@ void fmr_free(genasis_fmr* f) {
   if (f->stream) cudaStreamSynchronize(f->stream);
   if (f->graph) cudaGraphExecDestroy(f->graph);
   for (auto h : f->lev) genasis_hydro_destroy(h);
-  for (auto p : f->save) cudaFree(p);
   for (auto p : f->acc) cudaFree(p);
-  for (auto p : f->fc) cudaFree(p);
   cudaFree(f->part);
   cudaFree(f->d_hcell);
   cudaFree(f->ltime);
@@ -692,15 +752,9 @@ int genasis_fmr_create(const genasis_fmr_desc* d, genasis_fmr_t* out) {
   f->nblk = 1024;
   bool ok = true;
   for (int l = 0; l < f->L && ok; ++l) {
-    void* s = nullptr;
     double* a = nullptr;
-    double* c = nullptr;
-    ok &= cudaMalloc(&s, f->lev[l]->ncell * f->lev[l]->nv * f->lev[l]->esize) == cudaSuccess;
     ok &= cudaMalloc((void**)&a, f->cf_count * sizeof(double)) == cudaSuccess;
-    ok &= cudaMalloc((void**)&c, f->cf_count * sizeof(double)) == cudaSuccess;
-    f->save.push_back(s);
     f->acc.push_back(a);
-    f->fc.push_back(c);
   }
   ok &= cudaMalloc((void**)&f->part, (size_t)f->L * f->nblk * sizeof(double)) == cudaSuccess;
   ok &= cudaMalloc((void**)&f->d_hcell, f->L * sizeof(double)) == cudaSuccess;
