@@ -362,18 +362,27 @@ template <class T, int NDIM, int Q, int SOLVER>
 __device__ void face_eff(const StageArgs<T>& A, const T* U0, const T* K, T dt, int i, int j, int k, size_t vs,
                          double (&Fe)[NDIM + 2]) {
   constexpr int NV = NDIM + 2;
-  T w[4][NV];
+  T w[4][NV], u0[4][NV], kk[4][NV];
+  // both states' loads are in flight together (one state after the other: the
+  // child's faces of a 128^3 level 24 us, so 17)
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    int c[3] = {i, j, k};
+    c[Q] += a - 2;
+    const size_t cc = lin(NDIM, A.n[0], c[0], c[1], c[2]);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      u0[a][v] = U0[v * vs + cc];
+      kk[a][v] = K[v * vs + cc];
+    }
+  }
+#pragma unroll
   for (int s = 0; s < 2; ++s) {
+#pragma unroll
     for (int a = 0; a < 4; ++a) {
-      int c[3] = {i, j, k};
-      c[Q] += a - 2;
-      const size_t cc = lin(NDIM, A.n[0], c[0], c[1], c[2]);
       T u[NV];
-      for (int v = 0; v < NV; ++v) {
-        T x = U0[v * vs + cc];
-        if (s) x = fma(dt, K[v * vs + cc], x);
-        u[v] = x;
-      }
+#pragma unroll
+      for (int v = 0; v < NV; ++v) u[v] = s ? fma(dt, kk[a][v], u0[a][v]) : u0[a][v];
       recover<NDIM>(u, w[a]);
     }
     const int cq = (Q == 0 ? i : Q == 1 ? j : k);
