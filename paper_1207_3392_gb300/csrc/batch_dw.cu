@@ -1,31 +1,13 @@
-// batch_dw.cu -- persistent batch-kernel instantiations (double-word state, dword.cuh).
-#include "batch_kernel.cuh"
-#include "batch_registry.h"
+// batch_dw.cu -- persistent batch-kernel instantiations (double-word state, dword.cuh): warps on
+// their own strips (batch_strip.cuh), 4 or 8 of them per CTA.
+#include "batch_strip.cuh"
 
 namespace gh {
 
-template <int SOLVER, int STAGE, int TX>
-static void fill(BatchVariant* out) {
-  out->fn = reinterpret_cast<const void*>(&hydro_batch_kernel<dw, SOLVER, STAGE, TX>);
-  out->smem = BatchKernel<dw, SOLVER, STAGE, TX>::SMEM;
-  out->tx = TX;
-  out->cols = BatchKernel<dw, SOLVER, STAGE, TX>::K2::OWN;
-}
-
-template <int TX>
-static bool pick(int solver, int stage, BatchVariant* out) {
-  if (solver == SOLVER_HLL && stage == 1) fill<SOLVER_HLL, 1, TX>(out);
-  else if (solver == SOLVER_HLL && stage == 2) fill<SOLVER_HLL, 2, TX>(out);
-  else if (solver == SOLVER_HLLC && stage == 1) fill<SOLVER_HLLC, 1, TX>(out);
-  else if (solver == SOLVER_HLLC && stage == 2) fill<SOLVER_HLLC, 2, TX>(out);
-  else return false;
-  return true;
-}
-
 bool batch_variant_dw(int solver, int stage, int tile, BatchVariant* out) {
   switch (tile) {
-    case 0: return pick<128>(solver, stage, out);
-    case 1: return pick<256>(solver, stage, out);
+    case 0: return pick_batch_strip<dw, 4>(solver, stage, out);
+    case 1: return pick_batch_strip<dw, 8>(solver, stage, out);
   }
   return false;
 }

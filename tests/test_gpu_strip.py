@@ -1,4 +1,4 @@
-"""The 2D FP32 strips (one warp per 28 columns) and the FP32 batch built on them,
+"""The 2D FP32 strips (one warp per 28 columns) and the FP32 and double-word batches built on them,
 against the oracle at the sizes where a strip can go wrong: meshes narrower than
 a strip, its edges and remainders, chunks of rows and their remainders, every
 boundary rule, groups of 1D strips; and one mesh of more than 2^30 cells (64-bit
@@ -47,18 +47,19 @@ def test_strip_edges_match_the_oracle(n, bc):
                 np.testing.assert_allclose(tot, ref_tot, rtol=1e-12, atol=1e-12 * np.max(np.abs(ref_tot)))
 
 
-def test_batch_of_edge_sizes_matches_the_oracle():
+@pytest.mark.parametrize("precision,tol", [(H.FP32_MIXED, TOL_FP32), (H.FP64_DW, TOL_FP64)])
+def test_batch_of_edge_sizes_matches_the_oracle(precision, tol):
     probs = [P.random_blocks(1, (m,), seed=m, bc=bc) for m in (2, 27, 28, 29, 223, 224, 225, 449)
              for bc in (P.PERIODIC, P.REFLECT, P.OUTFLOW)]
     probs += [P.random_blocks(2, m, seed=m[0], bc=P.REFLECT) for m in ((2, 2), (28, 31), (29, 33), (57, 65))]
-    b = H.Batch(probs, precision=H.FP32_MIXED)
+    b = H.Batch(probs, precision=precision)
     for i, pr in enumerate(probs):
         b.set_primitive(i, pr.rho, pr.vel, pr.p)
     b.run(4, 0.4)
     assert b.status() == -1
     for i, pr in enumerate(probs):
         Uo, _ = oracle_run(pr.with_(cfl=0.4), steps=4)
-        check(b.get_conserved(i), Uo, pr.ndim, TOL_FP32, f"problem {i} {pr.n}")
+        check(b.get_conserved(i), Uo, pr.ndim, tol, f"problem {i} {pr.n}")
     b.close()
 
 
