@@ -73,7 +73,7 @@ def _config(args, n):
             "cells": n ** 3, "domain": "[-1,1]^3", "gamma": 1.4, "bc": "reflecting",
             "solver": args.solver.upper(),
             "precision": PRECISION_LABEL[args.precision],
-            "cfl": 0.3, "step": "one TVD-RK2 step: 2 stage kernels + dt/totals finalize",
+            "cfl": 0.3, "step": "one TVD-RK2 step: 2 stages + dt/totals finalize",
             "l2": f"inputs larger than L2 (state {n**3 * 5 * (4 if args.precision == 'fp32' else 8) / 1e6:.0f} MB)",
             "parallelism": "replicas" if args.gpus > 1 else "single GPU"}
 
@@ -152,16 +152,21 @@ FLOPS_STAGE1_3D = {"hllc": 744, "hll": 720}
 FLOPS_STEP_3D = {"hllc": 1469, "hll": 1421}
 FLOPS_STAGE1_3D["hllc_switch"] = FLOPS_STAGE1_3D["hllc"]  # away from shocks; the detector is not counted
 FLOPS_STEP_3D["hllc_switch"] = FLOPS_STEP_3D["hllc"]
-# DRAM bytes (read + write) per launch of the FP32 HLLC 3D stage kernels at
-# 256^3, from one ncu capture of the bench's own launch configuration (tile
-# 8, 40 planes per CTA; profiles/stage_fp32_hllc_sedov256_ncu.md).  Other
-# configurations, precisions and sizes report no traffic.
+# DRAM bytes (read + write) per stage of the FP32 HLLC 3D kernels at 256^3, from
+# ncu captures: tile 8, 40 planes per CTA (profiles/stage_fp32_hllc_sedov256_ncu.md);
+# tile 14, 48 planes, the strips along x and y and the march along z together
+# (profiles/split_and_strip_counters.md).  Other configurations, precisions and
+# sizes report no traffic.
 TRAFFIC_FP32_HLLC_256 = {
     (8, 40): {"stage1": 356.859136e6 + 300.052480e6, "stage2": 732.600576e6 + 312.649472e6},
+    (14, 48): {"stage1": 340.713216e6 + 291.104512e6 + 697.400832e6 + 290.496512e6,
+               "stage2": 686.102528e6 + 306.223104e6 + 1059.129856e6 + 303.567104e6},
 }
+# 3D tiles that run a stage as two launches (strips along x and y, march along z)
+SPLIT_TILE_3D = {"float": 14, "dw": 4}
 PRECISION_LABEL = {
     "fp32": ("FP32 storage, FP32 fluxes and FP32 per-cell CFL speeds; the internal-energy recovery "
-             "e = G - |S|^2/(2D) in FP64 only where the kinetic energy exceeds half of G; per-column "
+             "e = G - |S|^2/(2D) from error-compensated FP32 products; per-column "
              "conserved totals as compensated FP32 pairs; the dt and totals reductions across threads "
              "and CTAs in FP64"),
     "fp64": "FP64 throughout",
@@ -314,7 +319,9 @@ def _stage_roofline(args, prec, cells, tile, st1, fin, st2):
     achieved_f = flops_cell * cells / (dom_ms * 1e-3) / 1e12
     peak_f = _PEAKS.get(fkey)
     tname = {H.FP32_MIXED: "float", H.FP64: "double", H.FP64_DW: "dw"}[prec]
-    return {"bound": "hbm", "kernel": f"hydro_stage_kernel<3,{tname},{args.solver.upper()},{dom[-1]}>",
+    split = SPLIT_TILE_3D.get(tname) == tile["tile"]
+    names = ("hydro_strip_xy_kernel", "hydro_march_z_kernel") if split else ("hydro_stage_kernel",)
+    return {"bound": "hbm", "kernel": " + ".join(f"{k}<3,{tname},{args.solver.upper()},{dom[-1]}>" for k in names),
             "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
             "peak_source": f"{peak_kind} hbm_gbs (MEASURED_PEAKS.json)" if peak_kind == "measured"
             else "fallback 6800 GB/s",
@@ -644,7 +651,8 @@ def measure_batch(precisions, steps, warmup, stream, specs=None, autotune=True, 
         out[name] = {"value": cells * 2 / (ms * 1e-3), "ms_per_step": ms, "steps": k, "cells": cells,
                      "dtype": {"fp32": "f32", "fp64": "f64", "fp64dw": "f32x2 double-word"}[name],
                      "tile": info, "l2": f"inputs larger than L2 (state {cells_nv * esz / 1e9:.2f} GB)",
-                     "roofline": {"bound": "hbm", "kernel": f"hydro_batch_kernel ({dom})", "achieved": achieved,
+                     "roofline": {"bound": "hbm", "kernel": f"{'hydro_batch_kernel' if name == 'fp64' else 'hydro_batch_strip_kernel'} ({dom})",
+                                  "achieved": achieved,
                                   "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                                   "peak_source": f"{peak_kind} hbm_gbs",
                                   "algorithmic_bytes": dom_bytes,
@@ -882,10 +890,10 @@ def measure_sod(stream, n=256):
     h.close()
     return {"value": n * 2 * nsteps / (ms * 1e-3), "ms_per_step": ms / nsteps, "run_ms": ms, "steps": nsteps,
             "time_reached": t, "cells": n, "dtype": "f64",
-            # launches_per_step() == 1: the whole advance call is one cooperative launch
+            # launches_per_step() == 1: the whole advance call is one launch
             "gpu_launches": 1 if lps == 1 else nsteps * lps,
-            "launch": ("one cooperative launch for all steps (one CTA per 31-cell tile, grid barriers between "
-                       "phases)") if lps == 1 else f"{lps} launches per step",
+            "launch": ("one launch for all steps on one thread-block cluster (the cells in registers and "
+                       "distributed shared memory, cluster barriers between phases)") if lps == 1 else f"{lps} launches per step",
             "note": "the step is bound by latency and by each SM's FP64 rate, not by the 256 cells' bytes"}
 
 

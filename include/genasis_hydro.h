@@ -71,8 +71,9 @@ extern "C" {
 
 #define GENASIS_FP64 0         /* state stored and processed in FP64 */
 #define GENASIS_FP32_MIXED 1   /* state stored and fluxes in FP32 (FP32 results
-                                  below 2^-126 flush to zero); internal-energy
-                                  cancellation, dt and totals reductions in FP64 */
+                                  below 2^-126 flush to zero); the internal energy
+                                  from compensated FP32 products, dt and totals
+                                  reduced across CTAs in FP64 */
 #define GENASIS_FP64_DW 2      /* state and arithmetic as double-word pairs of FP32
                                   (hi + lo, ~48 bits) on the FP32 pipes; the same
                                   results as GENASIS_FP64 to ~1e-13; host arrays are
@@ -174,9 +175,13 @@ int genasis_hydro_clear_status(genasis_hydro_t h);
 /* Launch configuration: tile index (0 .. tile_count - 1 for this ndim) and
  * planes per CTA along the march axis (0 = automatic).  info[0..5] receives
  * (tile index, tile x, tile y, planes per CTA, CTAs per stage, tile count).
- * Tile x and y count the cells a CTA owns: in 1D/2D a CTA of n threads owns
- * n - 1 columns (its last thread loads the next tile's first cell as a
- * neighbour only). */
+ * Tile x and y count the cells a CTA owns: in 1D and in 2D FP64 a CTA of n
+ * threads owns n - 1 columns (its last thread loads the next tile's first cell
+ * as a neighbour only); in 2D FP32, and in tile 1 of 2D double word, each warp
+ * works alone on 28 columns.  3D tile 14 (FP32) and tile 4 (double word) are the
+ * same for the x and y axes, followed by a launch of one thread per (x, y)
+ * column for z.  They and tile 1 of 2D double word are the defaults (3D meshes
+ * of 29 to 32 columns along x: tile 0). */
 int genasis_hydro_set_tile(genasis_hydro_t h, int tile, int kchunk);
 int genasis_hydro_get_tile(genasis_hydro_t h, int *info);
 
@@ -460,8 +465,8 @@ int genasis_hydro_step_noalloc(const genasis_hydro_desc *desc, const void *U_in,
  * equations and passages as above) with its own mesh, boundaries, gamma, time
  * and CFL time step; all problems of a batch share solver, theta and
  * precision.  Each RK stage of the whole batch is one persistent kernel launch
- * whose CTAs take (problem, tile, chunk) work items largest first from a
- * device counter; genasis_batch_run captures nsteps steps as one CUDA graph.
+ * whose CTAs (FP32 and double word: warps) take (problem, tile, chunk) work
+ * items largest first from a device counter; genasis_batch_run captures nsteps steps as one CUDA graph.
  * Arrays of problem i use the single-handle layout for that problem's ndim
  * and n.  Ownership, pointer kinds, synchronisation and error codes follow the
  * conventions at the top of this file.
