@@ -10,7 +10,8 @@
 //   Euler coarse substep between them), prolongation of the ring, the time
 //   step (deepest level: C min_l dt_CFL(l) / 2^(L-1-l); others: the time the
 //   child advanced), the two RK stages with the ring held (its K zeroed after
-//   stage 1), flux replacement on the uncovered coarse cells next to the
+//   stage 1; a level with a child takes K from the provisional substep and
+//   recomputes it next to the ring only), flux replacement on the uncovered coarse cells next to the
 //   child's box, restriction of the child onto the covered cells, and the
 //   accumulation of this level's boundary fluxes for its parent.
 // All scalars (level times and steps) live on the device; the recursion only
@@ -47,8 +48,7 @@ __device__ __forceinline__ size_t lin(int nd, int n, int i, int j, int k) {
 // The cells of the exterior ring, numbered 0 .. ring_count - 1: the layers below
 // and above along the slowest axis in full, then those of the next axis over the
 // interior of the slower ones, and so on.  At 132^3 the ring is 9% of the level:
-// visiting only its cells (and the provisional state by swapping buffers, and
-// kernels placed while their predecessors drain) took the step of four 128^3
+// visiting only its cells (with kernels placed while their predecessors drain) took the step of four 128^3
 // levels from 5.09 to 4.64 ms.
 __host__ __device__ inline unsigned ring_count(int nd, unsigned np, unsigned N) {
   return nd == 2 ? 2 * FNG * (np + N) : 2 * FNG * (np * np + np * N + N * N);

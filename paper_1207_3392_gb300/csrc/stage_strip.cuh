@@ -27,7 +27,7 @@
 // and ZMarch 440 and 324 at 79% and 66%: 493 and 490 us together.  The price is
 // memory traffic, 100 and 140 algorithmic bytes a cell for 40 and 60, half of
 // what the launches' times could move.  Double word at 128^3: 558 and 549 ->
-// 464 and 530 us.  With the shock switch (bits read beside U, HLLC and HLL both
+// 430 and 451 us (464 and 530 before its shorter multiply-add).  With the shock switch (bits read beside U, HLLC and HLL both
 // compiled at every face), 203 x 91 x 61: 176 -> 148 us a step, 24^3 61 -> 39.
 #pragma once
 
