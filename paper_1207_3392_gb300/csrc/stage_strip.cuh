@@ -434,7 +434,8 @@ struct ZMarch {
 #pragma unroll
       for (int i = 0; i < COPIES; ++i) {
         const int idx = i * 32 + lane, arr = idx >> 3;
-        // columns past the mesh repeat its last four of U and K (L: left as it is)
+        // lanes past the plane repeat its last four columns of U and K (L: left as it
+        // is); nothing of theirs leaves the march
         const unsigned col = min(j0 + 4u * (lane & 7), plane - 4u);
         const T* base = arr < 5 ? A.un + arr * vs
                         : STAGE == 2 && arr < 10 ? A.k1 + (arr - 5) * vs
@@ -602,6 +603,8 @@ struct ZMarch {
       sl2 = sl2 + 1 == SLOTS ? 0 : sl2 + 1;
     }
     if constexpr (ASYNC) asm volatile("cp.async.wait_group 0;" ::: "memory");
+    // a lane past the plane has W of one cell and the widths of another
+    if (!own) speed_max = T(0);
     if (STAGE == 1 && A.want_totals && own) {
       const double area = A.wd[0][x] * A.wd[1][y];
 #pragma unroll

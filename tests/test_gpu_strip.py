@@ -135,3 +135,35 @@ def test_double_word_strips_match_the_oracle_and_the_tiles(n):
                 ref = U
                 check(U, Uo, 2, TOL_FP64, f"dw {n} bc={bc}")
             np.testing.assert_array_equal(U, ref, err_msg=f"tile {t} kchunk {kc}")
+
+
+@pytest.mark.parametrize("n", [(36, 5, 4), (20, 10, 8), (2, 34, 5), (3, 12, 4)])
+def test_split_cfl_speed_on_a_mesh_refined_towards_the_upper_walls(n):
+    """Planes of 4 k cells that are not whole warps of the z march, the smallest
+    cells at the upper end of x (of y where a row is shorter than 4 cells) and the
+    fastest sound just before them: dt is the largest cell speed's, and dt, time
+    and state are those of tile 0 bit for bit."""
+    pr = P.random_blocks(3, n, seed=5, bc=P.REFLECT)
+    axis = 0 if n[0] >= 4 else 1
+    widths = [np.full(m, 0.01) for m in n]
+    widths[axis] *= 0.6 ** np.maximum(0, np.arange(n[axis]) - (n[axis] - 5))
+    p = np.ones(pr.shape)
+    if axis == 0:
+        p[:, n[1] - 1, n[0] - 4:n[0] - 1] = 9.0
+    else:
+        p[:, n[1] - 2, :] = 9.0
+    pr = pr.with_(widths=widths, rho=np.ones(pr.shape), vel=np.zeros_like(pr.vel), p=p)
+    cs = np.sqrt(pr.gamma * p)
+    iw = [1.0 / w.reshape([-1 if a == 2 - q else 1 for a in range(3)]) for q, w in enumerate(widths)]
+    dt = 0.3 / max(np.max(cs * i) for i in iw)
+    ref = None
+    for tile, kc in ((14, 0), (14, 1), (14, 3), (0, 0)):
+        h = H.Hydro.from_problem(pr, precision=H.FP32_MIXED)
+        h.set_tile(tile, kc)
+        first = h.advance(1, 0.3)
+        assert first == pytest.approx(dt, rel=1e-6), f"tile {tile} kchunk {kc}"
+        out = first, h.advance(3, 0.3), h.get_conserved()
+        h.close()
+        ref = ref or out
+        assert out[:2] == ref[:2], f"tile {tile} kchunk {kc}"
+        np.testing.assert_array_equal(out[2], ref[2])
