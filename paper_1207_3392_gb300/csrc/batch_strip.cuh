@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(32 * NW, (strip_warps<T, 2>() / NW))
     T speed = T(0.0f);
     bool bad = false;
     if (P.ndim == 1) {
-      typename K1::Tot tot[3];
+      Shares<3> tot;
       const StageArgs<T> A = Args::template args_for<1>(B, P, w.prob);
       for (int k = 0; k < STRIP_GROUP_1D; ++k) {
         const int x0 = (w.tx * STRIP_GROUP_1D + k) * STRIP_OWN;
@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(32 * NW, (strip_warps<T, 2>() / NW))
         K1::strip(A, x0, 0, 1, 0, speed, tot, bad);
       }
     } else {
-      typename K2::Tot tot[4];
+      Shares<4> tot;
       const StageArgs<T> A = Args::template args_for<2>(B, P, w.prob);
       const int m0 = w.chunk * B.kchunk;
       K2::strip(A, w.tx * STRIP_OWN, m0, min(A.n[1], m0 + B.kchunk), 0, speed, tot, bad);

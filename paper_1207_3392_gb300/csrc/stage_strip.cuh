@@ -51,59 +51,103 @@ __device__ __forceinline__ double lane_down(double x) { return __shfl_down_sync(
 __device__ __forceinline__ dw lane_up(dw x) { return dw(lane_up(x.hi), lane_up(x.lo)); }
 __device__ __forceinline__ dw lane_down(dw x) { return dw(lane_down(x.hi), lane_down(x.lo)); }
 
-// A lane's share of the conserved totals and their sum over the warp.  FP32 and
-// double-word states: double word, reduced on the FP32 pipes (as FP64 additions
-// this tail took 2-5 us of a stage on a mesh of 0.2 to 1 million cells); FP64:
-// FP64.
-template <class T>
-struct TotalSum {
-  using type = dw;
+// A lane's share of the conserved totals: its column sums and the FP64 product of
+// the other axes' widths they are to be multiplied by.
+template <int NV>
+struct Shares {
+  dw c[NV];
+  double area = 0.0;
+  __device__ __forceinline__ Shares() {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) c[v] = dw(0.0f, 0.0f);
+  }
 };
-template <>
-struct TotalSum<double> {
-  using type = double;
-};
-
-// column sum times `area` (the FP64 product of the other axes' widths) as three
-// floats: the pair alone would leave 2^-49 of it out
-__device__ __forceinline__ dw share_of(dw c, double area) {
-  const float a1 = (float)area;
-  const double r1 = area - (double)a1;
-  const float a2 = (float)r1, a3 = (float)(r1 - (double)a2);
-  const dw r = c * dw(a1, a2);
-  dw s;
-  fast_two_sum(r.hi, __fmaf_rn(c.hi, a3, r.lo), s.hi, s.lo);
-  return s;
-}
-__device__ __forceinline__ dw share_of(const ColumnSum<float>& t, double area) {
+__device__ __forceinline__ dw pair_of(const ColumnSum<float>& t) {
   dw c;
   fast_two_sum(t.hi, t.lo, c.hi, c.lo);
-  return share_of(c, area);
+  return c;
 }
-__device__ __forceinline__ dw share_of(const ColumnSum<dw>& t, double area) { return share_of(t.s, area); }
-__device__ __forceinline__ double share_of(const ColumnSum<double>& t, double area) { return t.s * area; }
+__device__ __forceinline__ dw pair_of(const ColumnSum<dw>& t) { return t.s; }
 
-__device__ __forceinline__ dw shfl_xor(dw x, int o) {
-  return dw(__shfl_xor_sync(0xffffffffu, x.hi, o), __shfl_xor_sync(0xffffffffu, x.lo, o));
+// x 2^k exactly: on the integer pipe unless x is zero, not finite or subnormal,
+// or the result leaves the normal range
+__device__ __forceinline__ double times_pow2(double x, int k) {
+  const long long b = __double_as_longlong(x);
+  const int ex = (int)(b >> 52) & 0x7ff;
+  if (ex > 0 && ex < 2047 && ex + k > 0 && ex + k < 2047) return __longlong_as_double(b + ((long long)k << 52));
+  return scalbn(x, k);
 }
-__device__ __forceinline__ double shfl_xor(double x, int o) { return __shfl_xor_sync(0xffffffffu, x, o); }
-// Sums of the NV shares over the warp into red[0 .. NV - 1].  Halving the first
-// four variables with the lanes takes six additions instead of twenty.
-template <int NV, class S>
-__device__ __forceinline__ void warp_totals(const S (&s)[NV], double* red) {
+
+// Brings the warp's largest area, and the largest column sum of each variable,
+// to [1, 2) by powers of two; scale[v] is what the sum of variable v is then to
+// be multiplied by.
+template <int NV>
+__device__ __forceinline__ void scale_shares(Shares<NV>& t, int (&scale)[NV]) {
+  const long long ab = __double_as_longlong(t.area);  // areas are positive
+  const int ea = (int)(ab >> 52);
+  const int ea_max = (int)__reduce_max_sync(0xffffffffu, (unsigned)ea), up = 1023 - ea_max;
+  t.area = ea > 0 && ea + up > 0 ? __longlong_as_double(ab + ((long long)up << 52)) : 0.0;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(t.c[v].hi) & 0x7fffffffu) >> 23;
+    const int e = (int)min(max(m, 1u), 253u);
+    const float f = __uint_as_float((unsigned)(254 - e) << 23);  // 2^(127 - e)
+    t.c[v] = dw(mul_rn(t.c[v].hi, f), mul_rn(t.c[v].lo, f));
+    scale[v] = e - 127 - up;
+  }
+}
+
+// Sums of the NV shares over the warp into red[0 .. NV - 1], in double word on
+// the FP32 pipes (as FP64 additions this tail took 2-5 us of a stage on a mesh of
+// 0.2 to 1 million cells).  Where areas or column sums are so large or small that
+// a share or its low word could leave FP32's range (an area above 2^128 gave NaN,
+// a share below 2^-102 lost its low word), all are scaled first and the scales
+// return with the FP64 result (a step of 256 x 768 takes 0.5% longer for it, of
+// 1024^2 0.3%; scaled always 0.8% and 0.5%).
+// The area enters as three floats: the pair alone would leave 2^-49 of it out.
+// Halving the first four variables with the lanes takes six additions instead of
+// twenty.
+template <int NV>
+__device__ __forceinline__ void warp_totals(Shares<NV> t, double* red) {
   static_assert(NV == 4 || NV == 5, "2D or 3D");
   const int lane = threadIdx.x & 31;
   const bool h = lane & 16, q = lane & 8;
+  int scale[NV];
+  unsigned most = 0, least = 0xffffffffu;  // |column sums|; least: bits - 1, so that zeros are left out
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    scale[v] = 0;
+    const unsigned m = __float_as_uint(t.c[v].hi) & 0x7fffffffu;
+    most = max(most, m);
+    least = min(least, m - 1u);
+  }
+  // column sums in 2^-46 .. 2^60 or 0, areas in 2^-30 .. 2^30 or 0
+  const unsigned ea = (unsigned)(__double_as_longlong(t.area) >> 52);
+  const bool usual = most < (127u + 60u) << 23 && least >= (127u - 46u) << 23 && (ea - (1023u - 30u) < 60u || ea == 0u);
+  if (!__all_sync(0xffffffffu, usual)) scale_shares<NV>(t, scale);
+  const float a1 = (float)t.area;
+  const double r1 = t.area - (double)a1;
+  const float a2 = (float)r1, a3 = (float)(r1 - (double)a2);
+  dw s[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    const dw r = t.c[v] * dw(a1, a2);
+    fast_two_sum(r.hi, fma_rn(t.c[v].hi, a3, r.lo), s[v].hi, s[v].lo);
+  }
+  auto across = [](dw x, int o) {
+    return dw(__shfl_xor_sync(0xffffffffu, x.hi, o), __shfl_xor_sync(0xffffffffu, x.lo, o));
+  };
   // lanes 0..15 keep variables 0, 1; lanes 16..31 keep 2, 3
-  const S a = (h ? s[2] : s[0]) + shfl_xor(h ? s[0] : s[2], 16);
-  const S b = (h ? s[3] : s[1]) + shfl_xor(h ? s[1] : s[3], 16);
-  S r = (q ? b : a) + shfl_xor(q ? a : b, 8);
-  for (int o = 4; o > 0; o >>= 1) r += shfl_xor(r, o);
-  if ((lane & 7) == 0) red[lane >> 3] = (double)r;  // lane 8 v holds variable v
+  const dw a = (h ? s[2] : s[0]) + across(h ? s[0] : s[2], 16);
+  const dw b = (h ? s[3] : s[1]) + across(h ? s[1] : s[3], 16);
+  dw r = (q ? b : a) + across(q ? a : b, 8);
+  for (int o = 4; o > 0; o >>= 1) r += across(r, o);
+  const int k = h ? (q ? scale[3] : scale[2]) : (q ? scale[1] : scale[0]);
+  if ((lane & 7) == 0) red[lane >> 3] = k ? times_pow2((double)r, k) : (double)r;  // lane 8 v holds variable v
   if constexpr (NV == 5) {
-    S e = s[4];
-    for (int o = 16; o > 0; o >>= 1) e += shfl_xor(e, o);
-    if (lane == 0) red[4] = (double)e;
+    dw x = s[4];
+    for (int o = 16; o > 0; o >>= 1) x += across(x, o);
+    if (lane == 0) red[4] = scale[4] ? times_pow2((double)x, scale[4]) : (double)x;
   }
 }
 
@@ -136,7 +180,6 @@ struct StripKernel {
   using Base = StageKernel<NDIM, T, SOLVER, STAGE, 32, 1, false>;
   using Acc = CellAccess<T, WIDE>;
   using Off = typename Acc::Off;
-  using Tot = typename TotalSum<T>::type;
   static constexpr int NV = NDIM + 2;
   static constexpr bool SW = Base::SW;  // per-face HLLC/HLL choice from shock bits
 
@@ -162,7 +205,7 @@ struct StripKernel {
   // Accumulates the lane's CFL speed and, with totals, its share of them
   // (stage 1), and the non-physical flag.  The whole warp calls it.
   static __device__ __forceinline__ void strip(const StageArgs<T>& A, int x0, int m0, int m1, int k, T& speed_out,
-                                               Tot (&tot)[NV], bool& bad) {
+                                               Shares<NV>& tot, bool& bad) {
     const int lane = threadIdx.x & 31;
     const int nx = A.n[0], ny = NDIM >= 2 ? A.n[1] : 1;
     const size_t vs = NDIM == 3 ? (size_t)nx * ny * A.n[2] : (size_t)nx * ny;
@@ -313,7 +356,8 @@ struct StripKernel {
     if (NDIM < 3 && STAGE == 1 && own) {
       if (NDIM == 2 && A.want_totals) {
 #pragma unroll
-        for (int v = 0; v < NV; ++v) tot[v] = share_of(tcol[v], A.wd[0][col]);
+        for (int v = 0; v < NV; ++v) tot.c[v] = pair_of(tcol[v]);
+        tot.area = A.wd[0][col];
       }
       speed_out = fmax(speed_out, speed_max);
     }
@@ -321,14 +365,14 @@ struct StripKernel {
 };
 
 // Fixed-order reduction of the warps' speeds and totals into CTA blk's partials.
-template <int NV, int NW, class T, class S>
+template <int NV, int NW, class T>
 __device__ __forceinline__ void write_warp_partials(const StageArgs<T>& A, size_t blk, int warp, T speed,
-                                                    const S (&tot)[NV], double (&red)[NW][NV + 1]) {
+                                                    const Shares<NV>& tot, double (&red)[NW][NV + 1]) {
   double s;
   if constexpr (std::is_same<T, float>::value) s = (double)warp_max(speed);
   else s = warp_max((double)speed);
   if ((threadIdx.x & 31) == 0) red[warp][0] = s;
-  if (A.want_totals) warp_totals<NV, S>(tot, &red[warp][1]);
+  if (A.want_totals) warp_totals<NV>(tot, &red[warp][1]);
   else if ((threadIdx.x & 31) < NV) red[warp][1 + (threadIdx.x & 31)] = 0.0;
   __syncthreads();
   const int t = threadIdx.x;
@@ -356,9 +400,7 @@ __global__ void __launch_bounds__(32 * NW, (strip_warps<T, 2>() / NW)) hydro_str
   const int x0 = (blockIdx.x * NW + warp) * STRIP_OWN;
   const int m0 = blockIdx.z * A.kchunk, m1 = min(A.n[1], m0 + A.kchunk);
   T speed = T(0);
-  typename K::Tot tot[NV];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) tot[v] = typename K::Tot(0.0);
+  Shares<NV> tot;
   bool bad = false;
   if (x0 < A.n[0]) K::strip(A, x0, m0, m1, 0, speed, tot, bad);
   if (bad) atomicOr(A.status, STATUS_NONPHYS);
@@ -380,7 +422,7 @@ __global__ void __launch_bounds__(32 * NW, (strip_warps<T, 3>() / NW))
   const int x0 = (id - k * strips) * STRIP_OWN;
   const int m0 = blockIdx.y * ychunk, m1 = min(A.n[1], m0 + ychunk);
   T speed = T(0);
-  typename K::Tot tot[5];
+  Shares<5> tot;
   bool bad = false;
   K::strip(A, x0, m0, m1, k, speed, tot, bad);
 }
@@ -400,7 +442,6 @@ struct ZMarch {
   using Base = StageKernel<3, T, SOLVER, STAGE, 32, 1, false>;
   using Acc = CellAccess<T, WIDE>;
   using Off = typename Acc::Off;
-  using Tot = typename TotalSum<T>::type;
   static constexpr int NV = 5;
   static constexpr int NARR = STAGE == 1 ? 10 : 15;        // U, (K,) L
   static constexpr int SLOTS = STAGE == 1 ? 7 : 6;
@@ -411,7 +452,7 @@ struct ZMarch {
   static constexpr size_t SMEM = ASYNC ? 4 * sizeof(Ring) : 0;  // four warps a CTA
 
   static __device__ __forceinline__ void march(const StageArgs<T>& A, Ring* ring, unsigned j, int m0, int m1,
-                                               T& speed_max, Tot (&tot)[NV], bool& bad) {
+                                               T& speed_max, Shares<NV>& tot, bool& bad) {
     const int lane = threadIdx.x & 31;
     const int nx = A.n[0], ny = A.n[1], nz = A.n[2];
     const unsigned plane = (unsigned)nx * (unsigned)ny;
@@ -606,9 +647,9 @@ struct ZMarch {
     // a lane past the plane has W of one cell and the widths of another
     if (!own) speed_max = T(0);
     if (STAGE == 1 && A.want_totals && own) {
-      const double area = A.wd[0][x] * A.wd[1][y];
 #pragma unroll
-      for (int v = 0; v < NV; ++v) tot[v] = share_of(tcol[v], area);
+      for (int v = 0; v < NV; ++v) tot.c[v] = pair_of(tcol[v]);
+      tot.area = A.wd[0][x] * A.wd[1][y];
     }
   }
 };
@@ -626,9 +667,7 @@ __global__ void __launch_bounds__(128, (sizeof(T) == 8 ? 4 : ASYNC && STAGE == 2
   const int chunk = gridDim.z - 1 - blockIdx.z;
   const int m0 = chunk * A.kchunk, m1 = min(A.n[2], m0 + A.kchunk);
   T speed = T(0);
-  typename K::Tot tot[NV];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) tot[v] = typename K::Tot(0.0);
+  Shares<NV> tot;
   bool bad = false;
   K::march(A, reinterpret_cast<typename K::Ring*>(smem_z) + warp, blockIdx.x * 128u + threadIdx.x, m0, m1, speed, tot,
            bad);

@@ -167,3 +167,29 @@ def test_split_cfl_speed_on_a_mesh_refined_towards_the_upper_walls(n):
         ref = ref or out
         assert out[:2] == ref[:2], f"tile {tile} kchunk {kc}"
         np.testing.assert_array_equal(out[2], ref[2])
+
+
+@pytest.mark.parametrize("precision,tile", [(H.FP32_MIXED, {2: 0, 3: 14}), (H.FP64_DW, {2: 1, 3: 4})])
+@pytest.mark.parametrize("n", [(30, 9, 7), (57, 33)])
+def test_totals_in_any_unit_of_length_and_density(n, precision, tile):
+    """Widths times 2^66 (areas beyond FP32's range), widths times 2^-40 and
+    densities and pressures times 2^-30 (shares below 2^-102): the totals scale by
+    exactly that power of two, and without a scale they are FP64's to 2^-45."""
+    pr = P.random_blocks(len(n), n, seed=7)
+    got = {}
+    for lw, ls in ((0, 0), (66, 0), (-40, 0), (-20, -30)):
+        h = H.Hydro.from_problem(pr.with_(widths=[w * 2.0 ** lw for w in pr.widths], rho=pr.rho * 2.0 ** ls,
+                                          p=pr.p * 2.0 ** ls), precision=precision)
+        h.set_tile(tile[len(n)], 0)
+        U0 = h.get_conserved(precision=H.FP64)
+        h.advance(1, 0.3)
+        got[lw, ls] = np.array(h.step_totals()) / 2.0 ** (len(n) * lw + ls)
+        h.close()
+        if lw == ls == 0:
+            vol = np.ones(pr.shape)
+            for q in range(len(n)):
+                vol = vol * np.asarray(pr.widths[q]).reshape([-1 if a == len(n) - 1 - q else 1 for a in range(len(n))])
+            ref = np.array([np.sum(u * vol) for u in U0])
+            size = np.array([np.sum(np.abs(u) * vol) for u in U0])
+            assert np.all(np.abs(got[0, 0] - ref) <= 2.0 ** -45 * size)
+        np.testing.assert_array_equal(got[lw, ls], got[0, 0], err_msg=f"widths 2^{lw}, state 2^{ls}")
