@@ -248,6 +248,8 @@ int configure(genasis_hydro* h, int tile, int kchunk_req) {
       if (chunks < 1) chunks = 1;
       kchunk = (int)((nm + chunks - 1) / chunks);
     }
+    const int fewest = (nm + 65534) / 65535;  // chunks are grid z
+    if (kchunk < fewest) kchunk = fewest;
     if (kchunk > nm) kchunk = nm;
     if ((v1.pair || v2.pair) && (kchunk & 1)) ++kchunk;  // whole plane pairs per chunk
     gz = (nm + kchunk - 1) / kchunk;

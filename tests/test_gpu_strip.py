@@ -193,3 +193,27 @@ def test_totals_in_any_unit_of_length_and_density(n, precision, tile):
             size = np.array([np.sum(np.abs(u) * vol) for u in U0])
             assert np.all(np.abs(got[0, 0] - ref) <= 2.0 ** -45 * size)
         np.testing.assert_array_equal(got[lw, ls], got[0, 0], err_msg=f"widths 2^{lw}, state 2^{ls}")
+
+
+@pytest.mark.parametrize("precision,n,tile", [(H.FP32_MIXED, (2, 65535 * 32 + 1), 0), (H.FP64_DW, (2, 65535 * 32 + 1), 1),
+                                              (H.FP32_MIXED, (2, 2, 65535 * 48 + 1), 14)])
+def test_march_axis_beyond_65535_chunks(precision, n, tile):
+    """A march axis of more chunks than a grid has along z, at the automatic chunk
+    and at a requested one of one row: bitwise the state of long chunks."""
+    nd = len(n)
+    rng = np.random.default_rng(3)
+    shape = tuple(reversed(n))
+    rho, p = rng.uniform(0.5, 2.0, shape), rng.uniform(0.5, 2.0, shape)
+    vel = rng.uniform(-0.5, 0.5, (nd,) + shape)
+    ref = None
+    for kc in (64, 0, 1):
+        h = H.Hydro(nd, n, [np.full(m, 0.1) for m in n], (P.OUTFLOW,) * nd, (P.REFLECT,) * nd, 1.4, H.HLLC,
+                    precision=precision)
+        assert kc or h.tile_info()["tile"] == tile
+        h.set_tile(tile, kc)
+        h.set_primitive(rho, vel, p)
+        h.advance(1, 0.4)
+        U = h.get_conserved()
+        h.close()
+        ref = U if ref is None else ref
+        np.testing.assert_array_equal(U, ref, err_msg=f"kchunk {kc}")
