@@ -117,7 +117,7 @@ __global__ void fmr_prolong_kernel(const T* __restrict__ Uc, const T* __restrict
   constexpr int NV = NDIM + 2;
   const unsigned np = gf.npad;
   const int N = gf.N;
-  const unsigned nf = np * (NDIM > 1 ? np : 1) * (NDIM > 2 ? np : 1);  // < 2^31 (n <= 1024)
+  const size_t vsf = (size_t)np * (NDIM > 1 ? np : 1) * (NDIM > 2 ? np : 1);
   const size_t vsc = (size_t)gc.npad * (NDIM > 1 ? gc.npad : 1) * (NDIM > 2 ? gc.npad : 1);
   chain_wait();
   const CoarseState<T, PROV> S(Uc, Kc, ltime, coarse);
@@ -143,7 +143,7 @@ __global__ void fmr_prolong_kernel(const T* __restrict__ Uc, const T* __restrict
         const T s = dm * dp > T(0) ? (fabs(dm) < fabs(dp) ? dm : dp) : T(0);
         out = out + s * (p[q] % 2 == 0 ? T(-0.25) : T(0.25));
       }
-      Uf[v * nf + t] = out;
+      Uf[v * vsf + t] = out;
     }
   }
 }
@@ -196,14 +196,14 @@ template <class T, int NDIM>
 __global__ void fmr_ring_zero_kernel(T* __restrict__ K, LevelGeo g) {
   constexpr int NV = NDIM + 2;
   const unsigned np = g.npad;
-  const unsigned nf = np * (NDIM > 1 ? np : 1) * (NDIM > 2 ? np : 1);
+  const size_t vs = (size_t)np * (NDIM > 1 ? np : 1) * (NDIM > 2 ? np : 1);
   chain_wait();
   const unsigned cells = ring_count(NDIM, np, g.N);
   for (unsigned r = blockIdx.x * blockDim.x + threadIdx.x; r < cells; r += gridDim.x * blockDim.x) {
     int p[3];
     ring_cell<NDIM>(r, np, g.N, p);
     const size_t t = lin(NDIM, np, p[0], p[1], p[2]);
-    for (int v = 0; v < NV; ++v) K[v * nf + t] = T(0);
+    for (int v = 0; v < NV; ++v) K[v * vs + t] = T(0);
   }
 }
 

@@ -94,3 +94,33 @@ def test_fmr_hll_and_leaf_conservation():
     t1 = M.leaf_totals()
     assert t1[0] == pytest.approx(t0[0], rel=1e-13)
     assert t1[-1] == pytest.approx(t0[-1], rel=1e-13)
+
+
+def test_fmr_levels_whose_variables_end_beyond_2_32():
+    """Two 3D levels of 1020^3 cells, stored as 1024^3 with the ring: the offset of
+    the energy is 2^32.  A uniform state at rest stays what it is, on the ring too."""
+    import torch
+    N = 1020
+    if torch.cuda.mem_get_info()[0] < 190e9:
+        pytest.skip("needs 190 GB of device memory")
+    g = H.Fmr(3, N, 2, 1.0, 1, precision=H.FP32_MIXED)
+    want = (1.0, 0.0, 0.0, 0.0, 2.5)
+    for l in range(2):
+        U = torch.empty(g.stored_shape(l), dtype=torch.float64, device="cuda")
+        for v, x in enumerate(want):
+            U[v] = x
+        torch.cuda.synchronize()
+        g.set_level(l, U)
+        torch.cuda.synchronize()
+        if l == 0:
+            del U
+            torch.cuda.empty_cache()
+    g.step(1, 0.3)
+    H.check(H.load().genasis_fmr_get_level(g._h, 1, U.data_ptr()))
+    torch.cuda.synchronize()
+    for v, x in enumerate(want):
+        lo, hi = torch.aminmax(U[v])
+        assert abs(lo.item() - x) < 1e-5 and abs(hi.item() - x) < 1e-5, f"variable {v}: {lo.item()} .. {hi.item()}"
+    g.close()
+    del U
+    torch.cuda.empty_cache()
