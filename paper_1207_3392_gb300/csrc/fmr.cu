@@ -112,8 +112,8 @@ struct CoarseState {
 // Exterior ring of fine level from the coarse level: child = coarse value +
 // minmod-limited conserved slopes x (-+ h_c / 4) per axis (added in axis order).
 template <class T, int NDIM, bool PROV>
-__global__ void fmr_prolong_kernel(const T* __restrict__ Uc, const T* __restrict__ Kc, const double* ltime, int coarse,
-                                   LevelGeo gc, T* __restrict__ Uf, LevelGeo gf) {
+__global__ void fmr_prolong_kernel(const T* Uc, const T* Kc, const double* ltime, int coarse,
+                                   LevelGeo gc, T* Uf, LevelGeo gf) {
   constexpr int NV = NDIM + 2;
   const unsigned np = gf.npad;
   const int N = gf.N;
@@ -129,9 +129,11 @@ __global__ void fmr_prolong_kernel(const T* __restrict__ Uc, const T* __restrict
     int c[3] = {0, 0, 0};
     for (int q = 0; q < NDIM; ++q) c[q] = N / 4 + p[q] / 2 - 1 + gc.off;  // coarse stored index
     const size_t cc = lin(NDIM, gc.npad, c[0], c[1], c[2]);
-    for (int v = 0; v < NV; ++v) {
+    T out[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {  // all loads before the stores
       const T u = S(v * vsc + cc);
-      T out = u;
+      out[v] = u;
       for (int q = 0; q < NDIM; ++q) {
         int cm[3] = {c[0], c[1], c[2]}, cp[3] = {c[0], c[1], c[2]};
         cm[q] -= 1;
@@ -141,17 +143,18 @@ __global__ void fmr_prolong_kernel(const T* __restrict__ Uc, const T* __restrict
         // minmod of the one-sided differences times the child offset (-+1/4 of a coarse cell)
         const T dm = u - um, dp = up - u;
         const T s = dm * dp > T(0) ? (fabs(dm) < fabs(dp) ? dm : dp) : T(0);
-        out = out + s * (p[q] % 2 == 0 ? T(-0.25) : T(0.25));
+        out[v] = out[v] + s * (p[q] % 2 == 0 ? T(-0.25) : T(0.25));
       }
-      Uf[v * vsf + t] = out;
     }
+#pragma unroll
+    for (int v = 0; v < NV; ++v) Uf[v * vsf + t] = out[v];
   }
 }
 
 // Covered coarse cells = mean of their 2^d children (pairs along the slowest
 // axis first, as the reference averages).
 template <class T, int NDIM>
-__global__ void fmr_restrict_kernel(const T* __restrict__ Uf, LevelGeo gf, T* __restrict__ Uc, LevelGeo gc) {
+__global__ void fmr_restrict_kernel(const T* Uf, LevelGeo gf, T* Uc, LevelGeo gc) {
   constexpr int NV = NDIM + 2;
   chain_wait();
   const unsigned M = gc.N / 2;  // covered cells per axis
@@ -163,10 +166,12 @@ __global__ void fmr_restrict_kernel(const T* __restrict__ Uf, LevelGeo gf, T* __
     const int a[3] = {(int)(t - t1 * M), NDIM > 1 ? (int)(t1 % M) : 0, NDIM > 2 ? (int)(t1 / M) : 0};
     int f0[3] = {0, 0, 0};
     for (int q = 0; q < NDIM; ++q) f0[q] = gf.off + 2 * a[q];
-    for (int v = 0; v < NV; ++v) {
+    T mean[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {  // all loads before the stores
       const T* U = Uf + v * vsf;
       const T half = T(0.5);  // (a + b) / 2, exactly as the mean of two
-      T m;
+      T& m = mean[v];
       if (NDIM == 1) {
         m = (U[f0[0]] + U[f0[0] + 1]) * half;
       } else if (NDIM == 2) {
@@ -184,16 +189,18 @@ __global__ void fmr_restrict_kernel(const T* __restrict__ Uf, LevelGeo gf, T* __
         for (int dx = 0; dx < 2; ++dx) bx[dx] = (byx[0][dx] + byx[1][dx]) * half;
         m = (bx[0] + bx[1]) * half;
       }
-      int c[3] = {0, 0, 0};
-      for (int q = 0; q < NDIM; ++q) c[q] = gc.off + gc.N / 4 + a[q];
-      Uc[v * vsc + lin(NDIM, gc.npad, c[0], c[1], c[2])] = m;
     }
+    int c[3] = {0, 0, 0};
+    for (int q = 0; q < NDIM; ++q) c[q] = gc.off + gc.N / 4 + a[q];
+    const size_t cc = lin(NDIM, gc.npad, c[0], c[1], c[2]);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) Uc[v * vsc + cc] = mean[v];
   }
 }
 
 // K = 0 on the exterior ring (the ring is held through both RK stages).
 template <class T, int NDIM>
-__global__ void fmr_ring_zero_kernel(T* __restrict__ K, LevelGeo g) {
+__global__ void fmr_ring_zero_kernel(T* K, LevelGeo g) {
   constexpr int NV = NDIM + 2;
   const unsigned np = g.npad;
   const size_t vs = (size_t)np * (NDIM > 1 ? np : 1) * (NDIM > 2 ? np : 1);
@@ -209,8 +216,8 @@ __global__ void fmr_ring_zero_kernel(T* __restrict__ K, LevelGeo g) {
 
 // Per-block max over the interior of max_q (|v_q| + c_s).
 template <class T, int NDIM, bool PROV>
-__global__ void fmr_speed_kernel(const T* __restrict__ U, const T* __restrict__ K, const double* ltime, int level,
-                                 LevelGeo g, double gamma, double* __restrict__ part) {
+__global__ void fmr_speed_kernel(const T* U, const T* K, const double* ltime, int level,
+                                 LevelGeo g, double gamma, double* part) {
   constexpr int NV = NDIM + 2;
   __shared__ double red[32];
   chain_wait();
@@ -295,7 +302,7 @@ __global__ void fmr_sync_times_kernel(double* ltime, int L) {
 // are theirs bit for bit).  9% of the cells of a 128^3 level: about 13 us in place
 // of a whole first stage's 80.
 template <class T, int NDIM, int Q, int SOLVER>
-__device__ __forceinline__ void shell_axis(const StageArgs<T>& A, const T* __restrict__ U, size_t c, int i, size_t vs,
+__device__ __forceinline__ void shell_axis(const StageArgs<T>& A, const T* U, size_t c, int i, size_t vs,
                                            const T (&w)[NDIM + 2], T (&L)[NDIM + 2]) {
   constexpr int NV = NDIM + 2;
   const size_t st = Q == 0 ? 1 : Q == 1 ? (size_t)A.n[0] : (size_t)A.n[0] * A.n[1];
@@ -330,7 +337,7 @@ __device__ __forceinline__ void shell_axis(const StageArgs<T>& A, const T* __res
 }
 
 template <class T, int NDIM, int SOLVER>
-__global__ void __launch_bounds__(128) fmr_shell_kernel(StageArgs<T> A, const T* __restrict__ U, T* __restrict__ K,
+__global__ void __launch_bounds__(128) fmr_shell_kernel(StageArgs<T> A, const T* U, T* K,
                                                         LevelGeo g) {
   constexpr int NV = NDIM + 2;
   chain_wait();
@@ -420,9 +427,9 @@ __host__ __device__ inline size_t cf_index(int nd, int M, int q, int side, int v
 // above, with the Heun-effective flux of the coarse face.  One thread per coarse
 // face (a cell next to the box has one face on it, so no cell is written twice).
 template <class T, int NDIM, int SOLVER>
-__global__ void __launch_bounds__(64) fmr_replace_kernel(StageArgs<T> A, const T* __restrict__ U0,
-                                                         const T* __restrict__ K, T* __restrict__ U, LevelGeo g,
-                                                         const double* __restrict__ phi, double h) {
+__global__ void __launch_bounds__(64) fmr_replace_kernel(StageArgs<T> A, const T* U0,
+                                                         const T* K, T* U, LevelGeo g,
+                                                         const double* phi, double h) {
   constexpr int NV = NDIM + 2;
   const int M = g.N / 2;
   const int per = NDIM == 1 ? 1 : NDIM == 2 ? M : M * M;
@@ -446,10 +453,14 @@ __global__ void __launch_bounds__(64) fmr_replace_kernel(StageArgs<T> A, const T
     if (side == 0) c[q] -= 1;
     const double sign = side == 0 ? 1.0 : -1.0, hdt = 0.5 * dtd;
     const size_t cc = lin(NDIM, g.npad, c[0], c[1], c[2]);
+    T un[NV];
+#pragma unroll
     for (int v = 0; v < NV; ++v) {
       const double d = hdt * Fe[v] - phi[cf_index(NDIM, M, q, side, v, tr)];
-      U[v * vs + cc] = (T)((double)U[v * vs + cc] + sign * d / h);
+      un[v] = (T)((double)U[v * vs + cc] + sign * d / h);
     }
+#pragma unroll
+    for (int v = 0; v < NV; ++v) U[v * vs + cc] = un[v];
   }
 }
 
@@ -461,9 +472,9 @@ __global__ void __launch_bounds__(64) fmr_replace_kernel(StageArgs<T> A, const T
 // with exactly ceil(total / 128) blocks of 128 threads and no early return,
 // so every lane of a warp reaches the shuffles.
 template <class T, int NDIM, int SOLVER>
-__global__ void __launch_bounds__(128) fmr_child_faces_kernel(StageArgs<T> A, const T* __restrict__ U0,
-                                                              const T* __restrict__ K, LevelGeo g,
-                                                              double* __restrict__ acc) {
+__global__ void __launch_bounds__(128) fmr_child_faces_kernel(StageArgs<T> A, const T* U0,
+                                                              const T* K, LevelGeo g,
+                                                              double* acc) {
   constexpr int NV = NDIM + 2;
   constexpr int G = 1 << (NDIM - 1);  // fine faces per parent face
   const int M = g.N / 2;
@@ -503,10 +514,10 @@ __global__ void __launch_bounds__(128) fmr_child_faces_kernel(StageArgs<T> A, co
   }
   if (act && sub == 0) {
     const double share = dtd / (double)(2 * G);  // exact: m sums two fluxes of each of G faces
-    for (int v = 0; v < NV; ++v) {
-      const size_t o = cf_index(NDIM, M, q, side, v, tr);
-      acc[o] = acc[o] + share * m[v];
-    }
+#pragma unroll
+    for (int v = 0; v < NV; ++v) m[v] = acc[cf_index(NDIM, M, q, side, v, tr)] + share * m[v];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) acc[cf_index(NDIM, M, q, side, v, tr)] = m[v];
   }
 }
 

@@ -22,6 +22,9 @@ enum : unsigned { STATUS_NONPHYS = 1u, STATUS_TIMEOUT = 2u };
 // predecessor has finished and its writes are visible, and lets the successor's
 // CTAs be placed; a kernel of the chain calls it before any access to memory
 // that a kernel writes.  Without the launch attribute it is a no-op.
+// Such memory is then read with plain loads: __ldg, and const __restrict__
+// parameters, promise that nobody writes it while the kernel runs, which in a
+// chain begins before the wait, and would let the compiler load ahead of it.
 __device__ __forceinline__ void chain_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -344,9 +344,8 @@ constexpr int RED_PARAMS = 32, RED_SLICES = 8;
 constexpr int RED_CTAS = (mlp::NPARAM + RED_PARAMS - 1) / RED_PARAMS + 1;
 
 __global__ void __launch_bounds__(RED_PARAMS * RED_SLICES)
-    mlp_reduce_adam_kernel(const float* __restrict__ part, const float* __restrict__ part_loss, int nblk,
-                           float* __restrict__ grad_out, float* __restrict__ loss_out, float* P, float* m, float* v,
-                           int step, float lr, float b1, float b2, float eps) {
+    mlp_reduce_adam_kernel(const float* part, const float* part_loss, int nblk, float* grad_out, float* loss_out,
+                           float* P, float* m, float* v, int step, float lr, float b1, float b2, float eps) {
   __shared__ float sums[RED_SLICES][RED_PARAMS];
   chain_wait();
   const int col = threadIdx.x % RED_PARAMS, slice = threadIdx.x / RED_PARAMS;

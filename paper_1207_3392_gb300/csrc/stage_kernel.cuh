@@ -43,9 +43,9 @@ struct StageArgs {
   const double* wd[3];    // widths in FP64, index c (totals)
   const T* wdh[3];        // widths split as wdh + wdl (FP32 state: both floats; FP64 state: wdh = wd)
   const T* wdl[3];
-  const T* __restrict__ un;   // U^n      [NV][n2][n1][n0]
-  const T* __restrict__ k1;   // K of stage 1 (stage 2 only)
-  T* __restrict__ out;        // stage 1: K; stage 2: U^{n+1}
+  const T* un;                // U^n      [NV][n2][n1][n0]
+  const T* k1;                // K of stage 1 (stage 2 only)
+  T* out;                     // stage 1: K; stage 2: U^{n+1}
   const double* dt;           // device scalar (stage 2)
   int kchunk;                 // planes per CTA along the march axis
   double* part_speed;         // stage 1: per-CTA max over cells of max_q (|v_q| + c_s) / dq
@@ -61,12 +61,12 @@ struct StageArgs {
 // 1D/2D one axis gains less than the extra barrier costs.
 // COH: the state arrays may have been written earlier in the same launch (the
 // one-launch advance of small 1D meshes), so they are read through L2 (__ldcg), which
-// is coherent, instead of the read-only cache (__ldg).  Same values either way.
+// is coherent.  Same values either way.
 template <int NDIM, class T, int SOLVER, int STAGE, int TX, int TY, bool PRE = (NDIM == 3), bool COH = false>
 struct StageKernel {
   static __device__ __forceinline__ T ld(const T* p) {
     if constexpr (COH) return __ldcg(p);
-    else return __ldg(p);
+    else return *p;
   }
   static constexpr int NV = NDIM + 2;
   static constexpr bool SW = SOLVER == SOLVER_HLLC_SW;  // per-face HLLC/HLL choice from shock bits

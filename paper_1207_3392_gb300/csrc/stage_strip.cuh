@@ -151,11 +151,32 @@ __device__ __forceinline__ void warp_totals(Shares<NV> t, double* red) {
   }
 }
 
-// WIDE: 64-bit cell offsets, for meshes of more than 2^30 cells.
+// Loads of the state and of K in the marches.  WIDE: 64-bit cell offsets, for
+// meshes of more than 2^30 cells.
+// FP32: the loads are not ordered against the march's own stores (nothing that a
+// march reads is written by it), so that a row's can be issued before the last
+// row's stores; held() makes the address depend on a point after chain_wait(), which
+// keeps them behind the predecessor's writes.  With plain loads a step of 1024^2
+// takes 1687 us for 32 instead of 1668.  Double word has no registers left for the
+// pointers (128^3, 6 steps: 5824 us with them) and takes plain loads (5627).
 template <class T, bool WIDE>
 struct CellAccess {
   using Off = typename std::conditional<WIDE, size_t, unsigned>::type;
-  static __device__ __forceinline__ T at(const T* p, Off c) { return __ldg(p + c); }
+  static __device__ __forceinline__ const T* held(const T* p) { return p; }
+  static __device__ __forceinline__ T at(const T* p, Off c) { return p[c]; }
+};
+template <bool WIDE>
+struct CellAccess<float, WIDE> {
+  using Off = typename std::conditional<WIDE, size_t, unsigned>::type;
+  static __device__ __forceinline__ const float* held(const float* p) {
+    asm volatile("" : "+l"(p) : : "memory");
+    return p;
+  }
+  static __device__ __forceinline__ float at(const float* p, Off c) {
+    float x;
+    asm("ld.global.f32 %0, [%1];" : "=f"(x) : "l"(__cvta_generic_to_global(p + c)));
+    return x;
+  }
 };
 
 // The march-axis step shared by the strips (along y) and ZMarch (along z):
@@ -207,6 +228,8 @@ struct StripKernel {
   static __device__ __forceinline__ void strip(const StageArgs<T>& A, int x0, int m0, int m1, int k, T& speed_out,
                                                Shares<NV>& tot, bool& bad) {
     const int lane = threadIdx.x & 31;
+    const T* const un = Acc::held(A.un);
+    const T* const k1 = STAGE == 2 ? Acc::held(A.k1) : nullptr;
     const int nx = A.n[0], ny = NDIM >= 2 ? A.n[1] : 1;
     const size_t vs = NDIM == 3 ? (size_t)nx * ny * A.n[2] : (size_t)nx * ny;
     const T dt = STAGE == 2 ? (T)(*A.dt) : T(0);
@@ -224,8 +247,8 @@ struct StripKernel {
     auto load = [&](Off c, T (&u)[NV]) {
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        u[v] = Acc::at(A.un + v * vs, c);
-        if (STAGE == 2) u[v] = fma_rn(dt, Acc::at(A.k1 + v * vs, c), u[v]);
+        u[v] = Acc::at(un + v * vs, c);
+        if (STAGE == 2) u[v] = fma_rn(dt, Acc::at(k1 + v * vs, c), u[v]);
       }
     };
     // Epilogue of the own cell at offset c: L = minus the divergence, source,
@@ -254,7 +277,7 @@ struct StripKernel {
         T r[NV];
 #pragma unroll
         for (int v = 0; v < NV; ++v)
-          r[v] = fma_rn(hdt, add_rn(Acc::at(A.k1 + v * vs, c), L[v]), Acc::at(A.un + v * vs, c));
+          r[v] = fma_rn(hdt, add_rn(Acc::at(k1 + v * vs, c), L[v]), Acc::at(un + v * vs, c));
         if (own) {
 #pragma unroll
           for (int v = 0; v < NV; ++v) A.out[v * vs + c] = r[v];
@@ -454,6 +477,8 @@ struct ZMarch {
   static __device__ __forceinline__ void march(const StageArgs<T>& A, Ring* ring, unsigned j, int m0, int m1,
                                                T& speed_max, Shares<NV>& tot, bool& bad) {
     const int lane = threadIdx.x & 31;
+    const T* const un = Acc::held(A.un);
+    const T* const k1 = STAGE == 2 ? Acc::held(A.k1) : nullptr;
     const int nx = A.n[0], ny = A.n[1], nz = A.n[2];
     const unsigned plane = (unsigned)nx * (unsigned)ny;
     const size_t vs = (size_t)plane * nz;
@@ -518,8 +543,8 @@ struct ZMarch {
           if (STAGE == 2) u[v] = fma_rn(dt, ring->a[slot][5 + v][lane], u[v]);
         } else {
           const Off c = (Off)sm * (Off)plane + (Off)jc;
-          u[v] = Acc::at(A.un + v * vs, c);
-          if (STAGE == 2) u[v] = fma_rn(dt, Acc::at(A.k1 + v * vs, c), u[v]);
+          u[v] = Acc::at(un + v * vs, c);
+          if (STAGE == 2) u[v] = fma_rn(dt, Acc::at(k1 + v * vs, c), u[v]);
         }
       }
       if constexpr (Base::SW) fl = A.flags[(Off)sm * (Off)plane + (Off)jc];
@@ -622,8 +647,8 @@ struct ZMarch {
             u0 = ring->a[sl0][v][lane];
             k = ring->a[sl0][5 + v][lane];
           } else {
-            u0 = Acc::at(A.un + v * vs, c);
-            k = Acc::at(A.k1 + v * vs, c);
+            u0 = Acc::at(un + v * vs, c);
+            k = Acc::at(k1 + v * vs, c);
           }
           L[v] = fma_rn(hdt, add_rn(k, L[v]), u0);
         }
