@@ -117,6 +117,21 @@ __device__ __forceinline__ double max0(double a, double b) {
   return (ka < kb ? kb : ka) > 0 ? m : 0.0;
 }
 
+// The same with 2^-120 (FP64 2^-500) in place of 0, far below any speed, and
+// |x| <= that: HLLC's upwind test.  With it S_K - v_K is not zero where v_K and S_K are.
+__device__ __forceinline__ float max_floor(float a, float b) { return fmaxf(0x1p-120f, fmaxf(a, b)); }
+__device__ __forceinline__ dw max_floor(dw a, dw b) { return fmax(dw(0x1p-120f, 0.0f), fmax(a, b)); }
+__device__ __forceinline__ double max_floor(double a, double b) {
+  const long long ka = okey(a), kb = okey(b);
+  const double m = ka < kb ? b : a;
+  return (ka < kb ? kb : ka) > 0x20b0000000000000ll ? m : 0x1p-500;
+}
+__device__ __forceinline__ bool at_floor(float x) { return fabsf(x) <= 0x1p-120f; }
+__device__ __forceinline__ bool at_floor(dw x) { return fabsf(x.hi) <= 0x1p-120f; }
+__device__ __forceinline__ bool at_floor(double x) {  // to within the high word
+  return (unsigned)((unsigned long long)__double_as_longlong(x) >> 32 & 0x7fffffffu) <= 0x20b00000u;
+}
+
 // max(a, b) of a CFL speed a >= 0 that ignores a NaN b, x > 0, |x| < infinity,
 // x == 0 and x >= 0; FP64: on the integer pipe.
 template <class T>
@@ -137,8 +152,6 @@ __device__ __forceinline__ bool finite(double x) {
   return (__double_as_longlong(x) & 0x7fffffffffffffffll) < 0x7ff0000000000000ll;
 }
 __device__ __forceinline__ bool is_zero(float x) { return x == 0.0f; }
-__device__ __forceinline__ bool is_zero(dw x) { return x.hi == 0.0f; }
-__device__ __forceinline__ bool is_zero(double x) { return ((unsigned long long)__double_as_longlong(x) << 1) == 0; }
 __device__ __forceinline__ bool nonneg(float x) { return x >= 0.0f; }
 __device__ __forceinline__ bool nonneg(dw x) { return x.hi >= 0.0f; }
 __device__ __forceinline__ bool nonneg(double x) { return okey(x) >= -1; }
@@ -393,7 +406,11 @@ __device__ __forceinline__ void recover(const float (&u)[NDIM + 2], float (&w)[N
 //                1.36 -> 1.14, FP32 256^3 1.436 -> 1.383 (bound by issue).
 //                alpha_- = 0 gives F_L, alpha_+ = 0 gives F_R (upwind): there
 //                S_K = 0, and alpha_m is replaced by v_K, for which U* = U_K
-//                and the formulas above are F_K.
+//                and the formulas above are F_K.  (The code's S_K is then not 0
+//                but 2^-120, 2^-500 in FP64: that changes no bit of F_K, and the
+//                side may also be at rest, where 1 / (S_K - v_K) of S_K = 0 would
+//                make the vanishing terms NaN: a limited pressure at or
+//                below 0 on a stretched mesh.)
 // ---------------------------------------------------------------------------
 // Conserved state U(W) and physical flux F^Q(U) of one side of a face
 // (Sec. 3.5): p is its pressure, w[1 + Q] its normal velocity.
@@ -422,10 +439,10 @@ __device__ __forceinline__ void face_flux(const T (&wl)[NDIM + 2], const T (&wr)
   const T vl = wl[1 + Q], vr = wr[1 + Q];
   const T cl = sound_speed(gamma, pl, nl);
   const T cr = sound_speed(gamma, pr, nr);
-  const T ap = max0(add_rn(vl, cl), add_rn(vr, cr));
-  const T am = max0(sub_rn(cl, vl), sub_rn(cr, vr));
 
   if constexpr (SOLVER == SOLVER_HLL) {
+    const T ap = max0(add_rn(vl, cl), add_rn(vr, cr));
+    const T am = max0(sub_rn(cl, vl), sub_rn(cr, vr));
     T ul[NV], ur[NV], fl[NV], fr[NV];
     side_state<T, NDIM, Q>(wl, pl, ul, fl);
     side_state<T, NDIM, Q>(wr, pr, ur, fr);
@@ -435,11 +452,13 @@ __device__ __forceinline__ void face_flux(const T (&wl)[NDIM + 2], const T (&wr)
     for (int v = 0; v < NV; ++v)
       F[v] = mul_rn(fma_rn(-apam, sub_rn(ur[v], ul[v]), fma_rn(am, fr[v], mul_rn(ap, fl[v]))), inv);
   } else {
+    const T ap = max_floor(add_rn(vl, cl), add_rn(vr, cr));
+    const T am = max_floor(sub_rn(cl, vl), sub_rn(cr, vr));
     const T sl = add_rn(am, vl);  // = -(S_L - v_L) > 0
     const T sr = sub_rn(ap, vr);  // =   S_R - v_R  > 0
     const T al = mul_rn(nl, sl), ar = mul_rn(nr, sr);
     const T alpha = fdiv(fma_rn(ar, vr, fma_rn(al, vl, sub_rn(pl, pr))), add_rn(ar, al));
-    const bool left = is_zero(am) || (!is_zero(ap) && nonneg(alpha));
+    const bool left = at_floor(am) || (!at_floor(ap) && nonneg(alpha));
     const T SK = left ? -am : ap;
     const T dK = left ? -sl : sr;
     const T aK = left ? -al : ar;
@@ -448,7 +467,7 @@ __device__ __forceinline__ void face_flux(const T (&wl)[NDIM + 2], const T (&wr)
 #pragma unroll
     for (int v = 0; v < NV; ++v) wK[v] = left ? wl[v] : wr[v];
     const T vK = wK[1 + Q];
-    const T a = is_zero(SK) ? vK : alpha;
+    const T a = at_floor(SK) ? vK : alpha;
     const T dv = sub_rn(a, vK);
     T v2 = mul_rn(wK[1], wK[1]);
 #pragma unroll

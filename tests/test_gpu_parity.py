@@ -726,3 +726,39 @@ def test_fp32_kinetic_dominated_states(ndim, n):
         Uo, to, _ = O.evolve(g, U0.astype(np.float64), pr.cfl, max_steps=1)
         assert t == pytest.approx(to, rel=1e-5)
         _check(Ug, Uo, ndim, TOL_FP32, f"kinetic {ndim}d solver={solver}")
+
+
+@pytest.mark.parametrize("precision,tol", [(H.FP64, TOL_FP64), (H.FP64_DW, TOL_FP64), (H.FP32_MIXED, TOL_FP32)])
+@pytest.mark.parametrize("ndim", [1, 2, 3])
+def test_upwind_side_at_rest_without_pressure(ndim, precision, tol):
+    """A wide cell between narrow ones at theta 2: its limited pressure falls below
+    zero at the face towards a supersonic outflow, where that side, at rest, is the
+    upwind one.  The flux is its pressure's alone; every cell stays physical, as in
+    the oracle."""
+    for axis in range(ndim):
+        for flip in (False, True):
+            n = [5] * ndim
+            n[axis] = 32
+            w = np.full(32, 0.01)
+            w[15] = 0.2
+            p, v = np.full(32, 10.0), np.zeros(32)
+            p[15], p[16:], v[16:] = 1.0, 0.01, 30.0
+            if flip:
+                w, p, v = w[::-1].copy(), p[::-1].copy(), -v[::-1].copy()
+            pr = P.random_blocks(ndim, tuple(n), seed=1, bc=P.OUTFLOW)
+            widths = [np.full(m, 0.01) for m in n]
+            widths[axis] = w
+            line = [1] * ndim
+            line[ndim - 1 - axis] = 32
+            vel = np.zeros_like(pr.vel)
+            vel[axis] += v.reshape(line)
+            pr = pr.with_(widths=widths, rho=np.ones(pr.shape), p=np.zeros(pr.shape) + p.reshape(line), vel=vel, theta=2.0)
+            g = O.Grid(pr, solver=H.HLLC)
+            Uo, to, _ = O.evolve(g, O.initial_state(pr, g), 0.1, max_steps=1)
+            assert np.all(np.isfinite(Uo))
+            h = H.Hydro.from_problem(pr, precision=precision, solver=H.HLLC)
+            t = h.advance(1, 0.1)
+            U = h.get_conserved(precision=H.FP64)
+            h.close()
+            assert t == pytest.approx(to, rel=1e-5)
+            _check(U, Uo, ndim, tol, f"{ndim}d axis {axis} flip {flip}")
