@@ -81,6 +81,7 @@ struct genasis_batch {
   unsigned long long* speed = nullptr;
   unsigned* status = nullptr;
   int tile = 0, chunk = 32, ctas = 0;
+  int group_1d = 1;  // strips of a 1D item
   BatchVariant v1{}, v2{};
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   int g_nsteps = -1;
@@ -144,6 +145,21 @@ int configure(genasis_batch* b, int tile, int chunk) {
   for (BatchVariant* v : {&v1, &v2})
     if (v->fn_wide && most > ((size_t)1 << 30)) v->fn = v->fn_wide;
   if (chunk == 0) chunk = 32;
+  int occ1 = 0, occ2 = 0;
+  for (BatchVariant* v : {&v1, &v2})
+    if (v->smem > 48 * 1024) GH_CK(cudaFuncSetAttribute(v->fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v->smem));
+  GH_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ1, v1.fn, v1.tx, v1.smem));
+  GH_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ2, v2.fn, v2.tx, v2.smem));
+  const int occ = std::max(1, std::min(occ1, occ2));
+  // 1D items: as few strips as leave every resident warp one item (a warp takes
+  // its strips one after the other: a step of 30 problems of 100 to 1500 cells
+  // takes 10 us with 1 strip, 18 with 8, double word 13 and 34; with many items
+  // taking them costs more: 1000 problems of 128 to 4096 cells 73 us with 1 strip, 34 with 8)
+  long strips = 0;
+  for (const HostProblem& h : b->hp)
+    if (h.ndim == 1) strips += (h.n[0] + cols - 1) / cols;
+  const long slots = (long)occ * v1.warps * b->num_sms;
+  b->group_1d = (int)std::max(1L, std::min((long)v1.most_1d, (strips + slots - 1) / slots));
   // work items: (problem, x tile, y chunk), largest first
   struct Item {
     long cost;
@@ -152,7 +168,7 @@ int configure(genasis_batch* b, int tile, int chunk) {
   std::vector<Item> items;
   for (int p = 0; p < b->nprob; ++p) {
     const HostProblem& h = b->hp[p];
-    const int width = h.ndim == 1 ? cols * v1.group_1d : cols;
+    const int width = h.ndim == 1 ? cols * b->group_1d : cols;
     const int gx = (h.n[0] + width - 1) / width;
     const int gz = h.ndim == 2 ? (h.n[1] + chunk - 1) / chunk : 1;
     for (int x = 0; x < gx; ++x)
@@ -170,12 +186,6 @@ int configure(genasis_batch* b, int tile, int chunk) {
   GH_CK(cudaMalloc(&b->items, flat.size() * sizeof(BatchItem)));
   GH_CK(cudaMemcpy(b->items, flat.data(), flat.size() * sizeof(BatchItem), cudaMemcpyHostToDevice));
   b->nitems = (int)flat.size();
-  int occ1 = 0, occ2 = 0;
-  for (BatchVariant* v : {&v1, &v2})
-    if (v->smem > 48 * 1024) GH_CK(cudaFuncSetAttribute(v->fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v->smem));
-  GH_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ1, v1.fn, v1.tx, v1.smem));
-  GH_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ2, v2.fn, v2.tx, v2.smem));
-  int occ = std::max(1, std::min(occ1, occ2));
   b->ctas = std::min((b->nitems + v1.warps - 1) / v1.warps, occ * b->num_sms);
   if (b->ctas < 1) b->ctas = 1;
   b->v1 = v1;
@@ -207,6 +217,7 @@ BatchArgs<T> batch_args(genasis_batch* b, int stage, unsigned* counter) {
   A.speed = b->speed;
   A.status = b->status;
   A.kchunk = b->chunk;
+  A.group_1d = b->group_1d;
   return A;
 }
 

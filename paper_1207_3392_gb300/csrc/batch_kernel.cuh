@@ -42,6 +42,7 @@ struct BatchArgs {
   unsigned long long* speed;  // per-problem max CFL speed (FP64 bit pattern; stage 1)
   unsigned* status;         // per-problem status
   int kchunk;               // planes (rows) per 2D item
+  int group_1d;             // strips per 1D item (batch_strip.cuh)
 };
 
 template <class T, int SOLVER, int STAGE, int TX>

@@ -11,7 +11,7 @@ struct BatchVariant {
   int tx;    // threads per CTA (one tile row)
   int cols;  // columns of cells a tile owns
   int warps = 1;      // work items a CTA runs at once (one per warp), 1: the whole CTA runs one
-  int group_1d = 1;   // x tiles of a 1D item
+  int most_1d = 1;    // most x tiles of a 1D item
   const void* fn_wide = nullptr;  // the kernel when a problem has more than 2^30 cells, where it is another
 };
 

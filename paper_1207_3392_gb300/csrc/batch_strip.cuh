@@ -18,7 +18,7 @@
 
 namespace gh {
 
-constexpr int STRIP_GROUP_1D = 8;  // strips of a 1D item: one has a single row, less work than taking it
+constexpr int STRIP_GROUP_1D = 8;  // most strips of a 1D item: one has a single row, less work than taking it
 
 template <class T, int SOLVER, int STAGE, int NW, bool WIDE>
 __global__ void __launch_bounds__(32 * NW, (strip_warps<T, 2>() / NW))
@@ -39,8 +39,8 @@ __global__ void __launch_bounds__(32 * NW, (strip_warps<T, 2>() / NW))
     if (P.ndim == 1) {
       Shares<3> tot;
       const StageArgs<T> A = Args::template args_for<1>(B, P, w.prob);
-      for (int k = 0; k < STRIP_GROUP_1D; ++k) {
-        const int x0 = (w.tx * STRIP_GROUP_1D + k) * STRIP_OWN;
+      for (int k = 0; k < B.group_1d; ++k) {
+        const int x0 = (w.tx * B.group_1d + k) * STRIP_OWN;
         if (x0 >= A.n[0]) break;
         K1::strip(A, x0, 0, 1, 0, speed, tot, bad);
       }
@@ -69,7 +69,7 @@ void fill_batch_strip(BatchVariant* out) {
   out->tx = 32 * NW;
   out->cols = STRIP_OWN;
   out->warps = NW;
-  out->group_1d = STRIP_GROUP_1D;
+  out->most_1d = STRIP_GROUP_1D;
 }
 
 template <class T, int NW>

@@ -217,3 +217,29 @@ def test_march_axis_beyond_65535_chunks(precision, n, tile):
         h.close()
         ref = U if ref is None else ref
         np.testing.assert_array_equal(U, ref, err_msg=f"kchunk {kc}")
+
+
+@pytest.mark.parametrize("precision", [H.FP32_MIXED, H.FP64_DW])
+def test_batch_results_do_not_depend_on_the_strips_per_item(precision):
+    """1D problems at the edges of strips and of groups of strips, alone (one strip
+    an item) and beside meshes that make the items 2 to 8 strips: the same bits."""
+    probs = [P.random_blocks(1, (m,), seed=m, bc=bc) for m in (2, 28, 29, 56, 57, 85, 113, 141, 197, 224, 225, 449)
+             for bc in (P.PERIODIC, P.OUTFLOW)]
+    ref = None
+    for cells in (0, 200000, 500000, 1500000):
+        more = [P.random_blocks(1, (cells,), seed=1, bc=P.REFLECT)] if cells else []
+        b = H.Batch(probs + more, precision=precision)
+        for i, pr in enumerate(probs + more):
+            b.set_primitive(i, pr.rho, pr.vel, pr.p)
+        b.run(4, 0.4)
+        assert b.status() == -1
+        got = [b.get_conserved(i) for i in range(len(probs))]
+        if more:
+            h = H.Hydro.from_problem(more[0], precision=precision)
+            h.advance(4, 0.4)
+            np.testing.assert_array_equal(b.get_conserved(len(probs)), h.get_conserved(precision=H.FP64))
+            h.close()
+        b.close()
+        ref = ref or got
+        for a, c in zip(got, ref):
+            np.testing.assert_array_equal(a, c, err_msg=f"{cells} cells beside")
