@@ -10,6 +10,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <string>
 #include <type_traits>
 #include <vector>
@@ -224,17 +225,27 @@ int configure(genasis_hydro* h, int tile, int kchunk_req) {
       const long rows = (strips * nm + 16L * h->num_sms - 1) / (16L * h->num_sms);
       kchunk = (int)(rows < least ? least : rows > 32 ? 32 : rows);
     } else if (h->prec == GENASIS_FP64) {
-      // FP64 is bound by its pipe on every SM: the chunk whose CTAs per SM, each
-      // its planes and half a plane of warm-up, come to the least
+      // FP64 is bound by its pipe on every SM: the chunk whose warps per SM, each
+      // its CTA's planes and half a plane of warm-up, come to the least
       // (128^3: 19 planes in 448 CTAs, 2.95 per SM, 1.86 ms a stage; 13 in 640,
       // 4.2 per SM, 2.03; 16 in 512 2.10.  A step of 32^3: one plane 0.11 ms, 8
-      // planes 0.66)
-      long best = -1;
+      // planes 0.66).  Warps that hold cells count, and fewer than three on an SM
+      // take as long as three, whose latency they are bound by (a step of 7 x 3377:
+      // 23 rows in one CTA per SM 507 us, 8 rows in three 208, 4 in six 220; with
+      // 8 rows wherever they fill four CTAs an SM 267)
+      const double per = v1.threads / 32.0;  // warps of a CTA; fewer hold cells in the last ones
+      double live = per;
+      if (h->ndim == 2)
+        live = ((gx - 1) * per + std::min(per, (double)((h->n[0] - (gx - 1) * v1.tx + 32) / 32))) / gx;
+      else
+        live = per * h->n[1] / ((double)gy * v1.ty);
+      double best = -1.0;
       for (int gzt = 1; gzt <= nm && gzt <= 65535; ++gzt) {
         const int kc = (nm + gzt - 1) / gzt;
         const long ctas = (long)gx * gy * ((nm + kc - 1) / kc);
-        const long cost = (ctas + h->num_sms - 1) / h->num_sms * (2L * kc + 1);
-        if (best < 0 || cost < best) {
+        const long per_sm = (ctas + h->num_sms - 1) / h->num_sms;
+        const double cost = std::max(3.0, per_sm * live) * (2 * kc + 1);
+        if (best < 0.0 || cost < best) {
           best = cost;
           kchunk = kc;
         }

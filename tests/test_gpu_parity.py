@@ -762,3 +762,23 @@ def test_upwind_side_at_rest_without_pressure(ndim, precision, tol):
             h.close()
             assert t == pytest.approx(to, rel=1e-5)
             _check(U, Uo, ndim, tol, f"{ndim}d axis {axis} flip {flip}")
+
+
+@pytest.mark.parametrize("n,least", [((7, 3377), 2), ((16, 5043), 2), ((37, 4000), 1.5), ((127, 3000), 0.9)])
+def test_fp64_chunks_fill_the_sms_with_live_warps(n, least):
+    """Narrow FP64 meshes, whose CTAs hold cells in one or two of their four warps,
+    get two or more CTAs an SM; full CTAs one.  The automatic chunk gives the bits
+    of any other."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    pr = P.random_blocks(2, n, seed=2, bc=P.OUTFLOW)
+    h = H.Hydro.from_problem(pr, precision=H.FP64)
+    assert h.tile_info()["ctas"] >= least * sms
+    h.advance(2, 0.3)
+    a = h.get_conserved()
+    h.close()
+    h = H.Hydro.from_problem(pr, precision=H.FP64)
+    h.set_tile(0, 64)
+    h.advance(2, 0.3)
+    np.testing.assert_array_equal(h.get_conserved(), a)
+    h.close()
