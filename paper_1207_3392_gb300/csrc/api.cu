@@ -384,8 +384,7 @@ int launch_stage(genasis_hydro* h, int stage, cudaStream_t st) {
     void* q[] = {&A, &h->xy_strips, &h->xy_rows};
     GH_CK(launch_chained(v.xy_fn, h->xy_grid, 32 * v.xy_warps, q, 0, st, h->chained));
   }
-  // (the paired tiles do not wait for the chain)
-  GH_CK(launch_chained(v.fn, grid, v.threads, p, v.smem, st, h->chained && !v.pair));
+  GH_CK(launch_chained(v.fn, grid, v.threads, p, v.smem, st, h->chained && v.chain));
   return GENASIS_OK;
 }
 template int launch_stage<double>(genasis_hydro*, int, cudaStream_t);

@@ -17,6 +17,7 @@ inline void fill_variant(StageVariant* out) {
   out->tx = K::OWN;  // columns of cells per tile (TX - 1 in 1D/2D)
   out->ty = TY;
   out->threads = TX * TY;
+  out->chain = NDIM == 1;
 }
 
 // PRE: in-plane face states formed once per cell (see stage_kernel.cuh).
@@ -49,6 +50,7 @@ inline void fill_strip(StageVariant* out) {
   out->ty = 1;
   out->threads = 32 * NW;
   out->strips = 1;
+  out->chain = 1;
 }
 template <class T, int NW>
 inline bool pick_strip_switch(int stage, StageVariant* out) {
@@ -82,6 +84,7 @@ inline void fill_split(StageVariant* out) {
   out->tx = 128;
   out->ty = 1;
   out->threads = 128;
+  out->chain = 1;
 }
 template <class T>
 inline bool pick_split_switch(int stage, StageVariant* out) {

@@ -20,6 +20,7 @@ struct StageVariant {
   const void *xy_fn = nullptr, *xy_fn_wide = nullptr;
   int xy_warps = 0;
   const void* fn_odd = nullptr;  // fn for planes whose cell count is not a multiple of 4 (no shared memory)
+  int chain = 0;       // 1: the kernels begin with chain_wait()
   int pair = 0;        // 1: two march planes per thread (stage_pair.cuh); chunks of an even plane count
 };
 

@@ -61,16 +61,22 @@ struct StageArgs {
 // 1D/2D one axis gains less than the extra barrier costs.
 // COH: the state arrays may have been written earlier in the same launch (the
 // one-launch advance of small 1D meshes), so they are read through L2 (__ldcg), which
-// is coherent.  Same values either way.
+// is coherent.  Same values either way.  In 2D and 3D they are otherwise read-only
+// for the whole kernel, which therefore is never launched into a running
+// predecessor (chain_wait() in hydro_device.cuh): loads through the read-only path
+// may cross the barriers of a plane, and with plain ones behind a wait a step of
+// 96 x 100 x 128 on tile 0 takes 140 us instead of 133.  In 1D, one row a CTA, the
+// launch is worth more (5000 cells: 11.9 us a step against 12.8).
 template <int NDIM, class T, int SOLVER, int STAGE, int TX, int TY, bool PRE = (NDIM == 3), bool COH = false>
 struct StageKernel {
+  static constexpr bool MARCH = NDIM >= 2;
   static __device__ __forceinline__ T ld(const T* p) {
     if constexpr (COH) return __ldcg(p);
+    else if constexpr (MARCH) return __ldg(p);
     else return *p;
   }
   static constexpr int NV = NDIM + 2;
   static constexpr bool SW = SOLVER == SOLVER_HLLC_SW;  // per-face HLLC/HLL choice from shock bits
-  static constexpr bool MARCH = NDIM >= 2;
   static constexpr bool HAS_Y = NDIM == 3;
   static constexpr int AM = NDIM - 1;  // march axis (2D: y, 3D: z)
   static constexpr int NT = TX * TY;
@@ -821,7 +827,7 @@ struct StageKernel {
 // MINB: CTAs per SM the register allocation must allow (__launch_bounds__).
 template <int NDIM, class T, int SOLVER, int STAGE, int TX, int TY, int MINB, bool PRE>
 __global__ void __launch_bounds__(TX * TY, MINB) hydro_stage_kernel(const StageArgs<T> A) {
-  chain_wait();
+  if constexpr (NDIM == 1) chain_wait();
   StageKernel<NDIM, T, SOLVER, STAGE, TX, TY, PRE>::run(A);
 }
 
