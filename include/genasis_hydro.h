@@ -181,7 +181,8 @@ int genasis_hydro_clear_status(genasis_hydro_t h);
  * works alone on 28 columns.  3D tile 14 (FP32) and tile 4 (double word) are the
  * same for the x and y axes, followed by a launch of one thread per (x, y)
  * column for z.  They and tile 1 of 2D double word are the defaults (3D meshes
- * of 29 to 32 columns along x: tile 0). */
+ * of 29 to 32 columns along x and more than 655,360 cells, double word 262,144:
+ * tile 0). */
 int genasis_hydro_set_tile(genasis_hydro_t h, int tile, int kchunk);
 int genasis_hydro_get_tile(genasis_hydro_t h, int *info);
 

@@ -65,10 +65,14 @@ int stage_tile_count(int ndim, int prec) { return tile_count(ndim, prec); }
 
 // Independent warps wherever they are compiled: 3D FP32 (tile 14), 2D and 3D
 // double word (tiles 1 and 4).  A strip owns 28 columns, a tile 32: with 29 to
-// 32 columns along x in 3D two half-empty strips lose to one tile (29 x 160 x
-// 160: 96 to 99 us a step against 88 in FP32, 562 against 499 in double word).
-int stage_tile_default(int ndim, int prec, int nx) {
-  if (ndim == 3 && nx > 28 && nx <= 32) return 0;
+// 32 columns along x in 3D two half-empty strips lose to one tile once the mesh is
+// large enough to fill the SMs with tiles.  us a step, strips and tiles: FP32 HLLC
+// 39 and 56 at 29 x 40 x 40, 56 and 62 at 30 x 100 x 100, 97 and 90 at 32 x 160 x
+// 160; with the shock switch 55 and 70, 82 and 88, 155 and 138; double word HLLC 78
+// and 204, 248 and 257, 531 and 533, HLL 87 and 224, 307 and 288, 676 and 623.
+int stage_tile_default(int ndim, int prec, int nx, size_t ncell) {
+  const size_t large = prec == GENASIS_FP64_DW ? (size_t)1 << 18 : (size_t)5 << 17;
+  if (ndim == 3 && nx > 28 && nx <= 32 && ncell > large) return 0;
   if (prec == GENASIS_FP64_DW) return ndim == 3 ? 4 : ndim == 2 ? 1 : 0;
   if (prec == GENASIS_FP32_MIXED && ndim == 3) return 14;
   return 0;
@@ -724,7 +728,7 @@ int genasis_hydro_create(const genasis_hydro_desc* d, genasis_hydro_t* out) {
   rc = h->prec == GENASIS_FP64         ? upload_geometry<double>(h, d)
        : h->prec == GENASIS_FP32_MIXED ? upload_geometry<float>(h, d)
                                        : upload_geometry<dw>(h, d);
-  if (!rc) rc = configure(h, stage_tile_default(h->ndim, h->prec, h->n[0]), 0);
+  if (!rc) rc = configure(h, stage_tile_default(h->ndim, h->prec, h->n[0], h->ncell), 0);
   if (rc) {
     free_all(h);
     return rc;

@@ -28,7 +28,7 @@ struct StageVariant {
 // GENASIS_FP32_MIXED, GENASIS_FP64_DW); index `tile` selects one.
 int stage_tile_count(int ndim, int prec);
 // The tile a new handle starts with.
-int stage_tile_default(int ndim, int prec, int nx);
+int stage_tile_default(int ndim, int prec, int nx, size_t ncell);
 // Fills *out for (ndim, precision, solver, stage, tile); returns false if absent.
 bool stage_variant(int ndim, int prec, int solver, int stage, int tile, StageVariant* out);
 bool stage_variant_dw(int ndim, int solver, int stage, int tile, StageVariant* out);

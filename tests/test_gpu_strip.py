@@ -243,3 +243,20 @@ def test_batch_results_do_not_depend_on_the_strips_per_item(precision):
         ref = ref or got
         for a, c in zip(got, ref):
             np.testing.assert_array_equal(a, c, err_msg=f"{cells} cells beside")
+
+
+@pytest.mark.parametrize("precision,n,tile", [(H.FP32_MIXED, (29, 40, 40), 14), (H.FP32_MIXED, (32, 128, 160), 14),
+                                              (H.FP32_MIXED, (32, 128, 161), 0), (H.FP32_MIXED, (33, 160, 160), 14),
+                                              (H.FP64_DW, (32, 64, 128), 4), (H.FP64_DW, (32, 64, 129), 0)])
+def test_default_tile_of_3d_meshes_one_tile_wide(precision, n, tile):
+    pr = P.random_blocks(3, n, seed=3)
+    for solver in (H.HLLC, H.HLLC_SWITCH)[:2 if precision == H.FP32_MIXED else 1]:
+        h = H.Hydro.from_problem(pr, precision=precision, solver=solver)
+        assert h.tile_info()["tile"] == tile
+        h.advance(1, 0.3)
+        U = h.get_conserved()
+        h.set_primitive(pr.rho, pr.vel, pr.p)
+        h.set_tile(14 - tile if precision == H.FP32_MIXED else 4 - tile, 0)
+        h.advance(1, 0.3)
+        np.testing.assert_array_equal(h.get_conserved(), U)
+        h.close()
