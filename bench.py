@@ -153,10 +153,10 @@ FLOPS_STEP_3D = {"hllc": 1469, "hll": 1421}
 FLOPS_STAGE1_3D["hllc_switch"] = FLOPS_STAGE1_3D["hllc"]  # away from shocks; the detector is not counted
 FLOPS_STEP_3D["hllc_switch"] = FLOPS_STEP_3D["hllc"]
 # DRAM bytes (read + write) per stage of the FP32 HLLC 3D kernels at 256^3, from
-# ncu captures: tile 8, 40 planes per CTA (profiles/stage_fp32_hllc_sedov256_ncu.md);
-# tile 14, 48 planes, the strips along x and y and the march along z together
-# (profiles/split_and_strip_counters.md).  Other configurations, precisions and
-# sizes report no traffic.
+# ncu captures: tile 8, 40 planes per CTA; tile 14, 48 planes (its automatic
+# chunk), the strips along x and y and the march along z together.  Other
+# configurations, among them tile 14 with the planes that the bench's tuning may
+# choose, precisions and sizes report no traffic.
 TRAFFIC_FP32_HLLC_256 = {
     (8, 40): {"stage1": 356.859136e6 + 300.052480e6, "stage2": 732.600576e6 + 312.649472e6},
     (14, 48): {"stage1": 340.713216e6 + 291.104512e6 + 697.400832e6 + 290.496512e6,

@@ -2,8 +2,8 @@
 // problems of uneven size.  Each CTA repeatedly takes the next (problem, tile,
 // chunk) item from a global counter (items are sorted largest first) and runs
 // the same tile body as the single-grid stage kernel on it, with that
-// problem's mesh, boundaries, gamma and time step.  FP64 and double word; FP32
-// runs batch_strip.cuh.
+// problem's mesh, boundaries, gamma and time step.  FP64; FP32 and double word
+// run batch_strip.cuh on the same arguments.
 #pragma once
 
 #include "stage_kernel.cuh"

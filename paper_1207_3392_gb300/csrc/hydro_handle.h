@@ -49,11 +49,11 @@ struct genasis_hydro {
   CUtensorMap fmap[2];     // U[0], U[1] with the box of the TMA shock-flag pass
   bool flags_tma = false;  // the switch's stage-1 detector runs the TMA pass
   int want_totals = 1;
-  int one_launch = 1;  // small 1D meshes: a whole advance in one cooperative launch
+  int one_launch = 1;  // small 1D meshes: a whole advance in one launch
   int cluster_state = 0;  // small 1D meshes on one cluster: 0 not planned yet, 1 planned, -1 not on this device
   gh::Cluster1D cluster{};
   int mlp_tc = 0;      // attached network: on tcgen05 (1) or mma.sync (0)
-  unsigned* adv = nullptr;  // its grid-barrier words [2] (zero between launches), then one dt per CTA
+  unsigned* adv = nullptr;  // cooperative 1D advance: its barrier counter (zeroed before each launch), then (at 256 B) one dt per CTA
   // cached graphs of `advance`, one per starting state buffer
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   int g_nsteps = -1;

@@ -1,4 +1,4 @@
-// kern_3d_f32.cu -- 3D stage kernels, FP32 storage with FP64 recovery.
+// kern_3d_f32.cu -- 3D stage kernels, FP32 state and fluxes.
 #include "instantiate.cuh"
 
 namespace gh {

@@ -2,7 +2,7 @@
 // report instead of hanging.  Two waits that cannot complete, each on its own
 // status word:
 //   grid barrier (grid_sync.cuh): of two CTAs only the first arrives, so the
-//     generation word it polls never moves;
+//     counter it polls never reaches two;
 //   mbarrier (mbarrier.cuh): one thread waits on an mbarrier that nothing
 //     arrives on (the kind of wait of the TMA and tcgen05 kernels).
 // Each gives up after about one second and sets STATUS_TIMEOUT; the launches

@@ -113,10 +113,10 @@ struct StageKernel {
   // has its own plane.  The values are the same either way.
   // In 3D, stage 2 only: stage 1 also carries the column totals through the
   // march, and holding whole slots there spilled (measured: stage 1 slower,
-  // stage 2 4% faster).  1D and 2D FP32 (3 or 4 values per slot): one float4
-  // per slot (in 1D its last lane is unused).
+  // stage 2 4% faster).  1D FP32 (3 values per slot): one float4 per slot, its
+  // last lane unused.
   static constexpr bool VEC5 = NDIM == 3 && PRE && STAGE == 2 && std::is_same<T, float>::value;
-  static constexpr bool VEC4 = NDIM <= 2 && std::is_same<T, float>::value;
+  static constexpr bool VEC4 = NDIM == 1 && std::is_same<T, float>::value;
   static constexpr bool VEC = VEC5 || VEC4;
   static constexpr bool VECF = VEC;
   static constexpr int P = VEC ? 1 : 0;  // plane arrays collapse to one element under VEC
@@ -299,8 +299,9 @@ struct StageKernel {
   // L2 prefetch of the cell (ref, m) that load_col will read PFD - 2 march
   // iterations later (the same boundary-mapped address, so always inside the
   // arrays): the load then meets L2 latency instead of DRAM latency.  Only
-  // the 2D march (rows of one CTA) gains; in 3D the extra instructions cost
-  // more than the latency they hide.
+  // the 2D march (rows of one CTA) gains (double word, 3000^2: 3301 -> 2971 us a
+  // step, 1024^2 455 -> 460; FP64 0.0 to 0.9% slower); in 3D the extra
+  // instructions cost more than the latency they hide.
   static constexpr int PFD = NDIM == 2 ? 3 : 0;
   static __device__ __forceinline__ void prefetch_col(const StageArgs<T>& A, const ColRef& r, int m, size_t vs) {
     bool fm = false;

@@ -46,8 +46,6 @@ constexpr int STRIP_OWN = 28;  // columns a warp owns
 
 __device__ __forceinline__ float lane_up(float x) { return __shfl_up_sync(0xffffffffu, x, 1); }
 __device__ __forceinline__ float lane_down(float x) { return __shfl_down_sync(0xffffffffu, x, 1); }
-__device__ __forceinline__ double lane_up(double x) { return __shfl_up_sync(0xffffffffu, x, 1); }
-__device__ __forceinline__ double lane_down(double x) { return __shfl_down_sync(0xffffffffu, x, 1); }
 __device__ __forceinline__ dw lane_up(dw x) { return dw(lane_up(x.hi), lane_up(x.lo)); }
 __device__ __forceinline__ dw lane_down(dw x) { return dw(lane_down(x.hi), lane_down(x.lo)); }
 

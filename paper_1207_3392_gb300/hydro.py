@@ -340,7 +340,7 @@ class Hydro:
 
     def set_one_launch(self, enabled):
         """Small 1D meshes and an attached network: all steps of a call in one
-        cooperative launch (default on)."""
+        launch (default on)."""
         check(load().genasis_hydro_set_option(self._h, OPT_ONE_LAUNCH, int(bool(enabled))))
 
     def set_mlp_tcgen05(self, enabled):
