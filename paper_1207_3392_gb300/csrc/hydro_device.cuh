@@ -236,6 +236,10 @@ __device__ __forceinline__ bool seed_range(double x) {
   const unsigned ex = (unsigned)((unsigned long long)__double_as_longlong(x) >> 52) & 0x7ffu;
   return ex - 900u <= 246u;
 }
+// The same of a positive x: a negative x (a limited density below zero) has no root.
+__device__ __forceinline__ bool root_range(double x) {
+  return (unsigned)((unsigned long long)__double_as_longlong(x) >> 52) - 900u <= 246u;
+}
 // Hardware FP32 reciprocal and reciprocal square root (relative error about
 // 2^-23); arguments above 2^126 give 0.
 __device__ __forceinline__ float frcp(float x) {
@@ -273,8 +277,8 @@ __device__ __forceinline__ dw frcp(dw x) { return dw(1.0f, 0.0f) / x; }
 // Sound speed c = sqrt(gamma p / n) (Sec. 3.5) as gp rsqrt(gp n), gp = gamma p.
 // FP64: seed r = rsqrt(x) with relative error ~2^-22, residual e = 1 - x r^2,
 // then x^(-1/2) = r (1 - e)^(-1/2) = r (1 + e/2 + 3 e^2/8 + ...), which leaves
-// 5 e^3/16 ~ 2^-65: seven FP64 operations; CUDA's rsqrt outside the seed range,
-// and 0 where gamma p is not positive.  FP32: the hardware approximation.
+// 5 e^3/16 ~ 2^-65: seven FP64 operations; CUDA's rsqrt outside the seed range
+// (NaN for gp n < 0, which the wave speeds leave out), and 0 where gamma p is not positive.  FP32: the hardware approximation.
 // Double word: the same form with one correction (34 -> 26 operations), the
 // quotient and square root of dword.cuh where gp n nears the ends of FP32.
 __device__ __forceinline__ dw sound_speed(dw gamma, dw p, dw n) {
@@ -299,7 +303,7 @@ __device__ __forceinline__ float sound_speed(float gamma, float p, float n) {
 __device__ __forceinline__ double sound_speed(double gamma, double p, double n) {
   const double gp = mul_rn(gamma, p), x = mul_rn(gp, n);
   if (!(okey(gp) > 0)) return 0.0;
-  if (!seed_range(x)) return mul_rn(gp, rsqrt(x));
+  if (!root_range(x)) return mul_rn(gp, rsqrt(x));
   const double r = seed_double(frsqrt(seed_float(x)));
   const double e = fma_rn(-mul_rn(x, r), r, 1.0);
   const double c = mul_rn(gp, r);

@@ -782,3 +782,35 @@ def test_fp64_chunks_fill_the_sms_with_live_warps(n, least):
     h.advance(2, 0.3)
     np.testing.assert_array_equal(h.get_conserved(), a)
     h.close()
+
+
+@pytest.mark.parametrize("precision,tol", [(H.FP64, TOL_FP64), (H.FP32_MIXED, TOL_FP32)])
+@pytest.mark.parametrize("solver", [H.HLL, H.HLLC])
+def test_face_with_a_limited_density_below_zero(solver, precision, tol):
+    """A wide cell between narrow ones at theta 2: its limited density falls below
+    zero at a face.  That side has no sound speed and the wave speeds are the other
+    side's, as in the oracle; every cell stays physical."""
+    for ndim in (1, 2, 3):
+        for axis in range(ndim):
+            for vel in (0.0, 1.0, -1.0):
+                n = [5] * ndim
+                n[axis] = 32
+                w, rho = np.full(32, 0.01), np.full(32, 10.0)
+                w[15], rho[15], rho[16:] = 0.2, 1.0, 0.3
+                pr = P.random_blocks(ndim, tuple(n), seed=1, bc=P.OUTFLOW)
+                widths = [np.full(m, 0.01) for m in n]
+                widths[axis] = w
+                line = [1] * ndim
+                line[ndim - 1 - axis] = 32
+                v = np.zeros_like(pr.vel)
+                v[axis] = vel
+                pr = pr.with_(widths=widths, rho=np.zeros(pr.shape) + rho.reshape(line), p=np.ones(pr.shape), vel=v,
+                              theta=2.0)
+                g = O.Grid(pr, solver=solver)
+                Uo, to, _ = O.evolve(g, O.initial_state(pr, g), 0.05, max_steps=1)
+                h = H.Hydro.from_problem(pr, precision=precision, solver=solver)
+                t = h.advance(1, 0.05)
+                U = h.get_conserved(precision=H.FP64)
+                h.close()
+                assert t == pytest.approx(to, rel=1e-5)
+                _check(U, Uo, ndim, tol, f"{ndim}d axis {axis} v {vel}")
