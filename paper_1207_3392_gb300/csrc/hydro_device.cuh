@@ -280,11 +280,12 @@ __device__ __forceinline__ dw frcp(dw x) { return dw(1.0f, 0.0f) / x; }
 // 5 e^3/16 ~ 2^-65: seven FP64 operations; CUDA's rsqrt outside the seed range
 // (NaN for gp n < 0, which the wave speeds leave out), and 0 where gamma p is not positive.  FP32: the hardware approximation.
 // Double word: the same form with one correction (34 -> 26 operations), the
-// quotient and square root of dword.cuh where gp n nears the ends of FP32.
+// quotient and square root of dword.cuh where gp n nears the ends of FP32 or both
+// factors are limited below zero.
 __device__ __forceinline__ dw sound_speed(dw gamma, dw p, dw n) {
   const dw gp = gamma * p;
   const float x = mul_rn(gp.hi, n.hi);
-  if (!(x > 1e-30f && x < 1e30f)) return sqrt(gamma * (p / n));
+  if (!(x > 1e-30f && x < 1e30f && gp.hi > 0.0f)) return sqrt(gamma * (p / n));
   // c0 = gp rsqrt(gp n) and one Newton correction (gp - n c0^2) / (2 n c0) from
   // the exact residual, 1 / (n c0) = rsqrt(gp n)
   const float r = frsqrt(x), c0 = mul_rn(gp.hi, r);

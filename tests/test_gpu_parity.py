@@ -814,3 +814,23 @@ def test_face_with_a_limited_density_below_zero(solver, precision, tol):
                 h.close()
                 assert t == pytest.approx(to, rel=1e-5)
                 _check(U, Uo, ndim, tol, f"{ndim}d axis {axis} v {vel}")
+
+
+@pytest.mark.parametrize("solver", [H.HLL, H.HLLC])
+def test_double_word_face_with_density_and_pressure_below_zero(solver):
+    """The wide cell of the test above with the pressure falling as the density
+    does: at the face both are limited below zero and the sound speed is the root
+    of their positive ratio, as in the oracle."""
+    for vel in (0.0, 1.0, -1.0):
+        w, rho = np.full(32, 0.01), np.full(32, 10.0)
+        w[15], rho[15], rho[16:] = 0.2, 1.0, 0.3
+        pr = P.random_blocks(1, (32,), seed=1, bc=P.OUTFLOW)
+        pr = pr.with_(widths=[w], rho=rho, p=2.0 * rho, vel=np.full((1, 32), vel), theta=2.0)
+        g = O.Grid(pr, solver=solver)
+        Uo, to, _ = O.evolve(g, O.initial_state(pr, g), 0.05, max_steps=1)
+        h = H.Hydro.from_problem(pr, precision=H.FP64_DW, solver=solver)
+        t = h.advance(1, 0.05)
+        U = h.get_conserved()
+        h.close()
+        assert t == pytest.approx(to, rel=1e-10)
+        _check(U, Uo, 1, TOL_FP64, f"v {vel}")
