@@ -151,15 +151,21 @@ int configure(genasis_batch* b, int tile, int chunk) {
   GH_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ1, v1.fn, v1.tx, v1.smem));
   GH_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ2, v2.fn, v2.tx, v2.smem));
   const int occ = std::max(1, std::min(occ1, occ2));
-  // 1D items: as few strips as leave every resident warp one item (a warp takes
-  // its strips one after the other: a step of 30 problems of 100 to 1500 cells
-  // takes 10 us with 1 strip, 18 with 8, double word 13 and 34; with many items
-  // taking them costs more: 1000 problems of 128 to 4096 cells 73 us with 1 strip, 34 with 8)
+  // 1D items: in a batch of 1D problems alone as few strips as leave every
+  // resident warp one item (a warp takes its strips one after the other: a step of
+  // 30 problems of 100 to 1500 cells takes 10 us with 1 strip, 18 with 8, double
+  // word 13 and 34; with many items taking them costs more: 1000 problems of 128 to
+  // 4096 cells 73 us with 1 strip, 34 with 8).  Beside 2D problems, whose items are
+  // many times longer, always the most (16 1D and 16 2D problems, 18 steps with
+  // their copies: 1 strip 2624 us, 8 strips 2058)
   long strips = 0;
-  for (const HostProblem& h : b->hp)
-    if (h.ndim == 1) strips += (h.n[0] + cols - 1) / cols;
+  bool only_1d = true;
+  for (const HostProblem& h : b->hp) {
+    only_1d = only_1d && h.ndim == 1;
+    strips += (h.n[0] + cols - 1) / cols;
+  }
   const long slots = (long)occ * v1.warps * b->num_sms;
-  b->group_1d = (int)std::max(1L, std::min((long)v1.most_1d, (strips + slots - 1) / slots));
+  b->group_1d = only_1d ? (int)std::max(1L, std::min((long)v1.most_1d, (strips + slots - 1) / slots)) : v1.most_1d;
   // work items: (problem, x tile, y chunk), largest first
   struct Item {
     long cost;

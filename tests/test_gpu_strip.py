@@ -222,12 +222,15 @@ def test_march_axis_beyond_65535_chunks(precision, n, tile):
 @pytest.mark.parametrize("precision", [H.FP32_MIXED, H.FP64_DW])
 def test_batch_results_do_not_depend_on_the_strips_per_item(precision):
     """1D problems at the edges of strips and of groups of strips, alone (one strip
-    an item) and beside meshes that make the items 2 to 8 strips: the same bits."""
+    an item), beside 1D meshes that make the items 2 to 8 strips, and beside a 2D
+    one (8): the same bits."""
     probs = [P.random_blocks(1, (m,), seed=m, bc=bc) for m in (2, 28, 29, 56, 57, 85, 113, 141, 197, 224, 225, 449)
              for bc in (P.PERIODIC, P.OUTFLOW)]
     ref = None
-    for cells in (0, 200000, 500000, 1500000):
-        more = [P.random_blocks(1, (cells,), seed=1, bc=P.REFLECT)] if cells else []
+    for cells in (0, 200000, 500000, 1500000, -1):
+        more = [P.random_blocks(1, (cells,), seed=1, bc=P.REFLECT)] if cells > 0 else []
+        if cells < 0:
+            more = [P.random_blocks(2, (60, 40), seed=1, bc=P.REFLECT)]
         b = H.Batch(probs + more, precision=precision)
         for i, pr in enumerate(probs + more):
             b.set_primitive(i, pr.rho, pr.vel, pr.p)
